@@ -345,6 +345,17 @@ void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc) {
   pcg_scalars(B, c->stream, c->st, c->part, np, axpy_ctas(n), sm, ps, c->channels);
 }
 
+// The end of every outer step whose PCG has stopped: x += dx, the relative
+// change, the stopping rules.
+void enqueue_outer_end(firls_ctx* c, const firls_params& sc) {
+  const int B = run_batch(c), n = c->n;
+  outer_apply(B, n, c->stream, c->st, c->x, c->dx, c->part);
+  // the plateau stop needs a whole contraction window of nearly exact inner solves
+  const int plateau_after = sc.pcg_iters_late > 0 ? sc.outer_late + MU_WINDOW : 1 << 30;
+  outer_end(B, c->stream, c->st, c->part, axpy_ctas(n), sc.outer_tol, sc.outer_tol_kind, sc.outer_stall_tol,
+            plateau_after, c->channels);
+}
+
 // One macro step: every slice advances by one step of its own outer step.
 // In a boundary stage, slices whose PCG ended (PH_END) add their update to
 // x, measure the relative change and either stop or make their next outer
@@ -359,11 +370,7 @@ void enqueue_macro(firls_ctx* c, const firls_params& sc, bool boundary_stage = t
   if (boundary_stage) {
     {
       TMark m(c, FIRLS_K_OTHER, 3);
-      outer_apply(B, n, c->stream, c->st, c->x, c->dx, c->part);
-      // the plateau stop needs a whole contraction window of nearly exact inner solves
-      const int plateau_after = sc.pcg_iters_late > 0 ? sc.outer_late + MU_WINDOW : 1 << 30;
-      outer_end(B, c->stream, c->st, c->part, axpy_ctas(n), sc.outer_tol, sc.outer_tol_kind, sc.outer_stall_tol,
-                plateau_after, c->channels);
+      enqueue_outer_end(c, sc);
       boundary_view(B, c->stream, c->st, c->stw);
     }
     enqueue_weights(c, c->x, sc.precond, c->stw);
@@ -556,6 +563,40 @@ long solve_steps(const firls_params* p) {
 }
 bool has_tolerances(const firls_params* p) {
   return p->pcg_tol > 0.f || p->outer_tol > 0.f || p->outer_stall_tol > 0.f || period_of(*p) > 1;
+}
+
+// Without a PCG tolerance every slice takes the same PCG steps in each outer
+// step, so the batch moves in lockstep and an outer step of J PCG steps needs
+// its boundary stage only at the start of its J + 1 macro steps (a slice that
+// stops early, at rho = 0, waits there for the others).  One in every macro
+// step costs 9 launches that find nothing to do: 20 us a macro step for one
+// 256^2 slice, 110 us for 304.
+bool in_lockstep(const firls_params* p) { return !(p->pcg_tol > 0.f) && period_of(*p) == 1; }
+
+// params->outer_iters outer steps of a batch in lockstep: one graph replay of
+// J_k + 1 macro steps each, then the end of the last one.
+firls_status run_lockstep(firls_ctx* c, const firls_params& p, bool poll) {
+  auto late = [&](int k) { return p.pcg_iters_late > 0 && k >= p.outer_late; };
+  const int kPoll = 4;
+  for (int k = 0; k < p.outer_iters; ++k) {
+    const int steps = (late(k) ? p.pcg_iters_late : p.pcg_iters) + 1;
+    firls_params sc = p;
+    sc.boundary_period = steps;
+    const bool t = c->timing;
+    if (late(k) && !late(0)) c->timing = false;  // the marks stay those of the first schedule
+    const firls_status s = run_macro(c, sc, steps, steps, false);
+    c->timing = t;
+    TRY(s);
+    if (poll && (k + 1) % kPoll == 0 && k + 1 < p.outer_iters) {
+      bool ok = true;
+      const bool done = all_done(c, &ok);
+      if (!ok) return fail(c, FIRLS_E_CUDA, "state read-back failed");
+      if (done) break;
+    }
+  }
+  enqueue_outer_end(c, p);
+  c->marks_valid = c->timing;
+  return cuda_check(c, cudaGetLastError(), "outer step end");
 }
 
 firls_status collect_stats(firls_ctx* c, firls_stats* stats, bool* breakdown) {
@@ -776,7 +817,10 @@ extern "C" firls_status firls_solve(firls_ctx* c, const void* b, const firls_par
   if (!b || !x_out) return fail(c, FIRLS_E_INVALID_ARG, "b and x_out must be non-null");
   TRY(check_params(c, p));
   TRY(enqueue_setup(c, b, p, x0));
-  TRY(run_macro(c, *p, solve_steps(p), p->pcg_iters + 1, has_tolerances(p)));
+  if (in_lockstep(p))
+    TRY(run_lockstep(c, *p, has_tolerances(p)));
+  else
+    TRY(run_macro(c, *p, solve_steps(p), p->pcg_iters + 1, has_tolerances(p)));
   const size_t bytes = sizeof(float2) * (size_t)c->batch * c->n * c->n;
   CU(cudaMemcpyAsync(x_out, c->x, bytes, cudaMemcpyDeviceToDevice, c->stream));
   CU(cudaGetLastError());
@@ -830,12 +874,20 @@ extern "C" firls_status firls_solve_multi(firls_ctx* const* ctxs, int n_ctx, con
     }
   }
   const int chunk = p->pcg_iters + 1;  // macro steps of one outer step
+  // in lockstep one boundary stage at the start of a chunk serves it
+  const bool lockstep = in_lockstep(p) && p->pcg_iters_late <= 0;
+  const int period = lockstep ? chunk : period_of(*p);
+  firls_params sched = *p;
+  sched.boundary_period = period;
   if (!graphable) {
     const long total = solve_steps(p);
     for (long k = 0; k < total; ++k)
-      for (int i = 0; i < n_ctx; ++i) enqueue_macro(ctxs[i], *p, k % period_of(*p) == 0);
+      for (int i = 0; i < n_ctx; ++i) {
+        if (lockstep && k + 1 == total) enqueue_outer_end(ctxs[i], *p);
+        else enqueue_macro(ctxs[i], *p, k % period == 0);
+      }
   } else {
-    const bool same = g_multi.exec && same_schedule(g_multi.sched, *p) && (int)g_multi.ctxs.size() == n_ctx &&
+    const bool same = g_multi.exec && same_schedule(g_multi.sched, sched) && (int)g_multi.ctxs.size() == n_ctx &&
                       std::equal(g_multi.ctxs.begin(), g_multi.ctxs.end(), ctxs);
     // every context's set-up must precede the replays on c0's stream
     for (int i = 1; i < n_ctx; ++i) {
@@ -855,7 +907,7 @@ extern "C" firls_status firls_solve_multi(firls_ctx* const* ctxs, int n_ctx, con
       for (int i = 1; i < n_ctx; ++i) cudaStreamWaitEvent(ctxs[i]->stream, fork, 0);
       for (int i = 0; i < n_ctx; ++i) {
         if (ctxs[i]->timing) marks_reset(ctxs[i]);
-        for (int k = 0; k < chunk; ++k) enqueue_macro(ctxs[i], *p, k % period_of(*p) == 0);
+        for (int k = 0; k < chunk; ++k) enqueue_macro(ctxs[i], *p, k % period == 0);
       }
       for (int i = 1; i < n_ctx; ++i) {
         cudaEventRecord(join[i], ctxs[i]->stream);
@@ -874,7 +926,7 @@ extern "C" firls_status firls_solve_multi(firls_ctx* const* ctxs, int n_ctx, con
         return cuda_check(c0, e, "multi instantiate");
       }
       g_multi.ctxs.assign(ctxs, ctxs + n_ctx);
-      g_multi.sched = *p;
+      g_multi.sched = sched;
     }
     // replays of one outer step's worth of macro steps, then the remaining
     // steps (the last one applies every context's last outer step); with
@@ -908,7 +960,9 @@ extern "C" firls_status firls_solve_multi(firls_ctx* const* ctxs, int n_ctx, con
         if (i > 0) cudaStreamWaitEvent(c->stream, fork, 0);
         const bool t = c->timing;
         c->timing = false;
-        for (long k = 0; k < rem; ++k) enqueue_macro(c, *p);  // each with its boundary stage
+        if (lockstep) enqueue_outer_end(c, *p);  // all that is left (rem = 1)
+        else
+          for (long k = 0; k < rem; ++k) enqueue_macro(c, *p);  // each with its boundary stage
         c->timing = t;
         c->marks_valid = t;
         if (i > 0) {
