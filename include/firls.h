@@ -294,9 +294,7 @@ firls_status firls_set_active_slots(firls_ctx* ctx, int k);
  * thread-block cluster, the weights staged in shared memory or read from
  * HBM, where the slice fits; 4, 8, 16: rows per CTA of the tiled levels), the
  * largest wavelet block kept in shared memory by the tiled form (32, 64), the
- * ILU shared-memory ring
- * shape (10 * rows per stage + stages: 42, 43, 44, 22, 23, 24, as far as
- * they fit).  cache_path (may be NULL) is a text file of earlier
+ * ILU shape (42: long chunks, one CTA per SM; 22: short ones, two).  cache_path (may be NULL) is a text file of earlier
  * results keyed by "n batch psi levels": a hit skips the timing, a miss
  * appends the new result.  Overwrites the context's workspace; call after
  * firls_set_operator and before solving.  Synchronises the stream. */
@@ -322,9 +320,9 @@ firls_status firls_set_channels(firls_ctx* ctx, int channels);
 
 /* Failure-detection test hook (no counterpart in the paper).  With enable = 1
  * the TV preconditioner kernel (the ILU sweeps of Sec. 4.2) of every later
- * outer step runs in a test form: its producer issues no copy and every
- * bounded wait between its warps gives up after the first poll.  The waits
- * run out with nothing in flight, the slices are marked faulted and
+ * outer step runs in a test form: its warps hand nothing over and
+ * every bounded wait between them gives up at once.  The waits run out
+ * with nothing in flight, the slices are marked faulted and
  * firls_solve returns FIRLS_E_DEVICE_TIMEOUT; the context stays usable.
  * enable = 0 restores the normal kernel.  Only contexts with FIRLS_PSI_TV
  * launch that kernel. */
@@ -337,8 +335,9 @@ firls_status firls_get_tuning(const firls_ctx* ctx, int* rows_per_cta, int* coar
  * the wavelet form (1 or 2: the one-launch cluster form as above; 4, 8 or
  * 16: rows per CTA of the tiled levels; the default is the cluster form with
  * staged weights where a slice fits, else 8 rows), the largest wavelet block
- * kept in shared memory by the tiled form, and the ILU ring shape (10 * rows
- * per stage + stages).  FIRLS_E_INVALID_ARG if a shape does not exist or does
+ * kept in shared memory by the tiled form, and the ILU shape (10 * G + S, G = 4
+ * for long chunks of the sweeps, 2 for short ones; S has no effect and keeps
+ * the numbers of earlier tuning files valid).  FIRLS_E_INVALID_ARG if a shape does not exist or does
  * not fit this size.  A captured outer
  * step is re-captured at the next solve. */
 firls_status firls_set_tuning(firls_ctx* ctx, int rows_per_cta, int coarse_max, int ilu_shape);

@@ -13,6 +13,7 @@
 
 #include "firls.h"
 #include "launch.h"
+#include "per_device.h"
 
 using namespace firls;
 
@@ -40,9 +41,15 @@ struct firls_ctx {
   float2 *atb = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *d = nullptr, *q = nullptr;
   float2 *t = nullptr, *u = nullptr, *cw = nullptr, *dx = nullptr, *tmpA = nullptr, *tmpB = nullptr;
   // dx: the update of the current outer step, sum_j alpha_j d_j, accumulated
-  // from zero by the PCG steps and added to x once at the end of the step
+  // from zero one PCG step behind (each row FFT adds the step before) and
+  // added to x once at the end of the step
   float *ww = nullptr, *wtv = nullptr, *ia = nullptr, *wdiag = nullptr;
   float* wtv2 = nullptr;  // l1 TV: the vertical weights W2 (wtv then holds W1)
+  // TV: (lam W, 1/a) and lam W2 in the ILU's skewed layout; `skewed`: r, z (and q, u)
+  // are in it too, those of the PAPER and ILU0 preconditioners with TV
+  float4* wa = nullptr;
+  float2* w2s = nullptr;
+  bool skewed = false;
   float* wg = nullptr;
   int *gidx = nullptr, *goff = nullptr, *inv_off = nullptr, *inv_ids = nullptr;
   int *gcounts = nullptr, *gcursor = nullptr, *gerr = nullptr;
@@ -182,6 +189,7 @@ FftArgs fft_args(firls_ctx* c) {
 bool has_tv(const firls_ctx* c) { return (c->psi & (FIRLS_PSI_TV | FIRLS_PSI_TV_ANISO)) != 0; }
 bool is_aniso(const firls_ctx* c) { return (c->psi & FIRLS_PSI_TV_ANISO) != 0; }
 float* tv2_of(const firls_ctx* c) { return is_aniso(c) ? c->wtv2 : nullptr; }
+float2* w2s_of(const firls_ctx* c) { return is_aniso(c) ? c->w2s : nullptr; }
 
 // ---- timing marks: an event pair around each launch group of a class ----
 cudaEvent_t next_event(firls_ctx* c) {
@@ -226,15 +234,24 @@ void marks_reset(firls_ctx* c) {
   c->evnext = 0;
 }
 
+// The TV preconditioner's sweeps serve this solve (their vectors are skewed).
+bool uses_ilu(const firls_ctx* c, int precond) {
+  return has_tv(c) && (precond == FIRLS_PRECOND_PAPER || precond == FIRLS_PRECOND_ILU0);
+}
+
 // q = S d  (mode 0: d = z; 1: d = z + beta d; 2: d as given; -1: per slice,
-// d = x^k for a slice starting its outer step, else z or z + beta d)
-void enqueue_S(firls_ctx* c, int mode, const float2* zin, float2* din, float2* q) {
+// d = x^k for a slice starting its outer step, else z or z + beta d); skew: z
+// and q in the ILU's layout
+void enqueue_S(firls_ctx* c, int mode, const float2* zin, float2* din, float2* q, bool skew) {
   FftArgs a = fft_args(c);
+  a.skew = skew ? 1 : 0;
+  a.atb = c->atb;
   a.z = zin;
   a.d = din;
   a.t = c->t;
   a.mode = mode;
   a.xs = c->x;
+  a.dx = c->dx;
   { TMark m(c, FIRLS_K_ROW_FFT, 1); fft_row_fwd(c->n, a); }
   a.mask = c->mask;
   { TMark m(c, FIRLS_K_COL_FFT_MASK, 1); fft_col_mask(c->n, a); }
@@ -273,8 +290,9 @@ void enqueue_weights(firls_ctx* c, const float2* x, int precond, const SliceStat
     tv_weights(B, n, c->stream, view, x, c->wtv, tv2_of(c), c->channels);
     if (c->kind) wavelet_diag(B, n, c->levels, c->stream, view, c->ww, c->wdiag, c->sqtab, c->sqlen);
     penta_setup(B, n, c->stream, view, c->wtv, tv2_of(c), c->kind ? c->wdiag : nullptr, c->ia);
+    if (uses_ilu(c, precond)) ilu_pack(B, n, c->stream, view, false, c->wtv, tv2_of(c), c->ia, c->wa, w2s_of(c));
     // ILU(0): the pivots of the incomplete factorisation replace 1/a
-    if (precond == FIRLS_PRECOND_ILU0) ilu0_pivots(B, n, c->stream, view, c->wtv, tv2_of(c), c->ia);
+    if (precond == FIRLS_PRECOND_ILU0) ilu0_pivots(B, n, c->stream, c->st, view, c->wa, w2s_of(c), c->ia);
   } else if (precond == FIRLS_PRECOND_JACOBI) {
     wavelet_diag(B, n, c->levels, c->stream, view, c->ww, c->wdiag, c->sqtab, c->sqlen);
     jacobi_wavelet_setup(B, n, c->stream, view, c->wdiag, c->ia);
@@ -288,8 +306,7 @@ PcgSched pcg_sched(const firls_params& sc) {
 // alpha inside the ILU kernel (one launch fewer per macro step): the TV
 // preconditioners with one contrast per image
 bool alpha_in_ilu(const firls_ctx* c, const firls_params& sc) {
-  return has_tv(c) && c->channels == 1 &&
-         (sc.precond == FIRLS_PRECOND_PAPER || sc.precond == FIRLS_PRECOND_ILU0);
+  return uses_ilu(c, sc.precond) && c->channels == 1;
 }
 
 // Residual update and z = P^{-1} r, then rho (first residual) or beta and the
@@ -305,7 +322,7 @@ void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc) {
     // Jacobi or none: one fused pass, then the FP64 scalars
     {
       TMark m(c, FIRLS_K_AXPY, 1);
-      axpy_diag_step(B, n, c->stream, c->st, c->part, am, c->dx, c->d, c->r, c->q, c->atb,
+      axpy_diag_step(B, n, c->stream, c->st, c->part, am, c->r, c->q, c->atb,
                      sc.precond == FIRLS_PRECOND_JACOBI ? c->ia : nullptr, c->z);
     }
     TMark m(c, FIRLS_K_SCALARS, 1);
@@ -318,12 +335,12 @@ void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc) {
     const bool fuse = c->channels == 1;
     {
       TMark m(c, FIRLS_K_ILU, 1);
-      // the tuned ring shape for the whole batch, the default one for the
-      // fewer slots of a compacted launch (every shape gives the same sums)
-      const int shape = (c->tune_ilu && B == c->batch) ? c->tune_ilu : ilu_default_shape(n, B, is_aniso(c));
+      // the tuned shape for the whole batch, the default one for the fewer
+      // slots of a compacted launch (every shape gives the same results)
+      const int shape = (c->tune_ilu && B == c->batch) ? c->tune_ilu : 0;
       const int alpha_np = (mode == ILU_PER_SLICE && alpha_in_ilu(c, sc)) ? fft_row_ctas(n) : 0;
-      ilu_step(B, n, c->stream, c->st, c->part, mode, c->dx, c->d, c->r, c->q, c->atb, c->u, c->z, c->ia, c->wtv,
-               shape, fuse ? 1 : 0, ps, c->wait_test, tv2_of(c), alpha_np);
+      ilu_step(B, n, c->stream, c->st, c->part, mode, c->r, c->q, c->u, c->z, c->wa, w2s_of(c), shape,
+               fuse ? 1 : 0, ps, c->wait_test, alpha_np);
     }
     if (!fuse) {
       TMark m(c, FIRLS_K_SCALARS, 1);
@@ -333,7 +350,7 @@ void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc) {
   }
   {
     TMark m(c, FIRLS_K_AXPY, 1);
-    axpy_step(B, n, c->stream, c->st, c->part, am, c->dx, c->d, c->r, c->q, c->atb);
+    axpy_step(B, n, c->stream, c->st, c->part, am, c->r, c->q, c->atb);
   }
   WavArgs w = wav_args(c, c->st);
   {
@@ -349,7 +366,7 @@ void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc) {
 // change, the stopping rules.
 void enqueue_outer_end(firls_ctx* c, const firls_params& sc) {
   const int B = run_batch(c), n = c->n;
-  outer_apply(B, n, c->stream, c->st, c->x, c->dx, c->part);
+  outer_apply(B, n, c->stream, c->st, c->x, c->dx, c->d, c->part);
   // the plateau stop needs a whole contraction window of nearly exact inner solves
   const int plateau_after = sc.pcg_iters_late > 0 ? sc.outer_late + MU_WINDOW : 1 << 30;
   outer_end(B, c->stream, c->st, c->part, axpy_ctas(n), sc.outer_tol, sc.outer_tol_kind, sc.outer_stall_tol,
@@ -375,7 +392,7 @@ void enqueue_macro(firls_ctx* c, const firls_params& sc, bool boundary_stage = t
     }
     enqueue_weights(c, c->x, sc.precond, c->stw);
   }
-  enqueue_S(c, -1, c->z, c->d, c->q);
+  enqueue_S(c, -1, c->z, c->d, c->q, uses_ilu(c, sc.precond));
   if (!alpha_in_ilu(c, sc)) {
     TMark m(c, FIRLS_K_SCALARS, 1);
     pcg_alpha(B, c->stream, c->st, c->part, fft_row_ctas(n), c->channels);
@@ -439,6 +456,22 @@ firls_status upload_params(firls_ctx* c, const firls_params* p) {
   return FIRLS_OK;
 }
 
+// r and z of live slices in the layout that `precond` works in: they change
+// layout when a run continues under another preconditioner (outside capture).
+firls_status match_layout(firls_ctx* c, int precond) {
+  const bool want = uses_ilu(c, precond);
+  if (want == c->skewed) return FIRLS_OK;
+  const int B = c->batch, n = c->n;
+  if (want) ilu_pack(B, n, c->stream, c->st, true, c->wtv, tv2_of(c), c->ia, c->wa, w2s_of(c));
+  const size_t bytes = sizeof(float2) * (size_t)B * (want ? ilu_slice_elems(n) : (size_t)n * n);
+  for (float2* v : {c->r, c->z}) {  // u is free between macro steps
+    ilu_skew(B, n, c->stream, want, v, c->u);
+    CU(cudaMemcpyAsync(v, c->u, bytes, cudaMemcpyDeviceToDevice, c->stream));
+  }
+  c->skewed = want;
+  return cuda_check(c, cudaGetLastError(), "layout change");
+}
+
 float eps_of(const firls_params* p) { return p->eps > 0.f ? p->eps : 1e-10f; }
 
 // A^H b into atb (and x when x0 is null), ||A^H b||^2 partials, state init
@@ -459,6 +492,7 @@ firls_status enqueue_setup(firls_ctx* c, const void* b, const firls_params* p, c
     CU(cudaMemcpyAsync(c->x, x0, sizeof(float2) * (size_t)B * n * n, cudaMemcpyDeviceToDevice, c->stream));
   }
   CU(cudaMemsetAsync(c->dx, 0, sizeof(float2) * (size_t)B * n * n, c->stream));
+  c->skewed = uses_ilu(c, p->precond);  // every slice starts anew
   state_init(B, c->stream, c->st, c->part, fft_col_ctas(n), c->counts, n, c->lam_d, c->lamtv_d, eps_of(p),
              p->outer_iters, PH_BOUNDARY, c->channels);
   return cuda_check(c, cudaGetLastError(), "setup launch");
@@ -666,7 +700,10 @@ extern "C" firls_status firls_create(firls_ctx** out, int n_rows, int n_cols, in
   A(&c->mask, BN);
   A(&c->counts, (size_t)batch);
   A(&c->tw, (size_t)n);
-  for (float2** p : {&c->atb, &c->x, &c->r, &c->z, &c->d, &c->q, &c->t, &c->u, &c->cw, &c->dx}) A(p, BN);
+  for (float2** p : {&c->atb, &c->x, &c->d, &c->t, &c->cw, &c->dx}) A(p, BN);
+  // these take the ILU's skewed layout too
+  const size_t BS = std::max(N, ilu_slice_elems(n)) * batch;
+  for (float2** p : {&c->r, &c->z, &c->q, &c->u}) A(p, BS);
   A(&c->tmpA, BH);
   A(&c->tmpB, BH);
   for (float** p : {&c->ww, &c->wtv, &c->ia, &c->wdiag, &c->wtv2}) A(p, BN);
@@ -685,6 +722,8 @@ extern "C" firls_status firls_create(firls_ctx** out, int n_rows, int n_cols, in
     tw[j] = make_float2((float)std::cos(ang), (float)std::sin(ang));
   }
   cudaMemcpy(c->tw, tw.data(), sizeof(float2) * n, cudaMemcpyHostToDevice);
+  // weights that are read out before any were formed are 0
+  cudaMemset(c->wtv, 0, sizeof(float) * BN);
   // d is read (times 0) nowhere, but keep the workspace finite
   cudaMemset(c->d, 0, sizeof(float2) * BN);
   cudaMemset(c->part, 0, sizeof(double) * batch * NSLOT * MAXPART);
@@ -799,6 +838,8 @@ extern "C" firls_status firls_set_operator(firls_ctx* c, const uint8_t* mask, un
     CU(cudaMemcpy(c->sqtab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(c->sqlen, len.data(), sizeof(int) * len.size(), cudaMemcpyHostToDevice));
   }
+  if ((psi_kind & (FIRLS_PSI_TV | FIRLS_PSI_TV_ANISO)) && !c->wa) TRY(dalloc(c, &c->wa, ilu_slice_elems(n) / 2 * B));
+  if ((psi_kind & FIRLS_PSI_TV_ANISO) && !c->w2s) TRY(dalloc(c, &c->w2s, ilu_slice_elems(n) / 2 * B));
   c->psi = psi_kind;
   c->kind = kind;
   c->levels = kind ? wavelet_levels : 0;
@@ -1098,14 +1139,22 @@ extern "C" firls_status firls_apply_S_P(firls_ctx* c, const firls_params* p, con
   enqueue_weights(c, c->x, p->precond, c->st);  // every slice starts an outer step here
   // q = S d
   CU(cudaMemcpyAsync(c->d, d, bytes, cudaMemcpyDeviceToDevice, c->stream));
-  enqueue_S(c, 2, nullptr, c->d, static_cast<float2*>(q));
-  // z = P^{-1} r: feed r as "A^H b" with q = 0 through the INIT path
-  CU(cudaMemcpyAsync(c->atb, r, bytes, cudaMemcpyDeviceToDevice, c->stream));
-  CU(cudaMemsetAsync(c->q, 0, bytes, c->stream));
+  enqueue_S(c, 2, nullptr, c->d, static_cast<float2*>(q), false);
+  // z = P^{-1} r through the INIT path: r is the first residual, for the
+  // sweeps in their layout, else as "A^H b" with q = 0
   firls_params one = *p;
   one.pcg_tol = 0.f;
-  enqueue_precond(c, ILU_INIT, one);
-  CU(cudaMemcpyAsync(z, c->z, bytes, cudaMemcpyDeviceToDevice, c->stream));
+  c->skewed = uses_ilu(c, p->precond);
+  CU(cudaMemcpyAsync(c->atb, r, bytes, cudaMemcpyDeviceToDevice, c->stream));
+  if (c->skewed) {
+    ilu_skew(B, n, c->stream, true, c->atb, c->q);
+    enqueue_precond(c, ILU_INIT, one);
+    ilu_skew(B, n, c->stream, false, c->z, static_cast<float2*>(z));
+  } else {
+    CU(cudaMemsetAsync(c->q, 0, bytes, c->stream));
+    enqueue_precond(c, ILU_INIT, one);
+    CU(cudaMemcpyAsync(z, c->z, bytes, cudaMemcpyDeviceToDevice, c->stream));
+  }
   return cuda_check(c, cudaGetLastError(), "apply_S_P");
 }
 
@@ -1224,6 +1273,7 @@ extern "C" firls_status firls_run_steps(firls_ctx* c, const firls_params* p, int
   firls_params q = *p;
   q.outer_iters = 1;  // the per-slot limits come from firls_slot_load
   TRY(check_params(c, &q));
+  TRY(match_layout(c, q.precond));
   // one graph of all the steps: the caller polls with firls_slot_status
   c->cur_batch = c->active_slots;
   const firls_status st = run_macro(c, q, macro_steps, macro_steps, false);
@@ -1238,6 +1288,7 @@ extern "C" firls_status firls_run(firls_ctx* c, const firls_params* p) {
   firls_params q = *p;
   q.outer_iters = 1;
   TRY(check_params(c, &q));
+  TRY(match_layout(c, q.precond));
   c->cur_batch = c->active_slots;
   const firls_status st = run_macro(c, q, solve_steps(p), p->pcg_iters + 1, false);
   c->cur_batch = 0;
@@ -1285,7 +1336,12 @@ extern "C" firls_status firls_slot_move(firls_ctx* c, int from, int to) {
   };
   CU(mv(c->mask, N));
   CU(mv(c->counts, 1));
-  for (float2* v : {c->atb, c->x, c->r, c->z, c->d, c->q, c->t, c->u, c->cw, c->dx}) CU(mv(v, N));
+  // q, t, u and the coefficients are made anew in every macro step
+  const size_t NS = ilu_slice_elems(c->n);
+  for (float2* v : {c->atb, c->x, c->d, c->dx}) CU(mv(v, N));
+  for (float2* v : {c->r, c->z}) CU(mv(v, c->skewed ? NS : N));
+  if (c->wa) CU(mv(c->wa, NS / 2));
+  if (c->w2s) CU(mv(c->w2s, NS / 2));
   for (float* v : {c->ww, c->wtv, c->ia, c->wdiag, c->wtv2}) CU(mv(v, N));
   if (c->groups) CU(mv(c->wg, (size_t)c->n_groups));
   CU(mv(c->st, 1));
@@ -1382,11 +1438,11 @@ extern "C" firls_status firls_autotune(firls_ctx* c, const char* cache_path) {
     }
     if (has_tv(c)) {
       best = 1e30f;
-      for (int shape : {42, 43, 44, 22, 23, 24}) {
+      ilu_pack(B, n, c->stream, c->st, true, c->wtv, tv2_of(c), c->ia, c->wa, w2s_of(c));
+      for (int shape : {42, 22}) {
         if (!ilu_shape_fits(n, shape, is_aniso(c))) continue;
         const float t = time_ms(c, [&]() {
-          ilu_step(B, n, c->stream, c->st, c->part, ILU_STEP, c->x, c->d, c->r, c->q, c->atb, c->u, c->z, c->ia,
-                   c->wtv, shape, 0, PcgSched{0.f, 0, 1 << 30, 0, 0}, 0, tv2_of(c));
+          ilu_step(B, n, c->stream, c->st, c->part, ILU_STEP, c->r, c->q, c->u, c->z, c->wa, w2s_of(c), shape);
         }, 5);
         if (t < best) {
           best = t;
@@ -1592,5 +1648,7 @@ namespace {
 void prepare_kernels(int n) {
   fft_prepare(n);
   wav_prepare();
+  static PerDeviceOnce once;
+  once.run(ilu_prepare);
 }
 }  // namespace

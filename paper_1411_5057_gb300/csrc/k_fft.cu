@@ -24,7 +24,7 @@ template <int N> __host__ __device__ constexpr int rows_per_cta() {
 }
 
 // tv: staged d rows and TV weight rows; aniso (l1 TV): a second weight array
-template <int N> constexpr int row_smem_bytes(bool tv, bool aniso = false) {
+template <int N> constexpr int row_smem_bytes(bool tv = false, bool aniso = false) {
   constexpr int R = rows_per_cta<N>();
   int b = tw_bytes<N>() + R * 2 * fft_line_words<N>() * 4;
   if (tv) b += (R + 2) * N * 8 + (R + 1) * N * 4;
@@ -67,15 +67,29 @@ template <int N> FI void load_twiddles(float2* tw, const float2* __restrict__ tw
   }
 }
 
+// Column 0 or 1 of row `row` of slice s in the ILU's skewed layout (k_ilu.cu):
+// pair c is skew_pair float2 further on for each c.  The rows that share a warp
+// hold neighbouring 16-byte entries of a step, so a warp's accesses fill their
+// sectors without a pass through shared memory.  At 304 slices of 256^2 the row
+// FFT stays at the copy bandwidth (141 us with dx, 48 bytes a pixel); the row
+// IFFT takes 160 us instead of 142, for a warp's store touches nine lines
+// instead of two.  Through shared memory they took 159 and 164 us.
+constexpr int skew_pair = 64;
+template <int N> FI size_t skew_base(int s, int row) {
+  constexpr int K = N / 2 + 31, NB = (N + 31) / 32;
+  return ((((size_t)s * NB + (row >> 5)) * K + (row & 31)) * 32 + (row & 31)) * 2;
+}
+
 // d = z (mode 0) | d = z + beta d (mode 1) | use d as is (mode 2) | per slice
 // (mode < 0): d = x at the start of its outer step (S x^k), else d = z on the
-// first PCG step and z + beta d after it; t = rowFFT(d)
-template <int N>
+// first PCG step and z + beta d after it, with dx += alpha d for the direction
+// before (dx may be null); t = rowFFT(d)
+template <int N, bool SKEW>
 __global__ void __launch_bounds__(256) k_row_fwd(const float2* __restrict__ z, float2* __restrict__ d,
                                                  float2* __restrict__ t_out,
                                                  const SliceState* __restrict__ st,
                                                  const float2* __restrict__ twg, int mode_arg,
-                                                 const float2* __restrict__ x) {
+                                                 const float2* __restrict__ x, float2* __restrict__ dx) {
   using C = FftCfg<N>;
   constexpr int R = rows_per_cta<N>(), E = C::E, T = C::T, LW = fft_line_words<N>();
   const int s = blockIdx.y;
@@ -95,20 +109,43 @@ __global__ void __launch_bounds__(256) k_row_fwd(const float2* __restrict__ z, f
   const size_t base = (size_t)s * N * N + (size_t)row * N;
   const float beta = (float)st[s].beta;
   float2 v[E];
-  // one loop per mode, so that each touches only its own arrays
-  if (mode == 1) {
+  // one path per mode, so that each touches only its own arrays
+  if (mode == 0 || mode == 1) {
+    // element e of this thread: z at zb + e zs
+    const size_t zb = SKEW ? skew_base<N>(s, row) + (t >> 1) * skew_pair + (t & 1) : base + t;
+    constexpr int zs = SKEW ? T / 2 * skew_pair : T;
+    const float alpha = (float)st[s].alpha;
+    // EH elements at a time, all their loads in flight before the first store
+    constexpr int EH = E % 2 == 0 && E > 8 ? E / 2 : E;
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const size_t i = base + t + T * e;
-      v[e] = cfma(beta, d[i], z[i]);
-      d[i] = v[e];
+    for (int h = 0; h < E; h += EH) {
+      float2 dv[EH], xv[EH];
+#pragma unroll
+      for (int e = 0; e < EH; ++e) v[h + e] = z[zb + (h + e) * zs];
+      if (mode == 1) {
+#pragma unroll
+        for (int e = 0; e < EH; ++e) dv[e] = d[base + t + T * (h + e)];
+        if (dx) {
+#pragma unroll
+          for (int e = 0; e < EH; ++e) xv[e] = dx[base + t + T * (h + e)];
+        }
+      }
+      asm volatile("" ::: "memory");
+      if (mode == 1) {
+#pragma unroll
+        for (int e = 0; e < EH; ++e) {
+          if (dx) dx[base + t + T * (h + e)] = cfma(alpha, dv[e], xv[e]);
+          v[h + e] = cfma(beta, dv[e], v[h + e]);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < EH; ++e) d[base + t + T * (h + e)] = v[h + e];
     }
-  } else if (mode == 0 || mode == 3) {
-    const float2* __restrict__ src = mode == 0 ? z : x;
+  } else if (mode == 3) {
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const size_t i = base + t + T * e;
-      v[e] = src[i];
+      v[e] = x[i];
       d[i] = v[e];
     }
   } else {
@@ -376,12 +413,13 @@ __global__ void __launch_bounds__(512) k_col_resid(const float2* __restrict__ tb
 // q = (1/N) rowIFFT(t) [Re if real] + lam_tv (D1^T W1 D1 + D2^T W2 D2) d + lam u
 // (W1 = W2 = wtv for isotropic TV; wtv2 holds W2 for l1 TV); partial
 // Re<d, q>.
-template <int N>
+template <int N, bool SKEW>
 __global__ void __launch_bounds__(256) k_row_inv(const float2* __restrict__ tbuf, const float2* __restrict__ d,
                                                  const float2* __restrict__ u, const float* __restrict__ wtv,
                                                  float2* __restrict__ q, const SliceState* __restrict__ st,
                                                  double* __restrict__ part, int real,
-                                                 const float2* __restrict__ twg, const float* __restrict__ wtv2) {
+                                                 const float2* __restrict__ twg, const float* __restrict__ wtv2,
+                                                 const float2* __restrict__ atb) {
   using C = FftCfg<N>;
   constexpr int R = rows_per_cta<N>(), E = C::E, T = C::T, LW = fft_line_words<N>();
   const int s = blockIdx.y;
@@ -441,6 +479,10 @@ __global__ void __launch_bounds__(256) k_row_inv(const float2* __restrict__ tbuf
   fft_line<N, +1>(v, lines + lr * 2 * LW, lines + lr * 2 * LW + LW, tw, t);
   const float sc = 1.0f / ((float)N * (float)N);
   const float lam = st[s].lam, lam_tv = st[s].lam_tv;
+  // skewed q: also, the first residual of a slice at the start of its outer step
+  const bool start = SKEW && st[s].phase == PH_START;
+  const size_t qb = SKEW ? skew_base<N>(s, row) + (t >> 1) * skew_pair + (t & 1) : base + t;
+  constexpr int qs = SKEW ? T / 2 * skew_pair : T;
   float acc = 0.f;
 #pragma unroll
   for (int e = 0; e < E; ++e) {
@@ -468,8 +510,17 @@ __global__ void __launch_bounds__(256) k_row_inv(const float2* __restrict__ tbuf
       dc = d[base + col];
     }
     if (u) a = cfma(lam, uv[e], a);
-    q[base + col] = a;
     acc += rdot2(dc, a);
+    if (SKEW) v[e] = a;
+    else q[qb + e * qs] = a;
+  }
+  if (SKEW) {
+    if (start) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = csub(atb[base + t + T * e], v[e]);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) q[qb + e * qs] = v[e];
   }
   const double tot = block_sum((double)acc, red);
   if (threadIdx.x == 0) part[((size_t)s * NSLOT + SLOT_DQ) * MAXPART + blockIdx.x] = tot;
@@ -482,9 +533,11 @@ template <int N> static void set_smem_attrs() {
   static PerDeviceOnce once;
   once.run([] {
     const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    bool ok = cudaFuncSetAttribute(k_row_fwd<N>, A, row_smem_bytes<N>(false)) == cudaSuccess;
-    ok = cudaFuncSetAttribute(k_row_ahb<N>, A, row_smem_bytes<N>(false)) == cudaSuccess && ok;
-    ok = cudaFuncSetAttribute(k_row_inv<N>, A, row_smem_bytes<N>(true, true)) == cudaSuccess && ok;
+    bool ok = cudaFuncSetAttribute(k_row_fwd<N, false>, A, row_smem_bytes<N>()) == cudaSuccess;
+    ok = cudaFuncSetAttribute(k_row_fwd<N, true>, A, row_smem_bytes<N>()) == cudaSuccess && ok;
+    ok = cudaFuncSetAttribute(k_row_ahb<N>, A, row_smem_bytes<N>()) == cudaSuccess && ok;
+    ok = cudaFuncSetAttribute(k_row_inv<N, false>, A, row_smem_bytes<N>(true, true)) == cudaSuccess && ok;
+    ok = cudaFuncSetAttribute(k_row_inv<N, true>, A, row_smem_bytes<N>(true, true)) == cudaSuccess && ok;
     ok = cudaFuncSetAttribute(k_col_mask<N>, A, col_smem_bytes<N>()) == cudaSuccess && ok;
     ok = cudaFuncSetAttribute(k_col_inv<N>, A, col_smem_bytes<N>()) == cudaSuccess && ok;
     ok = cudaFuncSetAttribute(k_col_resid<N>, A, col_smem_bytes<N>()) == cudaSuccess && ok;
@@ -497,12 +550,13 @@ template <int N> struct FftLaunch {
   static constexpr int R = rows_per_cta<N>();
   static void row_fwd(const FftArgs& a) {
     set_smem_attrs<N>();
-    k_row_fwd<N><<<dim3(N / R, a.batch), R * FftCfg<N>::T, row_smem_bytes<N>(false), a.stream>>>(
-        a.z, a.d, a.t, a.st, a.tw, a.mode, a.xs);
+    const auto k = a.skew ? k_row_fwd<N, true> : k_row_fwd<N, false>;
+    k<<<dim3(N / R, a.batch), R * FftCfg<N>::T, row_smem_bytes<N>(), a.stream>>>(a.z, a.d, a.t, a.st, a.tw,
+                                                                                     a.mode, a.xs, a.dx);
   }
   static void row_ahb(const FftArgs& a) {
     set_smem_attrs<N>();
-    k_row_ahb<N><<<dim3(N / R, a.batch), R * FftCfg<N>::T, row_smem_bytes<N>(false), a.stream>>>(
+    k_row_ahb<N><<<dim3(N / R, a.batch), R * FftCfg<N>::T, row_smem_bytes<N>(), a.stream>>>(
         a.b, a.mask, a.t, a.tw);
   }
   static void col_mask(const FftArgs& a) {
@@ -527,9 +581,9 @@ template <int N> struct FftLaunch {
   }
   static void row_inv(const FftArgs& a) {
     set_smem_attrs<N>();
-    k_row_inv<N><<<dim3(N / R, a.batch), R * FftCfg<N>::T,
-                   row_smem_bytes<N>(a.wtv != nullptr, a.wtv2 != nullptr), a.stream>>>(
-        a.t, a.d, a.u, a.wtv, a.q, a.st, a.part, a.real, a.tw, a.wtv2);
+    const auto k = a.skew ? k_row_inv<N, true> : k_row_inv<N, false>;
+    k<<<dim3(N / R, a.batch), R * FftCfg<N>::T, row_smem_bytes<N>(a.wtv != nullptr, a.wtv2 != nullptr),
+        a.stream>>>(a.t, a.d, a.u, a.wtv, a.q, a.st, a.part, a.real, a.tw, a.wtv2, a.atb);
   }
 };
 

@@ -842,11 +842,10 @@ static void wcl_launch(const WavArgs& a, int R, bool mirror, const float2* x, co
 
 static int coarse_smem(int m0) { return m0 * (m0 + 1) * 8; }
 
-bool ilu_prepare();
 bool wavelet_diag_prepare();
 
-// Dynamic shared-memory limits of the wavelet, ILU and pseudo-diagonal
-// kernels, set once per device.
+// Dynamic shared-memory limits of the wavelet and pseudo-diagonal kernels,
+// set once per device.
 static void set_wav_attrs() {
   static PerDeviceOnce once;
   once.run([] {
@@ -858,7 +857,6 @@ static void set_wav_attrs() {
                               wcl_smem_bytes(WCL_NMAX, WCL_RMAX, WCL_LMAX, true)) == cudaSuccess && ok;
     ok = cudaFuncSetAttribute(k_wav_cluster<256, 32, 4, 2, WCL_THREADS_256>, A, wcl_smem_bytes(256, 32, 4, true)) ==
              cudaSuccess && ok;
-    ok = ilu_prepare() && ok;
     ok = wavelet_diag_prepare() && ok;
     return ok;
   });
@@ -1219,737 +1217,6 @@ void penta_setup(int batch, int n, cudaStream_t s, const SliceState* st, const f
   k_penta<<<dim3(blocks, batch), 256, 0, s>>>(n, st, wtv, wtv2, wdiag, ia);
 }
 
-// ILU(0) pivots of the penta-diagonal P: d_i = a_i - (lam W1_i)^2 / d_{i-1}
-// [col > 0] - (lam W2_i)^2 / d_{i-n} [row > 0] (the incomplete LU with zero
-// fill of Sec. 4.2 with updated pivots; W1 = W2 = W for isotropic TV).
-// In: ia = 1/a; out: ia = 1/d in place.  One warp per slice, a row at a time:
-// with alpha_i = a_i - (lam W2_i)^2 / d_{i-n} the row recurrence
-// d_i = alpha_i - (lam W1_i)^2 / d_{i-1} is a Moebius map of d_{i-1}, i.e.
-// (p, q) -> M_i (p, q) with M_i = [[alpha_i, -(lam W1_i)^2], [1, 0]] and
-// d = p / q, so the row is a scan of 2 x 2 matrix products: each lane folds
-// its E columns, a warp shuffle scan combines the lanes (every product
-// scaled by its largest entry: only the ratio p / q matters), and each lane
-// then runs its own columns from the incoming ratio.
-template <int E>
-__global__ void __launch_bounds__(32) k_ilu0_pivots(int n, const SliceState* __restrict__ st,
-                                                     const float* __restrict__ wtv, const float* __restrict__ wtv2,
-                                                     float* __restrict__ ia) {
-  const int s = blockIdx.x;
-  if (!slice_running(st, s)) return;
-  const int lane = threadIdx.x;
-  const float lam = st[s].lam_tv;
-  const float* w2 = wtv2 ? wtv2 : wtv;
-  const size_t base = (size_t)s * n * n;
-  float dprev[E];  // d of the row above in this lane's columns
-#pragma unroll
-  for (int e = 0; e < E; ++e) dprev[e] = 1.f;
-  for (int r = 0; r < n; ++r) {
-    const size_t rb = base + (size_t)r * n;
-    float al[E], k2[E];
-    // this lane's segment as a 2 x 2 matrix T = M_{last} ... M_{first}
-    float t00 = 1.f, t01 = 0.f, t10 = 0.f, t11 = 1.f;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int c = lane * E + e;
-      al[e] = 1.f;
-      k2[e] = 0.f;
-      if (c < n) {
-        const float a = 1.0f / ia[rb + c];
-        const float kv = r > 0 ? lam * w2[rb + c] : 0.f;
-        const float kh = c > 0 ? lam * wtv[rb + c] : 0.f;
-        al[e] = a - kv * kv / dprev[e];
-        k2[e] = kh * kh;
-      }
-      // M_e * T
-      const float n00 = al[e] * t00 - k2[e] * t10, n01 = al[e] * t01 - k2[e] * t11;
-      t10 = t00;
-      t11 = t01;
-      t00 = n00;
-      t01 = n01;
-      const float m = fmaxf(fmaxf(fabsf(t00), fabsf(t01)), fmaxf(fabsf(t10), fabsf(t11)));
-      if (m > 0.f) {
-        const float im = 1.0f / m;
-        t00 *= im;
-        t01 *= im;
-        t10 *= im;
-        t11 *= im;
-      }
-    }
-    // inclusive scan over the lanes: P_L = T_L ... T_0
-    float p00 = t00, p01 = t01, p10 = t10, p11 = t11;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const float q00 = __shfl_up_sync(0xffffffffu, p00, off), q01 = __shfl_up_sync(0xffffffffu, p01, off);
-      const float q10 = __shfl_up_sync(0xffffffffu, p10, off), q11 = __shfl_up_sync(0xffffffffu, p11, off);
-      if (lane >= off) {  // P = P_mine * P_earlier
-        const float n00 = p00 * q00 + p01 * q10, n01 = p00 * q01 + p01 * q11;
-        const float n10 = p10 * q00 + p11 * q10, n11 = p10 * q01 + p11 * q11;
-        const float m = fmaxf(fmaxf(fabsf(n00), fabsf(n01)), fmaxf(fabsf(n10), fabsf(n11)));
-        const float im = m > 0.f ? 1.0f / m : 1.f;
-        p00 = n00 * im;
-        p01 = n01 * im;
-        p10 = n10 * im;
-        p11 = n11 * im;
-      }
-    }
-    // the ratio entering this lane: the previous lane's prefix applied to
-    // (1, 0) (no left neighbour for column 0)
-    const float e00 = __shfl_up_sync(0xffffffffu, p00, 1), e10 = __shfl_up_sync(0xffffffffu, p10, 1);
-    float d = lane == 0 ? 0.f : e00 / e10;  // lane 0: column 0 has k2 = 0, d_in unused
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int c = lane * E + e;
-      if (c < n) {
-        d = k2[e] > 0.f ? al[e] - k2[e] / d : al[e];
-        dprev[e] = d;
-        ia[rb + c] = 1.0f / d;
-      }
-    }
-  }
-}
-
-void ilu0_pivots(int batch, int n, cudaStream_t s, const SliceState* st, const float* wtv, const float* wtv2,
-                 float* ia) {
-  const int E = (n + 31) / 32;
-  switch (E) {
-    case 1: k_ilu0_pivots<1><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    case 2: k_ilu0_pivots<2><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    case 3: k_ilu0_pivots<3><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    case 4: k_ilu0_pivots<4><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    case 5: k_ilu0_pivots<5><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    case 6: k_ilu0_pivots<6><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    case 8: k_ilu0_pivots<8><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    case 10: k_ilu0_pivots<10><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    case 12: k_ilu0_pivots<12><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    case 16: k_ilu0_pivots<16><<<batch, 32, 0, s>>>(n, st, wtv, wtv2, ia); break;
-    default: break;
-  }
-}
-
-// ------------------------------------------------ ILU solves (Sec. 4.2) -----
-// z = U^{-1} L^{-1} r with L = I + L_P diag(a)^{-1}, U = diag(a) + U_P, where
-// P = diag(a) + L_P + U_P is the TV penta-diagonal matrix.  Its off-diagonal
-// entries are b_i = -lam_tv W_{i+1} (couples i, i+1; zero at a row end) and
-// c_i = -lam_tv W_{i+n} (couples i, i+n; zero in the last row), so with
-// ia = 1/a the sweeps need only W and ia:
-//   forward  y_i = r_i + g_i y_{i-1} + h_i y_{i-n},
-//            g_i = lam W_i ia_{i-1} [col > 0],  h_i = lam W_i ia_{i-n} [row > 0]
-//   backward z_i = ia_i y_i + g_i z_{i+1} + h_i z_{i+n},
-//            g_i = lam ia_i W_{i+1} [col < n-1],  h_i = lam ia_i W_{i+n} [row < n-1]
-// P is symmetric, so U = diag(a) L^T and Re<r, z> = sum_i ia_i |y_i|^2.
-//
-// Kernel layout: one CTA per slice, five warps.
-//  * Warp 1 (scan warp) runs only the row recurrences: a row is E columns
-//    per lane, composed as affine maps and combined by a warp shuffle scan
-//    (no block barrier); it stores y (z) itself.
-//  * Warps 2-4 (helpers) own two-column chunks and process G rows at a time
-//    (independent rows, so their latencies overlap): the residual update
-//    r -= alpha q, x += alpha d, and per column (t, h, g) in the scan warp's
-//    lane-major layout.
-//  * Warp 0 (producer, one lane) fills a ring of S stages of G rows with
-//    1-D bulk copies (TMA), one copy per array and stage.
-// Handover per stage, with mbarriers: `full` (bytes landed), `empty`
-// (helpers done with the natural rows), `ready` (helpers wrote the group's
-// coefficients), `consumed` (scan warp done with them).  The scan warp waits
-// once per group of G rows and prefetches the next row of the group while
-// it scans the current one.  Every wait is bounded; a wait that runs out
-// marks the slice faulted and the CTA finishes without hanging.
-
-FI unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-FI void mbar_init(uint64_t* bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-FI void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
-}
-FI void mbar_arrive_tx(uint64_t* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-FI bool mbar_test(uint64_t* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// try_wait suspends the thread until the phase completes or the hint
-// (nanoseconds) runs out; the loop bounds the whole wait to about a second.
-FI bool mbar_try(uint64_t* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(100000u)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait: `tries` suspended polls of about 100 us each after a first
-// test (10000 tries: about a second).
-FI bool mbar_wait(uint64_t* bar, unsigned parity, int tries = 10000) {
-  if (mbar_test(bar, parity)) return true;
-  for (int it = 0; it < tries; ++it)
-    if (mbar_try(bar, parity)) return true;
-  return false;
-}
-// 1-D bulk copy global -> shared (16-byte aligned, size a multiple of 16),
-// completion counted in bytes on `bar`.
-FI void bulk_g2s(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-// The same with an L2 eviction policy (a hint: what the ILU reads again in
-// its backward sweep stays, what it streams through goes first).
-FI void bulk_g2s_hint(void* dst, const void* src, unsigned bytes, uint64_t* bar, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;\n" ::
-          "r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
-      : "memory");
-}
-FI uint64_t l2_evict_first() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(p));
-  return p;
-}
-FI uint64_t l2_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;\n" : "=l"(p));
-  return p;
-}
-FI void st_hint_f4(float2* dst, float4 v, uint64_t policy) {
-  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;\n" ::"l"(dst), "f"(v.x), "f"(v.y),
-               "f"(v.z), "f"(v.w), "l"(policy)
-               : "memory");
-}
-FI void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;\n" ::: "memory"); }
-FI int ld_acquire(const int* p) {
-  int v;
-  asm volatile("ld.acquire.cta.shared.b32 %0, [%1];\n" : "=r"(v) : "r"(smem_u32(p)) : "memory");
-  return v;
-}
-FI void st_release(int* p, int v) {
-  asm volatile("st.release.cta.shared.b32 [%0], %1;\n" ::"r"(smem_u32(p)), "r"(v) : "memory");
-}
-// Bounded poll until *p >= want (about a second at most); returns the value
-// seen, or -1 when the wait ran out.
-FI int poll_at_least(const int* p, int want, int tries = 1 << 24) {
-  for (int it = 0; it < tries; ++it) {
-    const int v = ld_acquire(p);
-    if (v >= want) return v;
-    if (it >= 256) __nanosleep(32);
-  }
-  return -1;
-}
-
-// Warp-wide exclusive scan of affine maps v -> A v + B in lane order
-// (REV: from lane 31 down).  Returns the value entering this lane's segment
-// for a zero value entering the row.
-template <bool REV>
-FI float2 warp_affine_exclusive(float A, float2 B) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const float Ap = REV ? __shfl_down_sync(0xffffffffu, A, off) : __shfl_up_sync(0xffffffffu, A, off);
-    const float bx = REV ? __shfl_down_sync(0xffffffffu, B.x, off) : __shfl_up_sync(0xffffffffu, B.x, off);
-    const float by = REV ? __shfl_down_sync(0xffffffffu, B.y, off) : __shfl_up_sync(0xffffffffu, B.y, off);
-    if (REV ? (lane + off < 32) : (lane >= off)) {
-      B = make_float2(fmaf(A, bx, B.x), fmaf(A, by, B.y));
-      A = A * Ap;
-    }
-  }
-  const float bx = REV ? __shfl_down_sync(0xffffffffu, B.x, 1) : __shfl_up_sync(0xffffffffu, B.x, 1);
-  const float by = REV ? __shfl_down_sync(0xffffffffu, B.y, 1) : __shfl_up_sync(0xffffffffu, B.y, 1);
-  if (lane == (REV ? 31 : 0)) return make_float2(0.f, 0.f);
-  return make_float2(bx, by);
-}
-
-// Store E consecutive complex values of one lane (columns c0 .. c0+E-1 < n),
-// with an L2 eviction policy.
-template <int E>
-FI void store_lane_row(float2* dst, int c0, int n, const float2 (&v)[E], uint64_t policy) {
-  if ((E & 1) == 0 && c0 + E <= n) {
-#pragma unroll
-    for (int e = 0; e < E; e += 2)
-      st_hint_f4(dst + c0 + e, make_float4(v[e].x, v[e].y, v[e + 1].x, v[e + 1].y), policy);
-  } else {
-#pragma unroll
-    for (int e = 0; e < E; ++e)
-      if (c0 + e < n) dst[c0 + e] = v[e];
-  }
-}
-
-constexpr int IW_HWARPS = 3;                   // helper warps (warps 2-4)
-constexpr int IW_HELPERS = 32 * IW_HWARPS;
-constexpr int IW_THREADS = 32 + IW_HELPERS + 32;
-constexpr int IW_MAXCH = 3;                    // chunks of two columns per helper thread (n <= 512)
-constexpr int IW_MAXSTAGES = 8;
-
-static int iw_cols_per_lane(int n) { return (n + 31) / 32; }
-// Stage of G rows (bytes): R, Q, X, D (8nG each), W (W1 for l1 TV), IA
-// (4nG each), W2 (4nG, l1 TV only), then SC: per row, float4 (t.x, t.y, h, g)
-// per lane-major column slot.
-struct IwLayout {
-  int n, G, ns, oQ, oX, oD, oW, oIA, oW2, oSC, bytes;
-};
-static IwLayout iw_layout(int n, int G, bool aniso = false) {
-  IwLayout L;
-  L.n = n;
-  L.G = G;
-  L.ns = 32 * iw_cols_per_lane(n);
-  L.oQ = 8 * n * G;
-  L.oX = 16 * n * G;
-  L.oD = 24 * n * G;
-  L.oW = 32 * n * G;
-  L.oIA = 36 * n * G;
-  L.oW2 = 40 * n * G;
-  L.oSC = (aniso ? 44 : 40) * n * G;
-  L.bytes = (L.oSC + 16 * L.ns * G + 127) / 128 * 128;
-  return L;
-}
-
-// Ring position: stage index and the parity of its current use.
-struct RingPos {
-  int s;
-  unsigned ph;
-  FI void next(int S) {
-    if (++s == S) {
-      s = 0;
-      ph ^= 1u;
-    }
-  }
-};
-
-// Groups: forward group g holds rows gG .. gG+G-1; backward group g (after
-// the NG = n/G forward ones) holds rows n-(g'+1)G .. n-g'G-1, g' = g - NG,
-// processed from the bottom row up.  Row uses: forward row k is use k,
-// backward step k (row n-1-k) is use n + k; use u sits in group u / G at
-// row slot u % G.
-template <int E, int G>
-__global__ void __launch_bounds__(IW_THREADS, (G == 2 && E <= 10) ? 3 : 1)
-    k_ilu(int n, int mode_arg, int S, IwLayout lay, SliceState* __restrict__ st, double* __restrict__ part,
-          float2* __restrict__ x, const float2* __restrict__ d, float2* __restrict__ r,
-          const float2* __restrict__ q, const float2* __restrict__ atb, float2* __restrict__ y,
-          float2* __restrict__ z, const float* __restrict__ ia, const float* __restrict__ wtv, int fuse,
-          PcgSched ps, int wait_test, const float* __restrict__ wtv2, int alpha_np) {
-  const int s = blockIdx.x;
-  if (!slice_running(st, s)) return;
-  // ILU_PER_SLICE: the first residual for a slice at the start of its outer
-  // step, a PCG step otherwise
-  int ph = st[s].phase;
-  if (alpha_np > 0 && mode_arg == ILU_PER_SLICE && ph == PH_PCG) {
-    // alpha = rho / <d, S d> from the S apply's alpha_np partial sums, as the
-    // scalar kernel forms it (same order); a slice that stops here (rho = 0
-    // or a breakdown) does nothing more in this macro step
-    __shared__ int ph_alpha;
-    if (threadIdx.x == 0) {
-      const double* pp = part + ((size_t)s * NSLOT + SLOT_DQ) * MAXPART;
-      double dq = 0.0;
-      for (int i = 0; i < alpha_np; ++i) dq += pp[i];
-      pcg_alpha_from(st + s, dq);
-      ph_alpha = st[s].done ? -1 : st[s].phase;
-    }
-    __syncthreads();
-    if (ph_alpha < 0) return;
-    ph = ph_alpha;
-  }
-  if (mode_arg == ILU_PER_SLICE && !slice_working(ph)) return;
-  const int mode = mode_arg != ILU_PER_SLICE ? mode_arg : (ph == PH_START ? ILU_INIT : ILU_STEP);
-  // wait_test (failure-detection test only): the producer issues no copy and
-  // every wait gives up after its first poll, so the waits run out with
-  // nothing in flight and the slice is reported faulted
-  const int tries = wait_test ? 0 : 10000;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ __align__(8) uint64_t bar_full[IW_MAXSTAGES], bar_empty[IW_MAXSTAGES];
-  __shared__ __align__(8) uint64_t bar_ready[IW_MAXSTAGES], bar_used[IW_MAXSTAGES];
-  __shared__ int y_stored;  // 1 once every y row is stored and fenced
-  __shared__ volatile int abort_flag;
-  __shared__ double red[32];
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int NCH = n >> 1;
-  const int NG = n / G;
-  const float lam = st[s].lam_tv;
-  const float alpha = (float)st[s].alpha;
-  const size_t base = (size_t)s * n * n;
-  // L2 policies: y, W and 1/a are read again by the backward sweep; the
-  // rest passes through once
-  const uint64_t pol_keep = l2_evict_last(), pol_stream = l2_evict_first();
-  if (t == 0) {
-    for (int i = 0; i < S; ++i) {
-      mbar_init(&bar_full[i], 1);
-      mbar_init(&bar_empty[i], IW_HWARPS);
-      mbar_init(&bar_ready[i], IW_HWARPS);
-      mbar_init(&bar_used[i], 1);
-    }
-    y_stored = 0;
-    abort_flag = 0;
-  }
-  if (lay.ns > n) {  // slots of columns >= n are never written: make them zero, not garbage
-    for (int i = t; i < S * G * lay.ns; i += IW_THREADS) {
-      const int row = i / lay.ns;
-      unsigned char* sp = smem + (size_t)(row / G) * lay.bytes + lay.oSC + (size_t)(row % G) * 16 * lay.ns;
-      reinterpret_cast<float4*>(sp)[i % lay.ns] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  }
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  __syncthreads();
-  auto fault = [&]() {
-    abort_flag = 1;
-    st[s].fault = 1;
-  };
-  // lane-major slot of column c (lane c / E, element c % E), XOR-swizzled so
-  // that helper stores of neighbouring columns hit different banks
-  auto slot_of = [&](int c) -> int {
-    const int e = c % E;
-    return e * 32 + ((c / E) ^ (e & 31));
-  };
-  auto sc_row = [&](int stg, int slot) -> float4* {
-    return reinterpret_cast<float4*>(smem + (size_t)stg * lay.bytes + lay.oSC + (size_t)slot * 16 * lay.ns);
-  };
-
-  float rr = 0.f, rho = 0.f;
-
-  if (warp == 1) {
-    // ============================================================ scan warp
-    // (alone on its SM sub-partition: of the five warps, 0 and 4 share one)
-    float2 vab[E];  // y of the row above (forward) / z of the row below (backward)
-    RingPos pos{0, 0u};
-    bool ok = true;
-    for (int sweep = 0; sweep < 2 && ok; ++sweep) {
-      if (sweep == 1) {
-        // y goes back to global memory and is re-read by bulk copies, so
-        // order the generic stores before the async proxy
-        fence_proxy_async_global();
-        __syncwarp();
-        if (lane == 0) st_release(&y_stored, 1);
-      }
-#pragma unroll
-      for (int e = 0; e < E; ++e) vab[e] = make_float2(0.f, 0.f);
-      for (int gg = 0; gg < NG; ++gg) {
-        if (!__all_sync(0xffffffffu, mbar_wait(&bar_ready[pos.s], pos.ph, tries))) {
-          ok = false;
-          break;
-        }
-        float4 cA[E], cB[E];
-        {
-          const float4* sc = sc_row(pos.s, 0);
-#pragma unroll
-          for (int e = 0; e < E; ++e) cA[e] = sc[e * 32 + (lane ^ (e & 31))];
-        }
-#pragma unroll
-        for (int i = 0; i < G; ++i) {
-          float4(&cur)[E] = (i & 1) ? cB : cA;
-          float4(&nxt)[E] = (i & 1) ? cA : cB;
-          if (i + 1 < G) {  // the next row of this group, while this one is scanned
-            const float4* sc = sc_row(pos.s, i + 1);
-#pragma unroll
-            for (int e = 0; e < E; ++e) nxt[e] = sc[e * 32 + (lane ^ (e & 31))];
-          } else {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bar_used[pos.s]);
-          }
-          float2 tv[E];
-          float A = 1.f;
-          float2 B = make_float2(0.f, 0.f);
-          if (sweep == 0) {
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-              tv[e] = make_float2(fmaf(cur[e].z, vab[e].x, cur[e].x), fmaf(cur[e].z, vab[e].y, cur[e].y));
-              B = make_float2(fmaf(cur[e].w, B.x, tv[e].x), fmaf(cur[e].w, B.y, tv[e].y));
-              A *= cur[e].w;
-            }
-            float2 v = warp_affine_exclusive<false>(A, B);
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-              v = make_float2(fmaf(cur[e].w, v.x, tv[e].x), fmaf(cur[e].w, v.y, tv[e].y));
-              vab[e] = v;
-            }
-            store_lane_row<E>(y + base + (size_t)(gg * G + i) * n, E * lane, n, vab, pol_keep);
-          } else {
-#pragma unroll
-            for (int e = E - 1; e >= 0; --e) {
-              tv[e] = make_float2(fmaf(cur[e].z, vab[e].x, cur[e].x), fmaf(cur[e].z, vab[e].y, cur[e].y));
-              B = make_float2(fmaf(cur[e].w, B.x, tv[e].x), fmaf(cur[e].w, B.y, tv[e].y));
-              A *= cur[e].w;
-            }
-            float2 v = warp_affine_exclusive<true>(A, B);
-#pragma unroll
-            for (int e = E - 1; e >= 0; --e) {
-              v = make_float2(fmaf(cur[e].w, v.x, tv[e].x), fmaf(cur[e].w, v.y, tv[e].y));
-              vab[e] = v;
-            }
-            store_lane_row<E>(z + base + (size_t)(n - 1 - gg * G - i) * n, E * lane, n, vab, pol_stream);
-          }
-        }
-        pos.next(S);
-      }
-    }
-    if (!ok) fault();
-  } else if (warp == 0) {
-    // ============================================================= producer
-    if (lane == 0) {
-      const float2* rsrc = (mode == ILU_INIT) ? atb : r;
-      const bool init = mode == ILU_INIT;
-      const unsigned c8 = 8u * n * G, c4 = 4u * n * G;
-      RingPos pos{0, 0u};
-      bool ok = true;
-      for (int g = 0; g < 2 * NG && ok; ++g) {
-        if (abort_flag) break;
-        if (wait_test) {  // no copy is issued: the consumers' waits run out
-          ok = false;
-          break;
-        }
-        // the stage's previous group (g - S) has been left by every helper
-        if (g >= S && !mbar_wait(&bar_empty[pos.s], pos.ph ^ 1u, tries)) {
-          ok = false;
-          break;
-        }
-        if (g == NG && poll_at_least(&y_stored, 1, tries ? 1 << 24 : 0) < 1) {  // backward copies read y
-          ok = false;
-          break;
-        }
-        unsigned char* sp = smem + (size_t)pos.s * lay.bytes;
-        uint64_t* bar = &bar_full[pos.s];
-        const unsigned cw2 = wtv2 ? c4 : 0u;
-        if (g < NG) {
-          const size_t go = base + (size_t)g * G * n;
-          mbar_arrive_tx(bar, (init ? 2 * c8 + 2 * c4 : 4 * c8 + 2 * c4) + cw2);
-          // streamed once: r, q, x, d; read again by the backward sweep: W, 1/a
-          bulk_g2s_hint(sp, rsrc + go, c8, bar, pol_stream);
-          bulk_g2s_hint(sp + lay.oQ, q + go, c8, bar, pol_stream);
-          if (!init) {
-            bulk_g2s_hint(sp + lay.oX, x + go, c8, bar, pol_stream);
-            bulk_g2s_hint(sp + lay.oD, d + go, c8, bar, pol_stream);
-          }
-          bulk_g2s_hint(sp + lay.oW, wtv + go, c4, bar, pol_keep);
-          bulk_g2s_hint(sp + lay.oIA, ia + go, c4, bar, pol_keep);
-          if (wtv2) bulk_g2s_hint(sp + lay.oW2, wtv2 + go, c4, bar, pol_keep);
-        } else {
-          const size_t go = base + (size_t)(n - (g - NG + 1) * G) * n;
-          mbar_arrive_tx(bar, c8 + 2 * c4 + cw2);
-          // last uses
-          bulk_g2s_hint(sp, y + go, c8, bar, pol_stream);
-          bulk_g2s_hint(sp + lay.oW, wtv + go, c4, bar, pol_stream);
-          bulk_g2s_hint(sp + lay.oIA, ia + go, c4, bar, pol_stream);
-          if (wtv2) bulk_g2s_hint(sp + lay.oW2, wtv2 + go, c4, bar, pol_stream);
-        }
-        pos.next(S);
-      }
-      if (!ok) fault();
-    }
-  } else {
-    // ============================================================== helpers
-    const int hh = t - 64;
-    float2 prev[IW_MAXCH];  // ia of the row above (forward) / W of the row below (backward)
-    // sums per column chunk: each chunk meets its rows in the same order for
-    // every ring shape, so the totals do not depend on G or S
-    float rr_c[IW_MAXCH], rho_c[IW_MAXCH];
-#pragma unroll
-    for (int c = 0; c < IW_MAXCH; ++c) rr_c[c] = rho_c[c] = 0.f;
-#pragma unroll
-    for (int c = 0; c < IW_MAXCH; ++c) prev[c] = make_float2(0.f, 0.f);
-    bool ok = true;
-    RingPos pos{0, 0u};
-    const size_t nG4 = (size_t)4 * n;  // bytes per float row
-    for (int g = 0; g < 2 * NG && ok; ++g) {
-      if (__any_sync(0xffffffffu, abort_flag != 0)) break;
-      if (g == NG) {
-#pragma unroll
-        for (int c = 0; c < IW_MAXCH; ++c) prev[c] = make_float2(0.f, 0.f);
-      }
-      unsigned char* sp = smem + (size_t)pos.s * lay.bytes;
-      bool got = mbar_wait(&bar_full[pos.s], pos.ph, tries);
-      if (g >= S) got = got && mbar_wait(&bar_used[pos.s], pos.ph ^ 1u, tries);  // scan warp left group g - S
-      if (!__all_sync(0xffffffffu, got)) {
-        ok = false;
-        break;
-      }
-      if (g < NG) {
-#pragma unroll
-        for (int ch = 0; ch < IW_MAXCH; ++ch) {
-          const int j = hh + IW_HELPERS * ch;
-          if (j < NCH) {
-            const int c = 2 * j;
-#pragma unroll
-            for (int i = 0; i < G; ++i) {
-              const size_t g0 = base + (size_t)(g * G + i) * n + c;
-              const unsigned char* rowp = sp + (size_t)i * 8 * n;
-              const float4 r4 = *reinterpret_cast<const float4*>(rowp + 16 * j);
-              const float4 q4 = *reinterpret_cast<const float4*>(rowp + lay.oQ + 16 * j);
-              float4 rn;
-              if (mode == ILU_INIT) {
-                rn = make_float4(r4.x - q4.x, r4.y - q4.y, r4.z - q4.z, r4.w - q4.w);
-              } else {
-                const float4 x4 = *reinterpret_cast<const float4*>(rowp + lay.oX + 16 * j);
-                const float4 d4 = *reinterpret_cast<const float4*>(rowp + lay.oD + 16 * j);
-                rn = make_float4(fmaf(-alpha, q4.x, r4.x), fmaf(-alpha, q4.y, r4.y), fmaf(-alpha, q4.z, r4.z),
-                                 fmaf(-alpha, q4.w, r4.w));
-                st_hint_f4(x + g0,
-                           make_float4(fmaf(alpha, d4.x, x4.x), fmaf(alpha, d4.y, x4.y), fmaf(alpha, d4.z, x4.z),
-                                       fmaf(alpha, d4.w, x4.w)),
-                           pol_stream);
-              }
-              st_hint_f4(r + g0, rn, pol_stream);
-              rr_c[ch] += rn.x * rn.x + rn.y * rn.y + rn.z * rn.z + rn.w * rn.w;
-              const float* wrow = reinterpret_cast<const float*>(sp + lay.oW + i * nG4);
-              const float* arow = reinterpret_cast<const float*>(sp + lay.oIA + i * nG4);
-              const float2 w2 = *reinterpret_cast<const float2*>(wrow + c);
-              const float2 a2 = *reinterpret_cast<const float2*>(arow + c);
-              const float ial = c > 0 ? arow[c - 1] : 0.f;
-              const float2 aab = prev[ch];  // ia of the row above
-              const float lw0 = lam * w2.x, lw1 = lam * w2.y;
-              // vertical couplings use W2 (l1 TV), else W
-              float lv0 = lw0, lv1 = lw1;
-              if (wtv2) {
-                const float2 v2 = *reinterpret_cast<const float2*>(
-                    reinterpret_cast<const float*>(sp + lay.oW2 + i * nG4) + c);
-                lv0 = lam * v2.x;
-                lv1 = lam * v2.y;
-              }
-              float4* sc = sc_row(pos.s, i);
-              sc[slot_of(c)] = make_float4(rn.x, rn.y, lv0 * aab.x, lw0 * ial);
-              sc[slot_of(c + 1)] = make_float4(rn.z, rn.w, lv1 * aab.y, lw1 * a2.x);
-              prev[ch] = a2;
-            }
-          }
-        }
-      } else {
-#pragma unroll
-        for (int ch = 0; ch < IW_MAXCH; ++ch) {
-          const int j = hh + IW_HELPERS * ch;
-          if (j < NCH) {
-            const int c = 2 * j;
-#pragma unroll
-            for (int i = 0; i < G; ++i) {
-              const int o = G - 1 - i;  // memory row of processing slot i
-              const float4 y4 = *reinterpret_cast<const float4*>(sp + (size_t)o * 8 * n + 16 * j);
-              const float* wrow = reinterpret_cast<const float*>(sp + lay.oW + o * nG4);
-              const float* arow = reinterpret_cast<const float*>(sp + lay.oIA + o * nG4);
-              const float2 w2 = *reinterpret_cast<const float2*>(wrow + c);
-              const float2 a2 = *reinterpret_cast<const float2*>(arow + c);
-              const float w3 = c + 2 < n ? wrow[c + 2] : 0.f;
-              const float2 wbl = prev[ch];  // W (W2 for l1 TV) of the row below
-              const float la0 = lam * a2.x, la1 = lam * a2.y;
-              const float2 t0 = make_float2(a2.x * y4.x, a2.x * y4.y), t1 = make_float2(a2.y * y4.z, a2.y * y4.w);
-              rho_c[ch] = fmaf(t0.x, y4.x, fmaf(t0.y, y4.y, rho_c[ch]));
-              rho_c[ch] = fmaf(t1.x, y4.z, fmaf(t1.y, y4.w, rho_c[ch]));
-              float4* sc = sc_row(pos.s, i);
-              sc[slot_of(c)] = make_float4(t0.x, t0.y, la0 * wbl.x, la0 * w2.y);
-              sc[slot_of(c + 1)] = make_float4(t1.x, t1.y, la1 * wbl.y, la1 * w3);
-              prev[ch] = wtv2 ? *reinterpret_cast<const float2*>(
-                                    reinterpret_cast<const float*>(sp + lay.oW2 + o * nG4) + c)
-                              : w2;
-            }
-          }
-        }
-      }
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&bar_empty[pos.s]);
-        mbar_arrive(&bar_ready[pos.s]);
-      }
-      pos.next(S);
-    }
-    if (!ok) fault();
-#pragma unroll
-    for (int c = 0; c < IW_MAXCH; ++c) {
-      rr += rr_c[c];
-      rho += rho_c[c];
-    }
-  }
-  __syncthreads();
-  const double trz = block_sum((double)rho, red);
-  __syncthreads();
-  const double trr = block_sum((double)rr, red);
-  if (t == 0) {
-    part[((size_t)s * NSLOT + SLOT_RZ) * MAXPART] = trz;
-    part[((size_t)s * NSLOT + SLOT_RR) * MAXPART] = trr;
-    if (fuse && !abort_flag) {
-      if (mode == ILU_INIT)
-        pcg_rho_init_from(st + s, 0.0 + trz, 0.0 + trr);
-      else
-        pcg_beta_from(st + s, 0.0 + trz, 0.0 + trr, ps);
-    }
-  }
-}
-
-typedef void (*IluKernel)(int, int, int, IwLayout, SliceState*, double*, float2*, const float2*, float2*,
-                          const float2*, const float2*, float2*, float2*, const float*, const float*, int, PcgSched,
-                          int, const float*, int);
-template <int G>
-static IluKernel ilu_kernel_g(int E) {
-  switch (E) {
-    case 1: return k_ilu<1, G>;
-    case 2: return k_ilu<2, G>;
-    case 3: return k_ilu<3, G>;
-    case 4: return k_ilu<4, G>;
-    case 5: return k_ilu<5, G>;
-    case 6: return k_ilu<6, G>;
-    case 8: return k_ilu<8, G>;
-    case 10: return k_ilu<10, G>;
-    case 12: return k_ilu<12, G>;
-    case 16: return k_ilu<16, G>;
-    default: return nullptr;
-  }
-}
-static IluKernel ilu_kernel(int n, int G) {
-  const int E = iw_cols_per_lane(n);
-  return G == 4 ? ilu_kernel_g<4>(E) : ilu_kernel_g<2>(E);
-}
-
-static constexpr int ILU_SMEM_MAX = 200 * 1024;
-
-bool ilu_prepare() {
-  bool ok = true;
-  for (int e : {1, 2, 3, 4, 5, 6, 8, 10, 12, 16})
-    for (int G : {2, 4})
-      ok = cudaFuncSetAttribute(ilu_kernel(32 * e, G), cudaFuncAttributeMaxDynamicSharedMemorySize, ILU_SMEM_MAX) ==
-               cudaSuccess && ok;
-  return ok;
-}
-
-// Ring shape, encoded 10 * G + S: G rows per stage and S stages.  With one
-// CTA per SM (batch <= 152) the ring takes 4-row stages, three of them as
-// long as they fit; with more CTAs per SM, 2-row stages in the shared
-// memory each CTA gets.
-int ilu_default_shape(int n, int batch, bool aniso) {
-  int per_sm = (batch + 151) / 152;
-  if (per_sm > 3) per_sm = 3;
-  const int budget = per_sm == 1 ? ILU_SMEM_MAX : (224 * 1024) / per_sm - 2048;
-  for (int G : {4, 2}) {
-    if (per_sm > 1 && G == 4) continue;
-    int S = budget / iw_layout(n, G, aniso).bytes;
-    if (S > 4) S = 4;
-    if (S >= 2) return 10 * G + S;
-  }
-  return 10 * 2 + 2;
-}
-
-bool ilu_shape_fits(int n, int shape, bool aniso) {
-  const int G = shape / 10, S = shape % 10;
-  if ((G != 2 && G != 4) || S < 2 || S > IW_MAXSTAGES || n % G) return false;
-  return (long)S * iw_layout(n, G, aniso).bytes <= ILU_SMEM_MAX;
-}
-
-void ilu_step(int batch, int n, cudaStream_t s, SliceState* st, double* part, int mode, float2* x,
-              const float2* d, float2* r, const float2* q, const float2* atb, float2* y, float2* z,
-              const float* ia, const float* wtv, int shape, int fuse_scalars, PcgSched ps, int wait_test,
-              const float* wtv2, int alpha_np) {
-  const bool aniso = wtv2 != nullptr;
-  if (shape <= 0 || !ilu_shape_fits(n, shape, aniso)) shape = ilu_default_shape(n, batch, aniso);
-  const int G = shape / 10, S = shape % 10;
-  const IwLayout lay = iw_layout(n, G, aniso);
-  ilu_kernel(n, G)<<<batch, IW_THREADS, (size_t)S * lay.bytes, s>>>(n, mode, S, lay, st, part, x, d, r, q, atb, y,
-                                                                     z, ia, wtv, fuse_scalars, ps, wait_test, wtv2,
-                                                                     alpha_np);
-}
-
 // =========================================================== PCG vectors ==
 
 int axpy_ctas(int n) {
@@ -1961,8 +1228,7 @@ int axpy_ctas(int n) {
 }
 
 __global__ void k_axpy(int N, int mode_arg, const SliceState* __restrict__ st, double* __restrict__ part,
-                       float2* __restrict__ x, const float2* __restrict__ d, float2* __restrict__ r,
-                       const float2* __restrict__ q, const float2* __restrict__ atb) {
+                       float2* r, const float2* __restrict__ q, const float2* atb) {
   const int s = blockIdx.y;
   if (!slice_running(st, s)) return;
   const int ph = st[s].phase;
@@ -1973,19 +1239,26 @@ __global__ void k_axpy(int N, int mode_arg, const SliceState* __restrict__ st, d
   const size_t base = (size_t)s * N;
   const int chunk = (N + gridDim.x - 1) / gridDim.x;
   const int lo = blockIdx.x * chunk, hi = min(N, lo + chunk);
+  const float2* src = mode == AXPY_INIT ? atb : r;
+  constexpr int UN = 4;  // elements in flight per thread
   float acc = 0.f;
-  for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    const size_t g = base + i;
-    if (mode == AXPY_INIT) {
-      const float2 rv = csub(atb[g], q[g]);
-      r[g] = rv;
-      acc += cabs2(rv);
-    } else {
-      x[g] = cfma(alpha, d[g], x[g]);
-      if (mode == AXPY_STEP) {
-        const float2 rv = cfma(-alpha, q[g], r[g]);
-        r[g] = rv;
-        acc += cabs2(rv);
+  for (int i = lo + threadIdx.x; i < hi; i += UN * blockDim.x) {
+    float2 rv[UN], qv[UN];
+#pragma unroll
+    for (int e = 0; e < UN; ++e) {
+      const int j = i + e * blockDim.x;
+      if (j < hi) {
+        rv[e] = src[base + j];
+        qv[e] = q[base + j];
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < UN; ++e) {
+      const int j = i + e * blockDim.x;
+      if (j < hi) {
+        rv[e] = mode == AXPY_INIT ? csub(rv[e], qv[e]) : cfma(-alpha, qv[e], rv[e]);
+        r[base + j] = rv[e];
+        acc += cabs2(rv[e]);
       }
     }
   }
@@ -1993,16 +1266,15 @@ __global__ void k_axpy(int N, int mode_arg, const SliceState* __restrict__ st, d
   if (threadIdx.x == 0) part[((size_t)s * NSLOT + SLOT_RR) * MAXPART + blockIdx.x] = tot;
 }
 
-void axpy_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* x,
-               const float2* d, float2* r, const float2* q, const float2* atb) {
-  k_axpy<<<dim3(axpy_ctas(n), batch), 256, 0, s>>>(n * n, mode, st, part, x, d, r, q, atb);
+void axpy_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* r,
+               const float2* q, const float2* atb) {
+  k_axpy<<<dim3(axpy_ctas(n), batch), 256, 0, s>>>(n * n, mode, st, part, r, q, atb);
 }
 
 // Residual update with a diagonal preconditioner (Jacobi PCG, sdiag = 1 /
 // diag(S)) or none (standard CG, sdiag null), for the comparison of Sec. 5.2.
 __global__ void k_axpy_diag(int N, int mode_arg, const SliceState* __restrict__ st, double* __restrict__ part,
-                            float2* __restrict__ x, const float2* __restrict__ d, float2* __restrict__ r,
-                            const float2* __restrict__ q, const float2* __restrict__ atb,
+                            float2* __restrict__ r, const float2* __restrict__ q, const float2* __restrict__ atb,
                             const float* __restrict__ sdiag, float2* __restrict__ z) {
   const int s = blockIdx.y;
   if (!slice_running(st, s)) return;
@@ -2017,13 +1289,7 @@ __global__ void k_axpy_diag(int N, int mode_arg, const SliceState* __restrict__ 
   float rz = 0.f, rr = 0.f;
   for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
     const size_t g = base + i;
-    float2 rv;
-    if (mode == AXPY_INIT) {
-      rv = csub(atb[g], q[g]);
-    } else {
-      x[g] = cfma(alpha, d[g], x[g]);
-      rv = cfma(-alpha, q[g], r[g]);
-    }
+    const float2 rv = mode == AXPY_INIT ? csub(atb[g], q[g]) : cfma(-alpha, q[g], r[g]);
     r[g] = rv;
     const float sc = sdiag ? sdiag[g] : 1.f;
     z[g] = cscale(rv, sc);
@@ -2040,9 +1306,9 @@ __global__ void k_axpy_diag(int N, int mode_arg, const SliceState* __restrict__ 
   }
 }
 
-void axpy_diag_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* x,
-                    const float2* d, float2* r, const float2* q, const float2* atb, const float* sdiag, float2* z) {
-  k_axpy_diag<<<dim3(axpy_ctas(n), batch), 256, 0, s>>>(n * n, mode, st, part, x, d, r, q, atb, sdiag, z);
+void axpy_diag_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* r,
+                    const float2* q, const float2* atb, const float* sdiag, float2* z) {
+  k_axpy_diag<<<dim3(axpy_ctas(n), batch), 256, 0, s>>>(n * n, mode, st, part, r, q, atb, sdiag, z);
 }
 
 __global__ void k_jacobi_wavelet(int N, const SliceState* __restrict__ st, const float* __restrict__ wdiag,
@@ -2062,21 +1328,24 @@ void jacobi_wavelet_setup(int batch, int n, cudaStream_t s, const SliceState* st
 }
 
 // End of a slice's outer step (PH_END): x^{k+1} = x^k + dx, where
-// dx = sum_j alpha_j d_j was accumulated from zero by the PCG steps (so its
-// rounding is relative to the step, not to x), and dx is cleared for the next
-// outer step; partial ||dx||^2 (SLOT_DX) and ||x^k||^2 (SLOT_XX) for the
+// dx = sum_j alpha_j d_j was accumulated from zero by the row FFTs of the PCG
+// steps (so its rounding is relative to the step, not to x), up to the last
+// step's alpha d, which is added here, and dx is cleared for the next outer
+// step; partial ||dx||^2 (SLOT_DX) and ||x^k||^2 (SLOT_XX) for the
 // relative change.  Slices stopped by a breakdown are done and keep x^k.
 __global__ void k_outer_apply(int N, const SliceState* __restrict__ st, float2* __restrict__ x,
-                              float2* __restrict__ dx, double* __restrict__ part) {
+                              float2* __restrict__ dx, const float2* __restrict__ d,
+                              double* __restrict__ part) {
   const int s = blockIdx.y;
   if (!slice_running(st, s) || st[s].phase != PH_END) return;
   __shared__ double red[32];
   const size_t base = (size_t)s * N;
   const int chunk = (N + gridDim.x - 1) / gridDim.x;
   const int lo = blockIdx.x * chunk, hi = min(N, lo + chunk);
+  const float alpha = (float)st[s].alpha;
   float a = 0.f, b = 0.f;
   for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    const float2 xv = x[base + i], dv = dx[base + i];
+    const float2 xv = x[base + i], dv = cfma(alpha, d[base + i], dx[base + i]);
     a += cabs2(dv);
     b += cabs2(xv);
     x[base + i] = cadd(xv, dv);
@@ -2091,9 +1360,9 @@ __global__ void k_outer_apply(int N, const SliceState* __restrict__ st, float2* 
   }
 }
 
-void outer_apply(int batch, int n, cudaStream_t s, const SliceState* st, float2* x, float2* dx,
+void outer_apply(int batch, int n, cudaStream_t s, const SliceState* st, float2* x, float2* dx, const float2* d,
                  double* part) {
-  k_outer_apply<<<dim3(axpy_ctas(n), batch), 256, 0, s>>>(n * n, st, x, dx, part);
+  k_outer_apply<<<dim3(axpy_ctas(n), batch), 256, 0, s>>>(n * n, st, x, dx, d, part);
 }
 
 // ================================================================ groups ===

@@ -26,6 +26,10 @@ struct FftArgs {
   const float* wtv2 = nullptr;  // l1 TV: the vertical weights W2 (wtv then holds W1)
   float2* q = nullptr;
   const float2* xs = nullptr;   // row FFT, per-slice mode: x^k of slices starting an outer step
+  // row FFT: z, row IFFT: q in the ILU's skewed layout (k_ilu.cu); q of a
+  // slice starting an outer step is then its first residual atb - S x^k
+  int skew = 0;
+  float2* dx = nullptr;         // row FFT: dx += alpha d of the PCG step before
   int mode = 0;
   int real = 0;
 };
@@ -90,41 +94,48 @@ void wavelet_diag(int batch, int n, int levels, cudaStream_t s, const SliceState
                   float* out, const float* sqtab, const int* sqlen);
 void penta_setup(int batch, int n, cudaStream_t s, const SliceState* st, const float* wtv, const float* wtv2,
                  const float* wdiag, float* ia);
-// ia = 1/a -> 1/d, the ILU(0) pivots (updated pivots, zero fill)
-void ilu0_pivots(int batch, int n, cudaStream_t s, const SliceState* st, const float* wtv, const float* wtv2,
-                 float* ia);
+// ---- the TV preconditioner's sweeps (k_ilu.cu), on arrays in a skewed layout ----
+size_t ilu_slice_elems(int n);  // float2 per slice of a skewed array
+bool ilu_prepare();
+// wa = (lam W, 1/a) skewed, and for l1 TV w2s = lam W2 skewed, of the slices st
+// shows running (or all); before a sweep with new weights
+void ilu_pack(int batch, int n, cudaStream_t s, const SliceState* st, bool all, const float* wtv,
+              const float* wtv2, const float* ia, float4* wa, float2* w2s);
+// 1/a -> 1/d, the ILU(0) pivots (updated pivots, zero fill), in wa and ia
+void ilu0_pivots(int batch, int n, cudaStream_t s, SliceState* st, const SliceState* view, float4* wa,
+                 const float2* w2s, float* ia);
+// a complex array between the natural layout (stride n n) and the skewed one
+void ilu_skew(int batch, int n, cudaStream_t s, bool to_skewed, const float2* src, float2* dst);
 
-// In the PCG-step kernels below, `x` is the vector that receives alpha d: the
-// solver passes the outer step's update accumulator dx (added to the iterate
-// once per outer step by outer_apply).
-enum IluMode { ILU_INIT = 0, ILU_STEP = 1, ILU_LAST = 2, ILU_PER_SLICE = -1 };
-// shape: shared-memory ring, 10 * rows per stage + stages (0: chosen from n and batch)
+// The outer step's update dx = sum_j alpha_j d_j is kept one step behind: the
+// row FFT, which reads d anyway, adds alpha d of the step before, and
+// outer_apply the last one.
+enum IluMode { ILU_INIT = 0, ILU_STEP = 1, ILU_PER_SLICE = -1 };
+// all arrays skewed.  INIT: r = q (the first residual); STEP: r -= alpha q.
+// w2s null: isotropic TV.
+// shape: the sweeps' chunks (ilu_default_shape; 0: by the batch)
 // fuse_scalars: the CTA finishes the PCG scalars itself from its sums (rho
 // at ILU_INIT; rr, the residual test against pcg_tol, beta and rho at ILU_STEP)
 // alpha_np > 0 (ILU_PER_SLICE): the CTA of a slice in PCG first forms alpha
 // from the S apply's alpha_np partial sums of <d, S d> (pcg_alpha's work)
-void ilu_step(int batch, int n, cudaStream_t s, SliceState* st, double* part, int mode,
-              float2* x, const float2* d, float2* r, const float2* q, const float2* atb, float2* y,
-              float2* z, const float* ia, const float* wtv, int shape, int fuse_scalars = 0,
-              PcgSched ps = PcgSched{0.f, 0, 1 << 30, 0, 0}, int wait_test = 0, const float* wtv2 = nullptr,
-              int alpha_np = 0);
-// aniso: the ring stages also hold the second weight array of l1 TV
-int ilu_default_shape(int n, int batch, bool aniso = false);
+void ilu_step(int batch, int n, cudaStream_t s, SliceState* st, double* part, int mode, float2* r, const float2* q,
+              float2* y, float2* z, const float4* wa, const float2* w2s, int shape, int fuse_scalars = 0,
+              PcgSched ps = PcgSched{0.f, 0, 1 << 30, 0, 0}, int wait_test = 0, int alpha_np = 0);
+int ilu_default_shape(int batch);
 bool ilu_shape_fits(int n, int shape, bool aniso = false);
 
 // AXPY_PER_SLICE (and ILU_PER_SLICE, SCALARS_PER_SLICE, mode < 0 of the row
 // FFT): each slice's own phase picks the first residual (PH_BOUNDARY) or a
 // PCG step (PH_PCG).
-enum AxpyMode { AXPY_INIT = 0, AXPY_STEP = 1, AXPY_LAST = 2, AXPY_PER_SLICE = -1 };
-// Residual update (INIT: r = A^H b - q; STEP: r -= alpha q, x += alpha d) with
-// a diagonal preconditioner z = sdiag o r (sdiag null: z = r), partial
+enum AxpyMode { AXPY_INIT = 0, AXPY_STEP = 1, AXPY_PER_SLICE = -1 };
+// Residual update (INIT: r = A^H b - q; STEP: r -= alpha q) with a diagonal preconditioner z = sdiag o r (sdiag null: z = r), partial
 // Re<r, z> into SLOT_RZ and ||r||^2 into SLOT_RR (axpy_ctas parts).
-void axpy_diag_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* x,
-                    const float2* d, float2* r, const float2* q, const float2* atb, const float* sdiag, float2* z);
+void axpy_diag_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* r,
+                    const float2* q, const float2* atb, const float* sdiag, float2* z);
 // Jacobi scale of a wavelet-only system: ia = 1 / (abar + lam diag(Phi^T W Phi)).
 void jacobi_wavelet_setup(int batch, int n, cudaStream_t s, const SliceState* st, const float* wdiag, float* ia);
-void axpy_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode,
-               float2* x, const float2* d, float2* r, const float2* q, const float2* atb);
+void axpy_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* r,
+               const float2* q, const float2* atb);
 int axpy_ctas(int n);
 
 void group_norms(int batch, int n, int n_groups, cudaStream_t s, const SliceState* st,
@@ -157,9 +168,10 @@ void pcg_scalars(int batch, cudaStream_t s, SliceState* st, const double* part, 
 // view = st with every slice not at the start of its outer step marked done
 // (and the slices whose outer step is due move to PH_START)
 void boundary_view(int batch, cudaStream_t s, SliceState* st, SliceState* view);
-// x += dx (the outer step's accumulated update) with partial ||dx||^2 and
-// ||x||^2 (before the update) for the relative change.
-void outer_apply(int batch, int n, cudaStream_t s, const SliceState* st, float2* x, float2* dx,
+// x += dx + alpha d (the outer step's accumulated update and its last step)
+// with partial norms squared of that update and of x before it, for the
+// relative change; dx cleared.
+void outer_apply(int batch, int n, cudaStream_t s, const SliceState* st, float2* x, float2* dx, const float2* d,
                  double* part);
 // plateau_after: first outer step at which kind 1 also stops on a plateau
 void outer_end(int batch, cudaStream_t s, SliceState* st, const double* part, int nparts,
