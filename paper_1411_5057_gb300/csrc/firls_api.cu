@@ -724,6 +724,7 @@ extern "C" firls_status firls_create(firls_ctx** out, int n_rows, int n_cols, in
   cudaMemcpy(c->tw, tw.data(), sizeof(float2) * n, cudaMemcpyHostToDevice);
   // weights that are read out before any were formed are 0
   cudaMemset(c->wtv, 0, sizeof(float) * BN);
+  cudaMemset(c->ww, 0, sizeof(float) * BN);
   // d is read (times 0) nowhere, but keep the workspace finite
   cudaMemset(c->d, 0, sizeof(float2) * BN);
   cudaMemset(c->part, 0, sizeof(double) * batch * NSLOT * MAXPART);
