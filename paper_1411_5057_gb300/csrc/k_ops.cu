@@ -1100,10 +1100,25 @@ void tv_sum(int batch, int n, cudaStream_t s, const float2* x, float eps, double
 
 // ========================================================== PCG scalars ===
 
+// The scalar kernels give a warp to each slice: its lanes fetch the partial sums
+// at once and lane 0 adds them in order, as one thread did (which took 15 us at
+// 60 slices of three contrasts, one load after the other).
+constexpr int SC_WARPS = 4;  // slices per CTA
+FI int sc_slice() { return blockIdx.x * SC_WARPS + (threadIdx.x >> 5); }
+static int sc_ctas(int batch) { return (batch + SC_WARPS - 1) / SC_WARPS; }
+
+// sum of slice s's np partial sums, valid in lane 0; called by a whole warp
 FI double sum_parts(const double* part, int s, int slot, int np) {
+  __shared__ double buf[SC_WARPS][MAXPART];
+  double* b = buf[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
   const double* p = part + ((size_t)s * NSLOT + slot) * MAXPART;
+  __syncwarp();
+  for (int i = lane; i < np; i += 32) b[i] = p[i];
+  __syncwarp();
   double a = 0.0;
-  for (int i = 0; i < np; ++i) a += p[i];
+  if (lane == 0)
+    for (int i = 0; i < np; ++i) a += b[i];
   return a;
 }
 
@@ -1122,13 +1137,15 @@ FI double image_parts(const double* part, int s, int slot, int np, int C) {
 
 __global__ void k_state_init(int B, SliceState* st, const double* part, int np, const int* counts, int N,
                              const float* lam, const float* lam_tv, float eps, int outer_max, int phase, int C) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = sc_slice();
   if (s >= B) return;
+  const double rhs2 = image_parts(part, s, SLOT_RHS, np, C);
+  if (threadIdx.x & 31) return;
   SliceState v;
   v.rho = 0.0;
   v.alpha = 0.0;
   v.beta = 0.0;
-  v.rhs2 = image_parts(part, s, SLOT_RHS, np, C);
+  v.rhs2 = rhs2;
   v.rr = v.rhs2;
   v.rr0 = v.rhs2;
   v.relchg = 0.0;
@@ -1155,7 +1172,7 @@ __global__ void k_state_init(int B, SliceState* st, const double* part, int np, 
 
 void state_init(int batch, cudaStream_t s, SliceState* st, const double* part, int np, const int* counts,
                 int n, const float* lam, const float* lam_tv, float eps, int outer_max, int phase, int channels) {
-  k_state_init<<<(batch + 127) / 128, 128, 0, s>>>(batch, st, part, np, counts, n * n, lam, lam_tv, eps,
+  k_state_init<<<sc_ctas(batch), 32 * SC_WARPS, 0, s>>>(batch, st, part, np, counts, n * n, lam, lam_tv, eps,
                                                    outer_max, phase, channels);
 }
 
@@ -1182,13 +1199,14 @@ void boundary_view(int batch, cudaStream_t s, SliceState* st, SliceState* view) 
 }
 
 __global__ void k_alpha(int B, SliceState* st, const double* part, int np, int C) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = sc_slice();
   if (s >= B || !slice_in_pcg(st, s)) return;
-  pcg_alpha_from(st + s, image_parts(part, s, SLOT_DQ, np, C));
+  const double dq = image_parts(part, s, SLOT_DQ, np, C);
+  if ((threadIdx.x & 31) == 0) pcg_alpha_from(st + s, dq);
 }
 
 void pcg_alpha(int batch, cudaStream_t s, SliceState* st, const double* part, int np, int channels) {
-  k_alpha<<<(batch + 127) / 128, 128, 0, s>>>(batch, st, part, np, channels);
+  k_alpha<<<sc_ctas(batch), 32 * SC_WARPS, 0, s>>>(batch, st, part, np, channels);
 }
 
 // After z = P^{-1} r: rho (first residual, slices at the start of an outer
@@ -1196,12 +1214,13 @@ void pcg_alpha(int batch, cudaStream_t s, SliceState* st, const double* part, in
 // of them for every running slice.
 __global__ void k_pcg_scalars(int B, SliceState* st, const double* part, int np_rz, int np_rr, int mode,
                               PcgSched ps, int C) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = sc_slice();
   if (s >= B || !slice_running(st, s) || st[s].fault) return;
   const int ph = st[s].phase;
   const bool init = mode == SCALARS_INIT || (mode == SCALARS_PER_SLICE && ph == PH_START);
   const bool step = mode == SCALARS_STEP || (mode == SCALARS_PER_SLICE && ph == PH_PCG);
   const double rz = image_parts(part, s, SLOT_RZ, np_rz, C), rr = image_parts(part, s, SLOT_RR, np_rr, C);
+  if (threadIdx.x & 31) return;
   if (init)
     pcg_rho_init_from(st + s, rz, rr);
   else if (step)
@@ -1210,7 +1229,7 @@ __global__ void k_pcg_scalars(int B, SliceState* st, const double* part, int np_
 
 void pcg_scalars(int batch, cudaStream_t s, SliceState* st, const double* part, int np_rz, int np_rr, int mode,
                  const PcgSched& ps, int channels) {
-  k_pcg_scalars<<<(batch + 127) / 128, 128, 0, s>>>(batch, st, part, np_rz, np_rr, mode, ps, channels);
+  k_pcg_scalars<<<sc_ctas(batch), 32 * SC_WARPS, 0, s>>>(batch, st, part, np_rz, np_rr, mode, ps, channels);
 }
 
 // Outer-loop stop.  kind 0: relative change <= tol.  kind 1: estimated
@@ -1229,11 +1248,12 @@ void pcg_scalars(int batch, cudaStream_t s, SliceState* st, const double* part, 
 // slice's FP32 floor, whatever its level.
 __global__ void k_outer_end(int B, SliceState* st, const double* part, int np, float tol, int kind,
                             float stall_tol, int plateau_after, int C) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = sc_slice();
   if (s >= B || !slice_running(st, s) || st[s].phase != PH_END) return;
   SliceState* v = st + s;
   const double dx = image_parts(part, s, SLOT_DX, np, C);
   const double xx = image_parts(part, s, SLOT_XX, np, C);
+  if (threadIdx.x & 31) return;
   const double rel = xx > 0.0 ? sqrt(dx / xx) : INFINITY;
   const int k = v->outer_done;  // this step's index
   const float old = v->hist[k % MU_WINDOW];  // relchg of step k - MU_WINDOW
@@ -1260,7 +1280,7 @@ __global__ void k_outer_end(int B, SliceState* st, const double* part, int np, f
 
 void outer_end(int batch, cudaStream_t s, SliceState* st, const double* part, int np, float tol, int kind,
                float stall_tol, int plateau_after, int channels) {
-  k_outer_end<<<(batch + 127) / 128, 128, 0, s>>>(batch, st, part, np, tol, kind, stall_tol, plateau_after,
+  k_outer_end<<<sc_ctas(batch), 32 * SC_WARPS, 0, s>>>(batch, st, part, np, tol, kind, stall_tol, plateau_after,
                                                   channels);
 }
 
