@@ -36,7 +36,7 @@ constexpr int COUTP[NL] = {32, 32, 32, 32, 32, 16};  // padded output channels
 constexpr int TH = 8, TW = 32;                       // output tile
 constexpr int HH = TH + 2, HW = TW + 2;              // halo tile
 constexpr int CONV_THREADS = 256;
-constexpr int WG_CTAS = 296;                         // weight-gradient partials
+constexpr int WG_CTAS = 304;                         // weight-gradient partials: two CTAs per SM
 
 FI uint32_t ld_u32(const __nv_bfloat16* p) { return *reinterpret_cast<const uint32_t*>(p); }
 
@@ -331,112 +331,134 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3x3_tc(int n, const __nv_
 }
 
 // dW[t][ci][co] = sum_p X[p + off(t)][ci] dZ[p][co]; db[co] = sum_p dZ[p][co].
-// Per-CTA partials over a strided set of tiles: pw [cta][9][CIN][COUT], pb [cta][COUT].
+// Per-CTA partials over a strided set of 8 x 32 tiles: pw [cta][9][CIN][COUT],
+// pb [cta][COUT].  Pixels are the K dimension of mma.m16n8k16, and both operands
+// lie pixel-major in memory: the tiles go to shared memory as they are (16-byte
+// asynchronous copies, the next tile's in flight under this one's products), and
+// ldmatrix.trans turns them.  A warp owns 16 input and 16 output channels and
+// every KS-th group of 16 pixels, for all nine taps: a B fragment serves nine
+// taps, an A fragment two products.  db is a product with ones.  Bound by the
+// shared-memory reads, about one ldmatrix per two products.  Measured, 16 images
+// of 256^2, 32 x 32 channels: 67 us; the form before (element-wise transposed
+// copies, operands packed from single values) took 414.
+constexpr int WG_THREADS = 256;
+
+FI unsigned wg_su32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+FI void ldsm_x4_trans(uint32_t (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+
+template <int CIN, int COUT> struct WgShape {
+  static constexpr int XS = CIN * 2 + 16, ZS = COUT * 2 + 16;  // bytes per pixel: rows of a fragment on distinct banks
+  static constexpr int STAGE = HH * HW * XS + TH * TW * ZS;
+  static constexpr int WM = CIN / 16, WN = COUT / 16, KS = 8 / (WM * WN);
+  static constexpr int SUMS = 9 * CIN * COUT * 4;  // reuses the stages
+  static constexpr int SMEM = 2 * STAGE > SUMS ? 2 * STAGE : SUMS;
+};
+
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(CONV_THREADS) k_wgrad(int n, int batch, const __nv_bfloat16* __restrict__ x,
-                                                        const __nv_bfloat16* __restrict__ dz,
-                                                        float* __restrict__ pw, float* __restrict__ pb) {
-  constexpr int HP = HH * HW + 8;  // transposed halo row stride
-  constexpr int ZP = TH * TW + 8;  // transposed dz row stride
-  constexpr int MT = CIN / 16, NT = COUT / 8, NCOMBO = 9 * MT * NT;
-  constexpr int PER_WARP = (NCOMBO + 7) / 8;
+__global__ void __launch_bounds__(WG_THREADS, 2) k_wgrad(int n, int batch, const __nv_bfloat16* __restrict__ x,
+                                                         const __nv_bfloat16* __restrict__ dz,
+                                                         float* __restrict__ pw, float* __restrict__ pb) {
+  using S = WgShape<CIN, COUT>;
   extern __shared__ __align__(16) unsigned char smem[];
-  __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(smem);  // [CIN][HP]
-  __nv_bfloat16* zs = xs + CIN * HP;                            // [COUT][ZP]
-  float* bsum = reinterpret_cast<float*>(zs + COUT * ZP);       // [COUT]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane >> 2, tg = lane & 3;
-  float acc[PER_WARP][4];
-#pragma unroll
-  for (int i = 0; i < PER_WARP; ++i)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
-  float bacc = 0.f;  // thread co = threadIdx.x < COUT
-  const int tiles_x = n / TW, tiles = tiles_x * (n / TH) * batch;
-  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const int img = tile / (tiles_x * (n / TH)), r = tile % (tiles_x * (n / TH));
-    const int ty0 = (r / tiles_x) * TH, tx0 = (r % tiles_x) * TW;
-    const size_t ibase = (size_t)img * n * n;
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < HH * HW * CIN; idx += blockDim.x) {
-      const int px = idx / CIN, ci = idx % CIN;
-      const int y = ty0 - 1 + px / HW, xx = tx0 - 1 + px % HW;
-      __nv_bfloat16 v = __float2bfloat16(0.f);
-      if (y >= 0 && y < n && xx >= 0 && xx < n) v = x[(ibase + (size_t)y * n + xx) * CIN + ci];
-      xs[ci * HP + px] = v;
-    }
-    for (int idx = threadIdx.x; idx < TH * TW * COUT; idx += blockDim.x) {
-      const int px = idx / COUT, co = idx % COUT;
-      zs[co * ZP + px] = dz[(ibase + (size_t)(ty0 + px / TW) * n + tx0 + px % TW) * COUT + co];
-    }
-    __syncthreads();
-    if (threadIdx.x < COUT) {
-      float s = 0.f;
-      for (int px = 0; px < TH * TW; ++px) s += __bfloat162float(zs[threadIdx.x * ZP + px]);
-      bacc += s;
-    }
-#pragma unroll
-    for (int i = 0; i < PER_WARP; ++i) {
-      const int combo = warp * PER_WARP + i;
-      if (combo >= NCOMBO) break;
-      const int t = combo / (MT * NT), mt = (combo / NT) % MT, nt = combo % NT;
-      const int dy = t / 3, dx = t % 3;
-      for (int kc = 0; kc < TH * TW / 16; ++kc) {
-        const int k0 = kc * 16 + 2 * tg;  // output pixel index (pairs stay in one tile row)
-        const int hp0 = (k0 / TW + dy) * HW + k0 % TW + dx;
-        const int hp1 = ((k0 + 8) / TW + dy) * HW + (k0 + 8) % TW + dx;
-        const __nv_bfloat16* xr0 = xs + (mt * 16 + g) * HP;
-        const __nv_bfloat16* xr1 = xs + (mt * 16 + g + 8) * HP;
-        uint32_t a[4];
-        auto pack = [](__nv_bfloat16 lo, __nv_bfloat16 hi) {
-          return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-        };
-        a[0] = pack(xr0[hp0], xr0[hp0 + 1]);
-        a[1] = pack(xr1[hp0], xr1[hp0 + 1]);
-        a[2] = pack(xr0[hp1], xr0[hp1 + 1]);
-        a[3] = pack(xr1[hp1], xr1[hp1 + 1]);
-        const __nv_bfloat16* zr = zs + (nt * 8 + g) * ZP;
-        const uint32_t b0 = ld_u32(zr + k0), b1 = ld_u32(zr + k0 + 8);
-        mma_bf16(acc[i], a, b0, b1);
+  const int mt = warp % S::WM, nt = warp / S::WM % S::WN, ks = warp / (S::WM * S::WN);
+  const int tiles_x = n / TW, per_img = tiles_x * (n / TH), tiles = per_img * batch;
+  auto fill = [&](int stage, int tile) {
+    if (tile < tiles) {
+      unsigned char* xs = smem + stage * S::STAGE;
+      unsigned char* zs = xs + HH * HW * S::XS;
+      const int img = tile / per_img, r = tile % per_img;
+      const int ty0 = (r / tiles_x) * TH, tx0 = (r % tiles_x) * TW;
+      const size_t ibase = (size_t)img * n * n;
+      for (int i = threadIdx.x; i < HH * HW * (CIN / 8); i += WG_THREADS) {
+        const int px = i / (CIN / 8), ch = i % (CIN / 8);
+        const int yy = ty0 - 1 + px / HW, xx = tx0 - 1 + px % HW;
+        const bool in = yy >= 0 && yy < n && xx >= 0 && xx < n;  // zeros outside the image
+        const __nv_bfloat16* src = x + (in ? (ibase + (size_t)yy * n + xx) * CIN + ch * 8 : 0);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(wg_su32(xs + px * S::XS + ch * 16)),
+                     "l"(src), "r"(in ? 16 : 0)
+                     : "memory");
+      }
+      for (int i = threadIdx.x; i < TH * TW * (COUT / 8); i += WG_THREADS) {
+        const int px = i / (COUT / 8), ch = i % (COUT / 8);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(wg_su32(zs + px * S::ZS + ch * 16)),
+                     "l"(dz + (ibase + (size_t)(ty0 + px / TW) * n + tx0 + px % TW) * COUT + ch * 8)
+                     : "memory");
       }
     }
-  }
-  float* pwc = pw + (size_t)blockIdx.x * 9 * CIN * COUT;
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  float acc[9][2][4], bacc[2][4];
 #pragma unroll
-  for (int i = 0; i < PER_WARP; ++i) {
-    const int combo = warp * PER_WARP + i;
-    if (combo >= NCOMBO) break;
-    const int t = combo / (MT * NT), mt = (combo / NT) % MT, nt = combo % NT;
+  for (int h = 0; h < 2; ++h)
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int ci = mt * 16 + g + 8 * (e >> 1), co = nt * 8 + 2 * tg + (e & 1);
-      pwc[((size_t)t * CIN + ci) * COUT + co] = acc[i][e];
+      bacc[h][e] = 0.f;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) acc[t][h][e] = 0.f;
     }
-  }
-  if (threadIdx.x < COUT) pb[(size_t)blockIdx.x * COUT + threadIdx.x] = bacc;
-  (void)bsum;
-}
-
-template <int CIN, int COUT> constexpr int wgrad_smem() {
-  return (CIN * (HH * HW + 8) + COUT * (TH * TW + 8)) * 2 + COUT * 4;
-}
-
-// Fixed-order sum of the per-CTA partials into the real-size FP32 gradients.
-__global__ void k_wgrad_reduce(int ctas, int cinp, int coutp, int cin, int cout, const float* __restrict__ pw,
-                               const float* __restrict__ pb, float* __restrict__ dw, float* __restrict__ db) {
-  const int total = 9 * cin * cout;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total + cout; i += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    if (i < total) {
-      const int t = i / (cin * cout), ci = (i / cout) % cin, co = i % cout;
-      for (int k = 0; k < ctas; ++k) s += pw[((size_t)k * 9 + t) * cinp * coutp + (size_t)ci * coutp + co];
-      dw[i] = (float)s;
-    } else {
-      const int co = i - total;
-      for (int k = 0; k < ctas; ++k) s += pb[(size_t)k * coutp + co];
-      db[co] = (float)s;
+  // this lane's address in an A fragment: matrices 0 and 1 are pixels 0..7 of
+  // channels 0..7 and 8..15, matrices 2 and 3 the same of pixels 8..15
+  const int fpx = (lane & 7) + ((lane >> 4) & 1) * 8, fch = (lane >> 3) & 1;
+  fill(0, blockIdx.x);
+  int stage = 0;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, stage ^= 1) {
+    fill(stage ^ 1, tile + gridDim.x);
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();
+    const unsigned xb = wg_su32(smem + stage * S::STAGE) + mt * 32 + fch * 16;
+    // B: matrices 0, 1 are pixels 0..7, 8..15 of the first 8 output channels
+    const unsigned zb = wg_su32(smem + stage * S::STAGE + HH * HW * S::XS) + nt * 32 + (lane >> 4) * 16;
+    const int bpx = lane & 15;
+    for (int kc = ks; kc < TH * TW / 16; kc += S::KS) {
+      const int py = kc / (TW / 16), px = kc % (TW / 16) * 16;  // 16 pixels of one tile row
+      uint32_t b[4];
+      ldsm_x4_trans(b, zb + (py * TW + px + bpx) * S::ZS);
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        uint32_t a[4];
+        ldsm_x4_trans(a, xb + ((py + t / 3) * HW + px + t % 3 + fpx) * S::XS);
+        mma_bf16(acc[t][0], a, b[0], b[1]);
+        mma_bf16(acc[t][1], a, b[2], b[3]);
+      }
+      if (mt == 0) {
+        const uint32_t ones[4] = {0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u};
+        mma_bf16(bacc[0], ones, b[0], b[1]);
+        mma_bf16(bacc[1], ones, b[2], b[3]);
+      }
     }
+    __syncthreads();  // the stage may be filled again
   }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+  // the KS pixel groups of each channel block, added in order
+  float* sums = reinterpret_cast<float*>(smem);
+  __shared__ float bsum[COUT];
+  const int g = lane >> 2, tg = lane & 3;
+  for (int k = 0; k < S::KS; ++k) {
+    if (ks == k) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int ci = mt * 16 + g + 8 * (e >> 1), co = nt * 16 + h * 8 + 2 * tg + (e & 1);
+#pragma unroll
+          for (int t = 0; t < 9; ++t) {
+            float* d = sums + (t * CIN + ci) * COUT + co;
+            *d = k == 0 ? acc[t][h][e] : *d + acc[t][h][e];
+          }
+          if (mt == 0 && g == 0 && e < 2) bsum[co] = k == 0 ? bacc[h][e] : bsum[co] + bacc[h][e];
+        }
+    }
+    __syncthreads();
+  }
+  float* pwc = pw + (size_t)blockIdx.x * 9 * CIN * COUT;
+  for (int i = threadIdx.x; i < 9 * CIN * COUT; i += WG_THREADS) pwc[i] = sums[i];
+  if (threadIdx.x < COUT) pb[(size_t)blockIdx.x * COUT + threadIdx.x] = bsum[threadIdx.x];
 }
 
 // NHWC bf16 input [B][n][n][16]: Re A^H b, Im A^H b, mask, zeros.
@@ -478,16 +500,68 @@ __global__ void k_cnn_loss(int total, const float2* __restrict__ x1, const float
   if (threadIdx.x == 0) part[blockIdx.x] = tot;
 }
 
-// Adam (Kingma & Ba) on the FP32 master copy.
-__global__ void k_adam(int count, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// One layer's parameters, gradients and partials, as the update kernel sees them.
+struct CnnLayer {
+  float *w, *mw, *vw, *gw, *b, *mb, *vb, *gb, *bp;
+  __nv_bfloat16 *wf, *wd;
+  const float *pw, *pb;
+  int cin, cout, cinp, coutp, first;  // first: the layer's first CTA
+};
+struct CnnLayers {
+  CnnLayer l[NL];
+};
+
+// The end of a training step for every layer: the gradients (fixed-order FP64
+// sums of the per-CTA partials), Adam (Kingma & Ba) on the FP32 masters and the
+// packed BF16 copies.  A CTA takes 32 parameters, 8 threads each to fetch and
+// add the partials (coalesced over the parameters).  One launch instead of 30,
+// and the sums no longer 296 loads in a row per thread (107 us per layer).
+constexpr int UP_PARAMS = 32, UP_PARTS = 8;
+__global__ void __launch_bounds__(UP_PARAMS* UP_PARTS) k_cnn_update(CnnLayers layers, int ctas, float lr, float b1,
+                                                                    float b2, float eps, float c1, float c2) {
+  __shared__ double red[UP_PARTS][UP_PARAMS];
+  int li = NL - 1;
+  while (li > 0 && (int)blockIdx.x < layers.l[li].first) --li;
+  const CnnLayer& L = layers.l[li];
+  const int nw = 9 * L.cin * L.cout;
+  const int u = threadIdx.x % UP_PARAMS, k = threadIdx.x / UP_PARAMS;
+  const int i = (blockIdx.x - L.first) * UP_PARAMS + u;
+  const int t = i / (L.cin * L.cout), ci = (i / L.cout) % L.cin, co = i % L.cout;
+  double s = 0.0;
+  if (i < nw) {
+    const size_t stride = (size_t)9 * L.cinp * L.coutp;
+    const float* p = L.pw + ((size_t)t * L.cinp + ci) * L.coutp + co;
+#pragma unroll 4
+    for (int c = k; c < ctas; c += UP_PARTS) s += p[c * stride];
+  } else if (i < nw + L.cout) {
+    const float* p = L.pb + (i - nw);
+    for (int c = k; c < ctas; c += UP_PARTS) s += p[(size_t)c * L.coutp];
+  }
+  red[k][u] = s;
+  __syncthreads();
+  if (k != 0 || i >= nw + L.cout) return;
+#pragma unroll
+  for (int c = 1; c < UP_PARTS; ++c) s += red[c][u];
+  const bool weight = i < nw;
+  const int q = weight ? i : i - nw;
+  const float gi = (float)s;
+  (weight ? L.gw : L.gb)[q] = gi;
+  float* m = weight ? L.mw : L.mb;
+  float* v = weight ? L.vw : L.vb;
+  float* p = weight ? L.w : L.b;
+  const float mi = b1 * m[q] + (1.f - b1) * gi;
+  const float vi = b2 * v[q] + (1.f - b2) * gi * gi;
+  m[q] = mi;
+  v[q] = vi;
+  float pi = p[q];
+  pi -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  p[q] = pi;
+  if (weight) {  // the padding of the packed copies stays zero
+    const __nv_bfloat16 h = __float2bfloat16(pi);
+    L.wf[((size_t)t * L.coutp + co) * L.cinp + ci] = h;
+    L.wd[((size_t)(8 - t) * L.cinp + ci) * L.coutp + co] = h;
+  } else {
+    L.bp[q] = pi;
   }
 }
 
@@ -521,7 +595,13 @@ struct firls_cnn {
   __nv_bfloat16 *wf[NL] = {}, *wd[NL] = {};
   __nv_bfloat16* act[NL] = {};  // act[0] input (16 ch), act[l] output of layer l (32 ch)
   __nv_bfloat16 *dza = nullptr, *dzb = nullptr;
-  float *pw = nullptr, *pb = nullptr;
+  // weight-gradient partials of each layer; the FP32 parameters, gradients and
+  // Adam moments of all layers lie in one block each (w, b of layer 0, of layer
+  // 1, ...: `params` floats)
+  float *pw[NL] = {}, *pb[NL] = {};
+  float *pall = nullptr, *gall = nullptr, *mall = nullptr, *vall = nullptr;
+  size_t params = 0;
+  int wg_ctas = 0;
   double* lpart = nullptr;
   int* err = nullptr;  // set by a tcgen05 convolution whose bounded wait ran out
   int adam_t = 0;
@@ -566,11 +646,24 @@ template <int CIN, int COUT> void launch_wgrad(firls_cnn* c, const __nv_bfloat16
   static PerDeviceOnce attr;
   attr.run([] {
     return cudaFuncSetAttribute(k_wgrad<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                wgrad_smem<CIN, COUT>()) == cudaSuccess;
+                                WgShape<CIN, COUT>::SMEM) == cudaSuccess;
   });
-  k_wgrad<CIN, COUT><<<WG_CTAS, CONV_THREADS, wgrad_smem<CIN, COUT>(), c->stream>>>(c->n, c->batch, x, dz, c->pw,
-                                                                                   c->pb);
-  k_wgrad_reduce<<<64, 256, 0, c->stream>>>(WG_CTAS, CIN, COUT, CH[l], CH[l + 1], c->pw, c->pb, c->gw[l], c->gb[l]);
+  k_wgrad<CIN, COUT><<<c->wg_ctas, WG_THREADS, WgShape<CIN, COUT>::SMEM, c->stream>>>(c->n, c->batch, x, dz, c->pw[l],
+                                                                                      c->pb[l]);
+}
+
+// Gradients of every layer from the partials, Adam, packed copies.
+void update(firls_cnn* c, float lr) {
+  CnnLayers layers;
+  int ctas = 0;
+  for (int l = 0; l < NL; ++l) {
+    layers.l[l] = CnnLayer{c->w[l],  c->mw[l], c->vw[l], c->gw[l], c->b[l],  c->mb[l], c->vb[l],  c->gb[l], c->bp[l],
+                           c->wf[l], c->wd[l], c->pw[l], c->pb[l], CH[l],    CH[l + 1], CINP[l], COUTP[l], ctas};
+    ctas += (9 * CH[l] * CH[l + 1] + CH[l + 1] + UP_PARAMS - 1) / UP_PARAMS;
+  }
+  c->adam_t += 1;
+  const float c1 = 1.f - (float)std::pow(0.9, c->adam_t), c2 = 1.f - (float)std::pow(0.999, c->adam_t);
+  k_cnn_update<<<ctas, UP_PARAMS * UP_PARTS, 0, c->stream>>>(layers, c->wg_ctas, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
 }
 
 void pack_all(firls_cnn* c) {
@@ -604,16 +697,13 @@ extern "C" firls_status firls_cnn_create(firls_cnn** out, int n, int batch, void
   auto A = [&](auto** p, size_t cnt) {
     if (s == FIRLS_OK) s = cnn_alloc(c, p, cnt);
   };
+  for (int l = 0; l < NL; ++l) c->params += (9 * (size_t)CH[l] + 1) * CH[l + 1];
+  for (float** v : {&c->pall, &c->gall, &c->mall, &c->vall}) A(v, c->params);
+  const long tiles = (long)(n / TW) * (n / TH) * batch;
+  c->wg_ctas = tiles < WG_CTAS ? (int)tiles : WG_CTAS;
   for (int l = 0; l < NL; ++l) {
-    const size_t nw = 9 * (size_t)CH[l] * CH[l + 1];
-    A(&c->w[l], nw);
-    A(&c->mw[l], nw);
-    A(&c->vw[l], nw);
-    A(&c->gw[l], nw);
-    A(&c->b[l], (size_t)CH[l + 1]);
-    A(&c->mb[l], (size_t)CH[l + 1]);
-    A(&c->vb[l], (size_t)CH[l + 1]);
-    A(&c->gb[l], (size_t)CH[l + 1]);
+    A(&c->pw[l], (size_t)c->wg_ctas * 9 * CINP[l] * COUTP[l]);
+    A(&c->pb[l], (size_t)c->wg_ctas * COUTP[l]);
     A(&c->bp[l], (size_t)COUTP[l]);
     A(&c->wf[l], 9 * (size_t)CINP[l] * COUTP[l]);
     A(&c->wd[l], 9 * (size_t)CINP[l] * COUTP[l]);
@@ -621,8 +711,6 @@ extern "C" firls_status firls_cnn_create(firls_cnn** out, int n, int batch, void
   }
   A(&c->dza, P * 32);
   A(&c->dzb, P * 32);
-  A(&c->pw, (size_t)WG_CTAS * 9 * 32 * 32);
-  A(&c->pb, (size_t)WG_CTAS * 32);
   A(&c->lpart, 1024);
   A(&c->err, 1);
   if (s != FIRLS_OK) {
@@ -630,6 +718,21 @@ extern "C" firls_status firls_cnn_create(firls_cnn** out, int n, int batch, void
     return s;
   }
   cudaMemset(c->err, 0, sizeof(int));
+  cudaMemset(c->gall, 0, c->params * 4);
+  size_t o = 0;
+  for (int l = 0; l < NL; ++l) {
+    const size_t nw = 9 * (size_t)CH[l] * CH[l + 1];
+    c->w[l] = c->pall + o;
+    c->gw[l] = c->gall + o;
+    c->mw[l] = c->mall + o;
+    c->vw[l] = c->vall + o;
+    o += nw;
+    c->b[l] = c->pall + o;
+    c->gb[l] = c->gall + o;
+    c->mb[l] = c->mall + o;
+    c->vb[l] = c->vall + o;
+    o += CH[l + 1];
+  }
   *out = c;
   return FIRLS_OK;
 }
@@ -641,11 +744,9 @@ extern "C" firls_status firls_cnn_set_params(firls_cnn* c, const float* const* w
     if (cudaMemcpyAsync(c->w[l], w[l], nw * 4, cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
         cudaMemcpyAsync(c->b[l], b[l], CH[l + 1] * 4, cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
       return FIRLS_E_CUDA;
-    cudaMemsetAsync(c->mw[l], 0, nw * 4, c->stream);
-    cudaMemsetAsync(c->vw[l], 0, nw * 4, c->stream);
-    cudaMemsetAsync(c->mb[l], 0, CH[l + 1] * 4, c->stream);
-    cudaMemsetAsync(c->vb[l], 0, CH[l + 1] * 4, c->stream);
   }
+  cudaMemsetAsync(c->mall, 0, c->params * 4, c->stream);
+  cudaMemsetAsync(c->vall, 0, c->params * 4, c->stream);
   c->adam_t = 0;
   pack_all(c);
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return FIRLS_E_CUDA;
@@ -653,28 +754,31 @@ extern "C" firls_status firls_cnn_set_params(firls_cnn* c, const float* const* w
   return FIRLS_OK;
 }
 
-extern "C" firls_status firls_cnn_get_params(firls_cnn* c, float* const* w, float* const* b) {
-  if (!c || !w || !b) return FIRLS_E_INVALID_ARG;
+// One copy of the whole block, then each layer's part on the host.
+static firls_status get_block(firls_cnn* c, const float* block, float* const* w, float* const* b) {
+  std::vector<float> h(c->params);
+  if (cudaMemcpyAsync(h.data(), block, c->params * 4, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
+      cudaStreamSynchronize(c->stream) != cudaSuccess)
+    return FIRLS_E_CUDA;
+  const float* p = h.data();
   for (int l = 0; l < NL; ++l) {
     const size_t nw = 9 * (size_t)CH[l] * CH[l + 1];
-    if (w[l] && cudaMemcpyAsync(w[l], c->w[l], nw * 4, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
-      return FIRLS_E_CUDA;
-    if (b[l] && cudaMemcpyAsync(b[l], c->b[l], CH[l + 1] * 4, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
-      return FIRLS_E_CUDA;
+    if (w[l]) std::memcpy(w[l], p, nw * 4);
+    p += nw;
+    if (b[l]) std::memcpy(b[l], p, CH[l + 1] * 4);
+    p += CH[l + 1];
   }
-  return cudaStreamSynchronize(c->stream) == cudaSuccess ? FIRLS_OK : FIRLS_E_CUDA;
+  return FIRLS_OK;
+}
+
+extern "C" firls_status firls_cnn_get_params(firls_cnn* c, float* const* w, float* const* b) {
+  if (!c || !w || !b) return FIRLS_E_INVALID_ARG;
+  return get_block(c, c->pall, w, b);
 }
 
 extern "C" firls_status firls_cnn_get_grads(firls_cnn* c, float* const* gw, float* const* gb) {
   if (!c || !gw || !gb) return FIRLS_E_INVALID_ARG;
-  for (int l = 0; l < NL; ++l) {
-    const size_t nw = 9 * (size_t)CH[l] * CH[l + 1];
-    if (gw[l] && cudaMemcpyAsync(gw[l], c->gw[l], nw * 4, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
-      return FIRLS_E_CUDA;
-    if (gb[l] && cudaMemcpyAsync(gb[l], c->gb[l], CH[l + 1] * 4, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
-      return FIRLS_E_CUDA;
-  }
-  return cudaStreamSynchronize(c->stream) == cudaSuccess ? FIRLS_OK : FIRLS_E_CUDA;
+  return get_block(c, c->gall, gw, gb);
 }
 
 extern "C" firls_status firls_cnn_forward(firls_cnn* c, const void* atb, const uint8_t* mask, void* x1) {
@@ -706,16 +810,7 @@ extern "C" firls_status firls_cnn_train_step(firls_cnn* c, const void* atb, cons
     nxt = t;
   }
   launch_wgrad<16, 32>(c, c->act[0], cur, 0);
-  // Adam
-  c->adam_t += 1;
-  const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = 1.f - (float)std::pow(0.9, c->adam_t), c2 = 1.f - (float)std::pow(0.999, c->adam_t);
-  for (int l = 0; l < NL; ++l) {
-    const int nw = 9 * CH[l] * CH[l + 1];
-    k_adam<<<64, 256, 0, c->stream>>>(nw, c->w[l], c->gw[l], c->mw[l], c->vw[l], lr, b1, b2, 1e-8f, c1, c2);
-    k_adam<<<1, 64, 0, c->stream>>>(CH[l + 1], c->b[l], c->gb[l], c->mb[l], c->vb[l], lr, b1, b2, 1e-8f, c1, c2);
-  }
-  pack_all(c);
+  update(c, lr);
   if (loss) {
     std::vector<double> h(lblocks);
     if (cudaMemcpyAsync(h.data(), c->lpart, sizeof(double) * lblocks, cudaMemcpyDeviceToHost, c->stream) !=
