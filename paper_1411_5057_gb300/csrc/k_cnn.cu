@@ -154,40 +154,71 @@ __global__ void __launch_bounds__(CONV_THREADS) k_conv3x3(int n, const __nv_bflo
 template <int CIN, int COUT> constexpr int conv_smem() { return (HH * HW * (CIN + 8) + 9 * COUT * (CIN + 8)) * 2; }
 
 // ---- the same convolution on the 5th-generation tensor cores (tcgen05) ----
-// A CTA computes TC_R image rows x TC_W pixels.  Per output row r the GEMM
+// Tiles of TC_R image rows x TC_W pixels.  Per output row r the GEMM
 // D_r[pixel][co] = sum_tap sum_ci X[row r + dy][pixel + dx][ci] W[tap][co][ci]
 // runs as 9 * CIN/16 tcgen05.mma (M = 128 pixels, N = COUT, K = 16) with its
 // FP32 accumulator in TMEM (columns 32 r ..).  Operands sit in shared memory
 // in the canonical K-major layout without swizzle: 8-channel planes of
 // 16-byte pixel (or weight-row) records, so the A operand of tap (dy, dx) is
 // the halo row r + dy starting at pixel dx: core matrices 128 bytes apart
-// along M (SBO), planes one plane apart along K (LBO).  One thread issues the
-// MMAs and commits them to an mbarrier; after the (bounded) wait each warp
-// reads its 32 pixel lanes with tcgen05.ld and runs the epilogue.
+// along M (SBO), planes one plane apart along K (LBO).
+//
+// One persistent CTA per SM walks the tiles with the weights resident, its
+// warps in three roles, so that a tile's copies, the next one's products and
+// the one's before it results run at the same time:
+//   warps 5-8   fill a ring of TC_STAGES tiles (asynchronous 16-byte copies),
+//   warp 4     one thread issues a tile's MMAs into one of TC_BUFS TMEM buffers,
+//   warps 0-3  read a finished buffer (tcgen05.ld), apply bias and ReLU, the last
+//              layer's correction or the ReLU gate (both fetched before the
+//              products are done), and store: a warp's 32 pixels of a row are
+//              2 KB in a row of the image, staged in shared memory and sent as
+//              one bulk copy (16-byte stores 64 bytes apart write every sector
+//              twice and took longer than the products).
+// Handover by mbarriers, every wait bounded.  A CTA per tile that filled,
+// multiplied and stored in series took 258 us for 32 x 32 channels at 64 images of
+// 256^2 (three CTAs per SM; the weights fetched for each tile); this takes 139 us
+// (537 MB read and written: 3.9 TB/s; 168 us with 16-byte stores from registers),
+// 16 x 32: 169 -> 127 us, 32 x 16 with the correction: 191 -> 105 us, and at 16
+// images 70 -> 41 us (hidden), 80 -> 55 us (gated).  What is left is the chain of
+// a tile's four epilogue rows per warp: TMEM read, conversion, staging.
 constexpr int TC_W = 128, TC_R = 4, TC_HW = TC_W + 2, TC_HR = TC_R + 2;
-constexpr int TC_THREADS = 128;
+constexpr int TC_STAGES = 3, TC_PRODUCERS = 128, TC_THREADS = 128 + 32 + TC_PRODUCERS;
+constexpr int TC_BUFS = 4, TC_TMEM = TC_BUFS * TC_R * 32;  // columns
 
 FI unsigned cnn_su32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
 // tcgen05 shared-memory matrix descriptor: start, leading (K) and stride (M/N)
-// byte offsets, fixed version bits 46-48 = 1, no swizzle.
-FI uint64_t umma_desc(const void* p, unsigned lbo, unsigned sbo) {
-  uint64_t d = (uint64_t)((cnn_su32(p) & 0x3FFFF) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
+// byte offsets, fixed version bits 46-48 = 1, no swizzle.  Its low word is the
+// start / 16 plus the leading offset, so a shifted operand is an addition to it.
+FI uint32_t umma_lo(unsigned addr, unsigned lbo) { return ((addr & 0x3FFFF) >> 4) | ((lbo >> 4) << 16); }
+__host__ __device__ constexpr uint32_t umma_hi(unsigned sbo) { return (sbo >> 4) | (1u << 14); }
+
+FI void cnn_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(cnn_su32(bar)) : "memory");
+}
+// Bounded wait (about a second) for the phase of that parity; every wait of a
+// CTA whose waits have run out once gives up after one poll.
+FI bool cnn_wait(uint64_t* bar, unsigned parity, const volatile int* abort_flag) {
+  for (int it = 0; it < 10000; ++it) {
+    unsigned ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok)
+                 : "r"(cnn_su32(bar)), "r"(parity), "r"(100000u)
+                 : "memory");
+    if (ok) return true;
+    if (*abort_flag) return false;
+  }
+  return false;
 }
 
-// Operand bytes, but at least 64 KB so that at most 3 CTAs share an SM and
-// their 3 x 128 TMEM columns fit the SM's 512.
+template <int CIN> constexpr int tc_stage_bytes() { return TC_HR * TC_HW * CIN * 2; }
+template <int COUT> __host__ __device__ constexpr int tc_row_bytes() { return 32 * COUT * 2; }  // of a warp
 template <int CIN, int COUT> constexpr int tc_smem() {
-  return TC_HR * TC_HW * CIN * 2 + 9 * COUT * CIN * 2 > 64 * 1024 ? TC_HR * TC_HW * CIN * 2 + 9 * COUT * CIN * 2
-                                                                   : 64 * 1024;
+  return TC_STAGES * tc_stage_bytes<CIN>() + 9 * COUT * CIN * 2 + 4 * 2 * tc_row_bytes<COUT>();
 }
 
 template <int CIN, int COUT, int MODE>
-__global__ void __launch_bounds__(TC_THREADS, 1) k_conv3x3_tc(int n, const __nv_bfloat16* __restrict__ in,
+__global__ void __launch_bounds__(TC_THREADS, 1) k_conv3x3_tc(int n, int tiles, const __nv_bfloat16* __restrict__ in,
                                                               const __nv_bfloat16* __restrict__ wt,
                                                               const float* __restrict__ bias,
                                                               __nv_bfloat16* __restrict__ out,
@@ -197,137 +228,255 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3x3_tc(int n, const __nv_
   constexpr int KP = CIN / 8;                  // 8-channel planes
   constexpr int XPL = TC_HR * TC_HW * 16;      // bytes per activation plane
   constexpr int WPL = COUT * 16;               // bytes per weight plane
+  constexpr int STAGE = TC_HR * TC_HW * CIN * 2;
   static_assert(COUT % 16 == 0 && COUT <= 32 && CIN % 16 == 0, "tcgen05 conv shape");
   extern __shared__ __align__(128) unsigned char smem[];
-  unsigned char* xs = smem;                    // [KP][TC_HR * TC_HW pixels][16 B]
-  unsigned char* wsm = smem + KP * XPL;        // [9][KP][COUT][16 B]
+  unsigned char* wsm = smem + TC_STAGES * STAGE;  // [9][KP][COUT][16 B]
   __shared__ uint32_t tmem_base;
-  __shared__ __align__(8) uint64_t bar;
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int segs = n / TC_W;
-  const int y0 = (blockIdx.x / segs) * TC_R, x0 = (blockIdx.x % segs) * TC_W;
-  const int img = blockIdx.y;
-  const size_t ibase = (size_t)img * n * n;
-  // halo rows y0-1 .. y0+TC_R, pixels x0-1 .. x0+TC_W (zero outside the
-  // image) and the weights: asynchronous 16-byte copies, all in flight at once
-  for (int idx = t; idx < TC_HR * TC_HW * KP; idx += TC_THREADS) {
-    const int px = idx / KP, ch = idx % KP;
-    const int y = y0 - 1 + px / TC_HW, x = x0 - 1 + px % TC_HW;
-    unsigned char* dst = xs + (size_t)ch * XPL + px * 16;
-    if (y >= 0 && y < n && x >= 0 && x < n)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(cnn_su32(dst)),
-                   "l"(reinterpret_cast<const uint4*>(in + (ibase + (size_t)y * n + x) * CIN) + ch)
-                   : "memory");
-    else
-      *reinterpret_cast<uint4*>(dst) = make_uint4(0, 0, 0, 0);
-  }
+  // full: a stage has landed; empty: its MMAs are done; ready: a TMEM buffer
+  // holds a tile; drained: it has been read
+  __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], ready[TC_BUFS], drained[TC_BUFS];
+  __shared__ volatile int abort_flag;
+  const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t >> 5, 0), lane = t & 31;
+  const int segs = n / TC_W, per_img = segs * (n / TC_R);
+  const int count = ((int)blockIdx.x < tiles) ? (tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  // the tile's image, first row and first pixel
+  auto where = [&](int i, int& img, int& y0, int& x0) {
+    const int tile = blockIdx.x + i * gridDim.x, r = tile % per_img;
+    img = tile / per_img;
+    y0 = r / segs * TC_R;
+    x0 = r % segs * TC_W;
+  };
   for (int idx = t; idx < 9 * COUT * KP; idx += TC_THREADS) {
     const int row = idx / KP, ch = idx % KP;  // row = tap * COUT + co
     const int tap = row / COUT, co = row % COUT;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
-                     cnn_su32(wsm + ((size_t)(tap * KP + ch) * COUT + co) * 16)),
-                 "l"(reinterpret_cast<const uint4*>(wt + (size_t)row * CIN) + ch)
-                 : "memory");
+    *reinterpret_cast<uint4*>(wsm + ((size_t)(tap * KP + ch) * COUT + co) * 16) =
+        reinterpret_cast<const uint4*>(wt + (size_t)row * CIN)[ch];
   }
-  asm volatile("cp.async.commit_group;\n cp.async.wait_all;\n" ::: "memory");
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // generic writes -> tensor core reads
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(cnn_su32(&tmem_base)),
-                 "r"(TC_R * 32)
+                 "r"(TC_TMEM)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
   }
-  if (t == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(cnn_su32(&bar)) : "memory");
+  if (t == 0) {
+    auto init = [](uint64_t* b, unsigned c) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(cnn_su32(b)), "r"(c) : "memory");
+    };
+    for (int i = 0; i < TC_STAGES; ++i) {
+      init(full + i, TC_PRODUCERS);
+      init(empty + i, 1);
+    }
+    for (int i = 0; i < TC_BUFS; ++i) {
+      init(ready + i, 1);
+      init(drained + i, 128);
+    }
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = tmem_base;
-  // D f32, A and B bf16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-  constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(COUT >> 3) << 17) | ((uint32_t)(TC_W >> 4) << 24);
-  if (t == 0) {
-    for (int r = 0; r < TC_R; ++r) {
-      const uint32_t d = tmem + (uint32_t)(r * 32);
-      int k = 0;
-      for (int tap = 0; tap < 9; ++tap) {
-        const int dy = tap / 3, dx = tap % 3;
-        for (int kk = 0; kk < CIN / 16; ++kk, ++k) {
-          const uint64_t ad = umma_desc(xs + (size_t)(2 * kk) * XPL + ((r + dy) * TC_HW + dx) * 16, XPL, 128);
-          const uint64_t bd = umma_desc(wsm + (size_t)(tap * KP + 2 * kk) * WPL, WPL, 128);
-          asm volatile(
-              "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-              "l"(ad), "l"(bd), "r"(idesc), "r"(k > 0 ? 1u : 0u)
-              : "memory");
+  bool ok = true;
+
+  if (warp > 4) {
+    // ============================================================ producers
+    const int pt = t - 160;
+    // halo rows y0-1 .. y0+TC_R, pixels x0-1 .. x0+TC_W, zero outside the image.
+    // A thread copies one 8-channel plane of every (TC_PRODUCERS / KP)-th pixel
+    // and steps its coordinates from one to the next.
+    constexpr int STEP = TC_PRODUCERS / KP;
+    static_assert(STEP < TC_HW, "one row crossed per step");
+    const int ch = pt % KP, px0 = pt / KP;
+    auto fill = [&](int i) {
+      int img, y0, x0;
+      where(i, img, y0, x0);
+      unsigned dst = cnn_su32(smem + (i % TC_STAGES) * STAGE + ch * XPL + px0 * 16);
+      const __nv_bfloat16* src = in + (size_t)img * n * n * CIN + ch * 8;
+      int x = x0 - 1 + px0, y = y0 - 1;
+      const int xe = x0 - 1 + TC_HW;
+#pragma unroll 4
+      for (int px = px0; px < TC_HR * TC_HW; px += STEP) {
+        const bool inside = (unsigned)y < (unsigned)n && (unsigned)x < (unsigned)n;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst),
+                     "l"(src + (inside ? (y * n + x) * CIN : 0)), "r"(inside ? 16 : 0)
+                     : "memory");
+        dst += STEP * 16;
+        x += STEP;
+        if (x >= xe) {
+          x -= TC_HW;
+          ++y;
         }
       }
-    }
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(cnn_su32(&bar))
-                 : "memory");
-  }
-  bool done = false;
-  for (int it = 0; it < 10000 && !done; ++it) {  // bounded (about a second): the MMAs take microseconds
-    unsigned ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0, %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(ok)
-                 : "r"(cnn_su32(&bar)), "r"(100000u)
-                 : "memory");
-    done = ok != 0;
-  }
-  done = __all_sync(0xffffffffu, done);
-  if (!done && lane == 0) atomicExch(err, 1);
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  if (done) {
-    for (int r = 0; r < TC_R; ++r) {
-      uint32_t v[32];
-      const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(r * 32);
-      if (COUT == 32) {
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
-            "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-              "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-              "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-            : "r"(ta));
-      } else {
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-            : "r"(ta));
+    };
+    // tile i - 1 is handed over once its copies have landed, tile i's in flight
+    for (int i = 0; i <= count && ok; ++i) {
+      if (i < count) {
+        if (i >= TC_STAGES) ok = cnn_wait(empty + i % TC_STAGES, (i / TC_STAGES - 1) & 1, &abort_flag);
+        if (ok) fill(i);
       }
-      asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-      // this thread's pixel: row y0 + r, column x0 + 32 warp + lane
-      const size_t p = ibase + (size_t)(y0 + r) * n + x0 + warp * 32 + lane;
-      if (MODE == MODE_LAST) {
-        const float2 ab = atb[p];
-        x1[p] = make_float2(ab.x + __uint_as_float(v[0]) + bias[0], ab.y + __uint_as_float(v[1]) + bias[1]);
-      } else {
-        uint32_t pk[COUT / 2];
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+      if (i > 0) {
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        cnn_arrive(full + (i - 1) % TC_STAGES);
+      }
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+  } else if (warp == 4) {
+    // ============================================================== products
+    // D f32, A and B bf16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24
+    constexpr uint32_t idesc =
+        (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(COUT >> 3) << 17) | ((uint32_t)(TC_W >> 4) << 24);
+    // The whole warp runs the loop, so that the descriptors are computed in the
+    // uniform datapath, and one elected thread issues: computed by one diverged
+    // thread, they took longer than the products.
+    uint32_t leader;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(leader));
+    const uint32_t bl = umma_lo(cnn_su32(wsm), WPL);
+    for (int i = 0; i < count; ++i) {
+      const int buf = i % TC_BUFS;
+      ok = cnn_wait(full + i % TC_STAGES, (i / TC_STAGES) & 1, &abort_flag);
+      if (ok && i >= TC_BUFS) ok = cnn_wait(drained + buf, (i / TC_BUFS - 1) & 1, &abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      const uint32_t al = umma_lo(cnn_su32(smem + (i % TC_STAGES) * STAGE), XPL);
+      const uint32_t d0 = tmem + (uint32_t)(buf * TC_R * 32);
 #pragma unroll
-        for (int j = 0; j < COUT / 2; ++j) {
-          float a = __uint_as_float(v[2 * j]), b = __uint_as_float(v[2 * j + 1]);
-          if (MODE == MODE_HIDDEN) {
-            a = fmaxf(a + bias[2 * j], 0.f);
-            b = fmaxf(b + bias[2 * j + 1], 0.f);
-          } else {
-            const __nv_bfloat162 gt = *reinterpret_cast<const __nv_bfloat162*>(gate + p * COUT + 2 * j);
-            if (!(__bfloat162float(gt.x) > 0.f)) a = 0.f;
-            if (!(__bfloat162float(gt.y) > 0.f)) b = 0.f;
+      for (int r = 0; r < TC_R; ++r) {
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+          const int dy = tap / 3, dx = tap % 3;
+#pragma unroll
+          for (int kk = 0; kk < CIN / 16; ++kk) {
+            asm volatile(
+                "{\n .reg .pred p, q;\n .reg .b64 a, b;\n setp.ne.u32 p, %5, 0;\n setp.ne.u32 q, %6, 0;\n"
+                " mov.b64 a, {%1, %3};\n mov.b64 b, {%2, %4};\n"
+                " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %7, p;\n}\n" ::"r"(d0 + r * 32),
+                "r"(al + (uint32_t)(2 * kk * XPL + ((r + dy) * TC_HW + dx) * 16) / 16),
+                "r"(bl + (uint32_t)((tap * KP + 2 * kk) * WPL) / 16), "r"(umma_hi(128)), "r"(umma_hi(128)),
+                "r"(tap + kk > 0 ? 1u : 0u), "r"(leader), "r"(idesc)
+                : "memory");
           }
-          const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-          pk[j] = *reinterpret_cast<const uint32_t*>(&h);
         }
-        uint4* o = reinterpret_cast<uint4*>(out + p * COUT);
+      }
+      auto commit = [&](uint64_t* b) {
+        asm volatile(
+            "{\n .reg .pred q;\n setp.ne.u32 q, %1, 0;\n"
+            " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(cnn_su32(b)),
+            "r"(leader)
+            : "memory");
+      };
+      commit(empty + i % TC_STAGES);
+      commit(ready + buf);
+    }
+  } else {
+    // =============================================================== results
+    unsigned char* stage_out = wsm + 9 * COUT * CIN * 2 + warp * 2 * tc_row_bytes<COUT>();
+    float bv[COUT];
+    if (MODE == MODE_HIDDEN) {
 #pragma unroll
-        for (int q = 0; q < COUT / 8; ++q) o[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+      for (int j = 0; j < COUT; ++j) bv[j] = bias[j];
+    }
+    for (int i = 0; i < count; ++i) {
+      int img, y0, x0;
+      where(i, img, y0, x0);
+      const int buf = i % TC_BUFS;
+      // this thread's pixel: row y0 + r, column x0 + 32 warp + lane
+      const size_t p0 = (size_t)img * n * n + (size_t)y0 * n + x0 + warp * 32 + lane;
+      uint4 gt[TC_R][COUT / 8];
+      float2 ab[TC_R];
+#pragma unroll
+      for (int r = 0; r < TC_R; ++r) {
+        if (MODE == MODE_DGRAD) {
+#pragma unroll
+          for (int q = 0; q < COUT / 8; ++q)
+            gt[r][q] = reinterpret_cast<const uint4*>(gate + (p0 + (size_t)r * n) * COUT)[q];
+        }
+        if (MODE == MODE_LAST) ab[r] = atb[p0 + (size_t)r * n];
+      }
+      ok = __all_sync(0xffffffffu, cnn_wait(ready + buf, (i / TC_BUFS) & 1, &abort_flag));
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+#pragma unroll
+      for (int r = 0; r < TC_R; ++r) {
+        const size_t p = p0 + (size_t)r * n;
+        uint32_t v[32];
+        const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(buf * TC_R * 32 + r * 32);
+        if (COUT == 32) {
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,"
+              "%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+                "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
+                "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
+                "=r"(v[30]), "=r"(v[31])
+              : "r"(ta));
+        } else {
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+              : "r"(ta));
+        }
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        if (r + 1 == TC_R) {  // the buffer has been read
+          asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+          cnn_arrive(drained + buf);
+        }
+        if (MODE == MODE_LAST) {
+          x1[p] = make_float2(ab[r].x + __uint_as_float(v[0]) + bias[0], ab[r].y + __uint_as_float(v[1]) + bias[1]);
+        } else {
+          uint32_t pk[COUT / 2];
+#pragma unroll
+          for (int j = 0; j < COUT / 2; ++j) {
+            float a = __uint_as_float(v[2 * j]), b = __uint_as_float(v[2 * j + 1]);
+            if (MODE == MODE_HIDDEN) {
+              a = fmaxf(a + bv[2 * j], 0.f);
+              b = fmaxf(b + bv[2 * j + 1], 0.f);
+            } else {  // the gate's BF16 values as FP32
+              const uint4 g4 = gt[r][j / 4];
+              const uint32_t gw = j % 4 == 0 ? g4.x : j % 4 == 1 ? g4.y : j % 4 == 2 ? g4.z : g4.w;
+              if (!(__uint_as_float(gw << 16) > 0.f)) a = 0.f;
+              if (!(__uint_as_float(gw & 0xffff0000u) > 0.f)) b = 0.f;
+            }
+            const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+            pk[j] = *reinterpret_cast<const uint32_t*>(&h);
+          }
+          // two staging rows per warp: the copy of the row before last has left
+          // this one
+          unsigned char* row = stage_out + (r & 1) * tc_row_bytes<COUT>();
+          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory");
+          __syncwarp();
+          uint4* o = reinterpret_cast<uint4*>(row + lane * COUT * 2);
+#pragma unroll
+          for (int q = 0; q < COUT / 8; ++q) o[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+          __syncwarp();
+          if (lane == 0) {
+            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n cp.async.bulk.commit_group;\n" ::"l"(
+                             out + p * COUT),
+                         "r"(cnn_su32(row)), "r"(tc_row_bytes<COUT>())
+                         : "memory");
+          }
+        }
       }
     }
+  }
+  if (warp < 4 && MODE != MODE_LAST && lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+  if (!ok) {
+    abort_flag = 1;
+    if (lane == 0) atomicExch(err, 1);
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TC_R * 32) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TC_TMEM) : "memory");
 }
 
 // dW[t][ci][co] = sum_p X[p + off(t)][ci] dZ[p][co]; db[co] = sum_p dZ[p][co].
@@ -602,6 +751,7 @@ struct firls_cnn {
   float *pall = nullptr, *gall = nullptr, *mall = nullptr, *vall = nullptr;
   size_t params = 0;
   int wg_ctas = 0;
+  int sms = 152;
   double* lpart = nullptr;
   int* err = nullptr;  // set by a tcgen05 convolution whose bounded wait ran out
   int adam_t = 0;
@@ -627,9 +777,10 @@ template <int CIN, int COUT, int MODE> void launch_conv(firls_cnn* c, const __nv
       return cudaFuncSetAttribute(k_conv3x3_tc<CIN, COUT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   tc_smem<CIN, COUT>()) == cudaSuccess;
     });
-    const dim3 grid((c->n / TC_W) * (c->n / TC_R), c->batch);
-    k_conv3x3_tc<CIN, COUT, MODE><<<grid, TC_THREADS, tc_smem<CIN, COUT>(), c->stream>>>(c->n, in, wt, bias, out, gate,
-                                                                                          atb, x1, c->err);
+    const int tiles = (c->n / TC_W) * (c->n / TC_R) * c->batch;
+    const int grid = tiles < c->sms ? tiles : c->sms;
+    k_conv3x3_tc<CIN, COUT, MODE><<<grid, TC_THREADS, tc_smem<CIN, COUT>(), c->stream>>>(c->n, tiles, in, wt, bias, out,
+                                                                                          gate, atb, x1, c->err);
     return;
   }
   static PerDeviceOnce attr;
@@ -692,6 +843,8 @@ extern "C" firls_status firls_cnn_create(firls_cnn** out, int n, int batch, void
   c->n = n;
   c->batch = batch;
   c->stream = static_cast<cudaStream_t>(cuda_stream);
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t P = (size_t)batch * n * n;
   firls_status s = FIRLS_OK;
   auto A = [&](auto** p, size_t cnt) {
