@@ -25,7 +25,7 @@ using namespace firls;
 namespace {
 
 constexpr int RT = 256;   // threads of the row kernel
-constexpr int PT = 1024;  // threads of the per-problem PCG kernel
+constexpr int PT = 1024;  // threads of the per-problem set-up kernel
 
 // Which problems a row pass serves and what it multiplies.
 enum DenseRows {
@@ -202,110 +202,284 @@ __global__ void __launch_bounds__(PT) k_dense_setup(int N, int CH, const float* 
 
 enum DensePcg { DP_INIT = 0, DP_STEP = 1 };
 
-// One PCG step of problem p (or the start of its outer step), on its whole
-// vectors; ends the outer step in place when its PCG stops.
-__global__ void __launch_bounds__(PT) k_dense_pcg(int N, int CH, int mode, SliceState* __restrict__ st,
-                                                  const float* __restrict__ qpart, float* __restrict__ x,
-                                                  float* __restrict__ dx, float* __restrict__ r,
-                                                  float* __restrict__ z, float* __restrict__ d,
-                                                  float* __restrict__ q, float* __restrict__ w,
-                                                  float* __restrict__ pinv, const float* __restrict__ atb,
-                                                  const float* __restrict__ dAtA, int shared, int precond,
-                                                  PcgSched ps, float outer_tol) {
-  const int p = blockIdx.x;
-  if (!slice_running(st, p)) return;
-  const int ph = st[p].phase;
-  if (ph != (mode == DP_INIT ? PH_BOUNDARY : PH_PCG)) return;
-  __shared__ double red[32];
-  __shared__ double bc;
+constexpr int QT = 512;  // threads of the PCG kernel
+
+// Inner products of a problem's vectors.  The device has 2 FP64 lanes per
+// clock and SM: converting and accumulating 4000 products in FP64 took most of
+// the PCG kernel.  A product of two floats is exactly p + e with
+// e = fma(a, b, -p), and a sum carried in three floats loses less than an FP64
+// one (each two_sum is exact, the third float takes the remainders), so only
+// the final value is FP64.  Floats have less range than doubles: a result
+// outside [SUM_LO, SUM_HI] (or NaN) is formed again in FP64, so tiny and huge
+// problems give what they gave.  Inside, the low halves lost to underflow are
+// at most N 2^-149 < 2e-41, 2e-16 of SUM_LO.
+constexpr double SUM_LO = 1e-25, SUM_HI = 1e30;
+
+FI void two_sum(float a, float b, float& s, float& e) {
+  const float t = a + b, bb = t - a;
+  e = (a - (t - bb)) + (b - bb);
+  s = t;
+}
+
+struct Sum3 {
+  float s, c, cc;  // value s + c + cc
+  FI void add(float v, float lo) {  // v + lo, |lo| <= ulp(v)
+    float e, f;
+    two_sum(s, v, s, e);
+    two_sum(c, lo, c, f);
+    cc += f;
+    two_sum(c, e, c, f);
+    cc += f;
+  }
+  FI void add_product(float a, float b) {
+    const float p = a * b;
+    add(p, fmaf(a, b, -p));
+  }
+  FI void add(const Sum3& o) {
+    add(o.s, o.c);
+    cc += o.cc;
+  }
+  FI Sum3 from_lane(int o) const {
+    return {__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o),
+            __shfl_xor_sync(0xffffffffu, cc, o)};
+  }
+};
+
+struct DotRed {
+  Sum3 part[2][QT / 32];
+  double wide[32];
+  int again;
+};
+
+// a_0 . b_0 and a_1 . b_1 over the block's vectors; `use` runs in thread 0 with
+// both values, and every thread sees what it wrote to shared memory.
+template <int V, typename Use>
+FI void dots(DotRed& red, const float4 (&a0)[V], const float4 (&b0)[V], const float4 (&a1)[V], const float4 (&b1)[V],
+             bool two, Use&& use) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  Sum3 u{0.f, 0.f, 0.f}, v{0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    u.add_product(a0[k].x, b0[k].x);
+    u.add_product(a0[k].y, b0[k].y);
+    u.add_product(a0[k].z, b0[k].z);
+    u.add_product(a0[k].w, b0[k].w);
+    if (two) {
+      v.add_product(a1[k].x, b1[k].x);
+      v.add_product(a1[k].y, b1[k].y);
+      v.add_product(a1[k].z, b1[k].z);
+      v.add_product(a1[k].w, b1[k].w);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    u.add(u.from_lane(o));
+    if (two) v.add(v.from_lane(o));
+  }
+  if (lane == 0) {
+    red.part[0][warp] = u;
+    if (two) red.part[1][warp] = v;
+  }
+  __syncthreads();
+  if (warp == 0) {  // lanes 0-15 the first sum, 16-31 the second
+    static_assert(QT / 32 == 16, "half a warp per sum");
+    Sum3 t{0.f, 0.f, 0.f};
+    if (two || lane < 16) t = red.part[lane >> 4][lane & 15];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t.add(t.from_lane(o));
+    const double mine = (double)t.s + ((double)t.c + (double)t.cc);
+    const double other = __shfl_xor_sync(0xffffffffu, mine, 16);
+    if (lane == 0) {
+      const bool ok = fabs(mine) > SUM_LO && fabs(mine) < SUM_HI && (!two || (fabs(other) > SUM_LO && fabs(other) < SUM_HI));
+      red.again = !ok;
+      if (ok) use(mine, other);
+    }
+  }
+  __syncthreads();
+  if (!red.again) return;
+  double du = 0.0, dv = 0.0;
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    du += (double)a0[k].x * b0[k].x + (double)a0[k].y * b0[k].y + (double)a0[k].z * b0[k].z + (double)a0[k].w * b0[k].w;
+    if (two)
+      dv += (double)a1[k].x * b1[k].x + (double)a1[k].y * b1[k].y + (double)a1[k].z * b1[k].z + (double)a1[k].w * b1[k].w;
+  }
+  du = block_sum(du, red.wide);
+  if (two) dv = block_sum(dv, red.wide);
+  if (threadIdx.x == 0) use(du, dv);
+  __syncthreads();
+}
+
+FI float4 f4zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+
+// One PCG step of problem p (or the start of its outer step); ends the outer
+// step in place when its PCG stops.  A thread keeps its V float4 of every
+// vector in registers from the load to the store, all loads are issued before
+// the first reduction, and z = P^{-1} r and q = S d exist only there.
+// 4000 unknowns: 256 problems 52 -> 16 us, 152 problems
+// 28 -> 14 us a step (scalar passes over memory with FP64 sums
+// before).  V = 2 (N <= 4096) leaves room for two CTAs per SM, so 304 problems
+// run at once.
+template <int V>
+__global__ void __launch_bounds__(QT, V <= 2 ? 2 : 1)
+    k_dense_pcg(int N, int CH, int mode, SliceState* __restrict__ st, const float* __restrict__ qpart,
+                float* __restrict__ x, float* __restrict__ dx, float* __restrict__ r, float* __restrict__ d,
+                float* __restrict__ w, float* __restrict__ pinv, const float* __restrict__ atb,
+                const float* __restrict__ dAtA, int shared, int precond, PcgSched ps, float outer_tol) {
+  const int p = blockIdx.x, t = threadIdx.x;
+  __shared__ SliceState sv;
+  __shared__ DotRed red;
   __shared__ int phase_s;
-  SliceState* v = st + p;
-  const size_t o = (size_t)p * N;
-  const float lam = v->lam, eps = v->eps, abar = v->abar;
-  const float* dg = dAtA + (shared ? (size_t)0 : o);
+  constexpr int SW = sizeof(SliceState) / 4;
+  static_assert(sizeof(SliceState) % 4 == 0 && SW <= QT, "state copied by words");
+  if (t < SW) reinterpret_cast<int*>(&sv)[t] = reinterpret_cast<const int*>(st + p)[t];
+  __syncthreads();
+  if (!sv.active || sv.done || sv.phase != (mode == DP_INIT ? PH_BOUNDARY : PH_PCG)) return;
+  const int N4 = N >> 2;
+  const size_t o = (size_t)p * N4;
+  auto vec = [&](float* a) { return reinterpret_cast<float4*>(a) + o; };
+  auto cvec = [&](const float* a) { return reinterpret_cast<const float4*>(a) + o; };
+  const float4* qp = reinterpret_cast<const float4*>(qpart) + o * CH;
+  const float lam = sv.lam;
+  auto save_state = [&]() {
+    __syncthreads();
+    if (t < SW) reinterpret_cast<int*>(st + p)[t] = reinterpret_cast<const int*>(&sv)[t];
+  };
+  // sums of the chunk partials, in chunk order
+  float4 q[V];
+  auto load_q = [&]() {
+#pragma unroll
+    for (int k = 0; k < V; ++k) q[k] = f4zero();
+#pragma unroll 4
+    for (int c = 0; c < CH; ++c)
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        const int f = t + QT * k;
+        if (f < N4) {
+          const float4 a = __ldcs(qp + (size_t)c * N4 + f);
+          q[k].x += a.x;
+          q[k].y += a.y;
+          q[k].z += a.z;
+          q[k].w += a.w;
+        }
+      }
+  };
   if (mode == DP_INIT) {
     // W and P from x^k, r_0 = A^T b - S x^k, z_0 = P^{-1} r_0, d_0 = z_0
-    double rz = 0.0, rr = 0.0;
-    for (int i = threadIdx.x; i < N; i += PT) {
-      const float xi = x[o + i];
-      const float wi = rsqrtf(fmaf(xi, xi, eps));
-      const float pd = precond == FIRLS_PRECOND_JACOBI ? dg[i] + lam * wi
+    const float eps = sv.eps, abar = sv.abar;
+    const float4* dg = reinterpret_cast<const float4*>(dAtA) + (shared ? (size_t)0 : o);
+    float4 rv[V], zv[V];
+    load_q();
+    auto one = [&](float xi, float di, float bi, float qi, float& wi, float& pi, float& ri, float& zi) {
+      wi = rsqrtf(fmaf(xi, xi, eps));
+      const float pd = precond == FIRLS_PRECOND_JACOBI ? di + lam * wi
                        : precond == FIRLS_PRECOND_NONE ? 1.f
                                                        : abar + lam * wi;
-      const float pi = 1.f / pd;
-      w[o + i] = wi;
-      pinv[o + i] = pi;
-      const float ri = atb[o + i] - (qsum(qpart, p, CH, N, i) + lam * wi * xi);
-      const float zi = pi * ri;
-      r[o + i] = ri;
-      z[o + i] = zi;
-      d[o + i] = zi;
-      rz += (double)ri * zi;
-      rr += (double)ri * ri;
+      pi = 1.f / pd;
+      ri = bi - (qi + lam * wi * xi);
+      zi = pi * ri;
+    };
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      const int f = t + QT * k;
+      rv[k] = zv[k] = f4zero();
+      if (f >= N4) continue;
+      const float4 xi = vec(x)[f], di = dg[f], bi = cvec(atb)[f];
+      float4 wi, pi;
+      one(xi.x, di.x, bi.x, q[k].x, wi.x, pi.x, rv[k].x, zv[k].x);
+      one(xi.y, di.y, bi.y, q[k].y, wi.y, pi.y, rv[k].y, zv[k].y);
+      one(xi.z, di.z, bi.z, q[k].z, wi.z, pi.z, rv[k].z, zv[k].z);
+      one(xi.w, di.w, bi.w, q[k].w, wi.w, pi.w, rv[k].w, zv[k].w);
+      vec(w)[f] = wi;
+      vec(pinv)[f] = pi;
+      vec(r)[f] = rv[k];
+      vec(d)[f] = zv[k];
     }
-    rz = bsum(rz, red, &bc);
-    rr = bsum(rr, red, &bc);
-    if (threadIdx.x == 0) pcg_rho_init_from(v, rz, rr);
+    dots<V>(red, rv, zv, rv, rv, true, [&](double rz, double rr) { pcg_rho_init_from(&sv, rz, rr); });
+    save_state();
     return;
   }
   // q = S d, alpha = rho / <d, q>
-  double dq = 0.0;
-  for (int i = threadIdx.x; i < N; i += PT) {
-    const float di = d[o + i];
-    const float qi = qsum(qpart, p, CH, N, i) + lam * w[o + i] * di;
-    q[o + i] = qi;
-    dq += (double)di * qi;
+  float4 dv[V], rv[V], pv[V], ev[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const int f = t + QT * k;
+    const bool in = f < N4;
+    dv[k] = in ? vec(d)[f] : f4zero();
+    rv[k] = in ? vec(r)[f] : f4zero();
+    pv[k] = in ? vec(pinv)[f] : f4zero();
+    ev[k] = in ? vec(dx)[f] : f4zero();
   }
-  dq = bsum(dq, red, &bc);
-  if (threadIdx.x == 0) {
-    pcg_alpha_from(v, dq);
-    phase_s = v->done ? -1 : v->phase;
+  load_q();
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const int f = t + QT * k;
+    const float4 wi = f < N4 ? vec(w)[f] : f4zero();
+    q[k].x = q[k].x + lam * wi.x * dv[k].x;
+    q[k].y = q[k].y + lam * wi.y * dv[k].y;
+    q[k].z = q[k].z + lam * wi.z * dv[k].z;
+    q[k].w = q[k].w + lam * wi.w * dv[k].w;
   }
-  __syncthreads();
-  if (phase_s < 0) return;  // breakdown: x keeps x^k
+  dots<V>(red, dv, q, dv, q, false, [&](double dq, double) {
+    pcg_alpha_from(&sv, dq);
+    phase_s = sv.done ? -1 : sv.phase;
+  });
+  if (phase_s < 0) {  // breakdown: x keeps x^k
+    save_state();
+    return;
+  }
   if (phase_s == PH_PCG) {
-    const float alpha = (float)v->alpha;
-    double rz = 0.0, rr = 0.0;
-    for (int i = threadIdx.x; i < N; i += PT) {
-      dx[o + i] = fmaf(alpha, d[o + i], dx[o + i]);
-      const float ri = fmaf(-alpha, q[o + i], r[o + i]);
-      const float zi = pinv[o + i] * ri;
-      r[o + i] = ri;
-      z[o + i] = zi;
-      rz += (double)ri * zi;
-      rr += (double)ri * ri;
+    const float alpha = (float)sv.alpha;
+    auto upd = [&](float di, float& ei, float& ri, float pi, float& qi) {  // q becomes z
+      ei = fmaf(alpha, di, ei);
+      ri = fmaf(-alpha, qi, ri);
+      qi = pi * ri;
+    };
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      upd(dv[k].x, ev[k].x, rv[k].x, pv[k].x, q[k].x);
+      upd(dv[k].y, ev[k].y, rv[k].y, pv[k].y, q[k].y);
+      upd(dv[k].z, ev[k].z, rv[k].z, pv[k].z, q[k].z);
+      upd(dv[k].w, ev[k].w, rv[k].w, pv[k].w, q[k].w);
+      const int f = t + QT * k;
+      if (f < N4) vec(r)[f] = rv[k];
     }
-    rz = bsum(rz, red, &bc);
-    rr = bsum(rr, red, &bc);
-    if (threadIdx.x == 0) {
-      pcg_beta_from(v, rz, rr, ps);
-      phase_s = v->phase;
-    }
-    __syncthreads();
+    dots<V>(red, rv, q, rv, rv, true, [&](double rz, double rr) {
+      pcg_beta_from(&sv, rz, rr, ps);
+      phase_s = sv.phase;
+    });
     if (phase_s == PH_PCG) {
-      const float beta = (float)v->beta;
-      for (int i = threadIdx.x; i < N; i += PT) d[o + i] = fmaf(beta, d[o + i], z[o + i]);
+      const float beta = (float)sv.beta;
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        const int f = t + QT * k;
+        if (f >= N4) continue;
+        vec(dx)[f] = ev[k];
+        vec(d)[f] = make_float4(fmaf(beta, dv[k].x, q[k].x), fmaf(beta, dv[k].y, q[k].y),
+                                fmaf(beta, dv[k].z, q[k].z), fmaf(beta, dv[k].w, q[k].w));
+      }
+      save_state();
       return;
     }
   }
   // end of the outer step: x^{k+1} = x^k + dx, relative change, stop
-  double xx = 0.0, dd = 0.0;
-  for (int i = threadIdx.x; i < N; i += PT) {
-    const float xi = x[o + i], di = dx[o + i];
-    xx += (double)xi * xi;
-    dd += (double)di * di;
-    x[o + i] = xi + di;
-    dx[o + i] = 0.f;
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const int f = t + QT * k;
+    rv[k] = f4zero();
+    if (f >= N4) continue;
+    rv[k] = vec(x)[f];
+    vec(x)[f] = make_float4(rv[k].x + ev[k].x, rv[k].y + ev[k].y, rv[k].z + ev[k].z, rv[k].w + ev[k].w);
+    vec(dx)[f] = f4zero();
   }
-  xx = bsum(xx, red, &bc);
-  dd = bsum(dd, red, &bc);
-  if (threadIdx.x == 0) {
+  dots<V>(red, rv, rv, ev, ev, true, [&](double xx, double dd) {
     const double rel = xx > 0.0 ? sqrt(dd / xx) : INFINITY;
-    v->relchg = rel;
-    v->outer_done += 1;
-    if ((outer_tol > 0.f && rel <= (double)outer_tol) || v->outer_done >= v->outer_max) v->done = 1;
-    else v->phase = PH_BOUNDARY;
-  }
+    sv.relchg = rel;
+    sv.outer_done += 1;
+    if ((outer_tol > 0.f && rel <= (double)outer_tol) || sv.outer_done >= sv.outer_max) sv.done = 1;
+    else sv.phase = PH_BOUNDARY;
+  });
+  save_state();
 }
 
 // diag(A^T A)_j = sum_i A_ij^2 per matrix (thread per column, rows in order).
@@ -470,12 +644,19 @@ int gemm_splits(int tiles, int K, int slots) {
 }
 
 // T[p][i] = sum over the splits of Tpart[s][p][i] (split order).
-__global__ void k_dense_sum_splits(int count, int S, const float* __restrict__ part, float* __restrict__ out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-    float a = 0.f;
-    for (int sp = 0; sp < S; ++sp) a += part[(size_t)sp * count + i];
-    out[i] = a;
+__global__ void k_dense_sum_splits(int count4, int S, const float4* __restrict__ part, float4* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count4) return;
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+  for (int sp = 0; sp < S; ++sp) {
+    const float4 v = __ldcs(part + (size_t)sp * count4 + i);
+    a.x += v.x;
+    a.y += v.y;
+    a.z += v.z;
+    a.w += v.w;
   }
+  out[i] = a;
 }
 
 }  // namespace
@@ -491,7 +672,7 @@ struct firls_dense_ctx {
   bool matrix_set = false;
   float *A = nullptr, *dAtA = nullptr, *abar = nullptr;
   double* abar64 = nullptr;
-  float *atb = nullptr, *x = nullptr, *dx = nullptr, *r = nullptr, *z = nullptr, *d = nullptr, *q = nullptr;
+  float *atb = nullptr, *x = nullptr, *dx = nullptr, *r = nullptr, *d = nullptr;
   float *w = nullptr, *pinv = nullptr, *qpart = nullptr, *lam = nullptr;
   SliceState* st = nullptr;
   std::vector<void*> allocs;
@@ -556,9 +737,9 @@ void launch_rows(firls_dense_ctx* c, int mode, const float* v, const float* b) {
     const int kper1 = ((N + c->S1 - 1) / c->S1 + GK - 1) / GK * GK;
     k_dense_gemm<true><<<dim3((M + GN - 1) / GN, (P + GM - 1) / GM, c->S1), GT, 0, c->stream>>>(
         P, M, N, kper1, v, N, c->A, N, c->tpart, M, (size_t)P * M);
-    const int cnt = P * M;
-    k_dense_sum_splits<<<(cnt + 255) / 256 < 1024 ? (cnt + 255) / 256 : 1024, 256, 0, c->stream>>>(cnt, c->S1,
-                                                                                                    c->tpart, c->tmat);
+    const int cnt4 = P * M / 4;  // M % 4 = 0 on this path
+    k_dense_sum_splits<<<(cnt4 + 127) / 128, 128, 0, c->stream>>>(cnt4, c->S1, reinterpret_cast<const float4*>(c->tpart),
+                                                                  reinterpret_cast<float4*>(c->tmat));
   }
   // q partials = T A over CH splits of M: partial s of problem p at qpart[(p CH + s) N]
   const int kper2 = ((M + c->CH - 1) / c->CH + GK - 1) / GK * GK;
@@ -567,8 +748,10 @@ void launch_rows(firls_dense_ctx* c, int mode, const float* v, const float* b) {
 }
 
 void launch_pcg(firls_dense_ctx* c, int mode, int precond, const PcgSched& ps, float outer_tol) {
-  k_dense_pcg<<<c->P, PT, 0, c->stream>>>(c->N, c->CH, mode, c->st, c->qpart, c->x, c->dx, c->r, c->z, c->d, c->q,
-                                           c->w, c->pinv, c->atb, c->dAtA, c->shared, precond, ps, outer_tol);
+  const int v = ((c->N >> 2) + QT - 1) / QT;  // N <= 8192
+  auto k = v <= 1 ? k_dense_pcg<1> : v <= 2 ? k_dense_pcg<2> : k_dense_pcg<4>;
+  k<<<c->P, QT, 0, c->stream>>>(c->N, c->CH, mode, c->st, c->qpart, c->x, c->dx, c->r, c->d, c->w, c->pinv, c->atb,
+                                c->dAtA, c->shared, precond, ps, outer_tol);
 }
 
 // One outer step: the start (S x^k, r_0, z_0) and J PCG steps; problems
@@ -641,7 +824,7 @@ extern "C" firls_status firls_dense_create(firls_dense_ctx** out, int M, int N, 
   al(&c->dAtA, (size_t)c->nA * N);
   al(&c->abar, (size_t)c->nA);
   al(&c->abar64, (size_t)c->nA);
-  for (float** v : {&c->atb, &c->x, &c->dx, &c->r, &c->z, &c->d, &c->q, &c->w, &c->pinv}) al(v, PN);
+  for (float** v : {&c->atb, &c->x, &c->dx, &c->r, &c->d, &c->w, &c->pinv}) al(v, PN);
   al(&c->qpart, PN * c->CH);
   if (c->gemm) {
     al(&c->tpart, (size_t)c->S1 * problems * M);
