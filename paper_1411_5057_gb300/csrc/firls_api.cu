@@ -1422,9 +1422,12 @@ extern "C" firls_status firls_autotune(firls_ctx* c, const char* cache_path) {
     if (has_tv(c)) penta_setup(B, n, c->stream, c->st, c->wtv, tv2_of(c), nullptr, c->ia);
     float best = 1e30f;
     if (c->kind) {
-      for (int r : {1, 2, 4, 8, 16})
+      // rb 0 only where it is a form of its own (the clusters above 256^2)
+      const bool wide = wavelet_cluster_ctas(n, c->levels, c->kind, 0) && !wavelet_cluster_ctas(n, c->levels, c->kind, 1);
+      for (int r : {0, 1, 2, 4, 8, 16})
         for (int m : {32, 64}) {
           const bool cluster = r < 4;
+          if (r == 0 && !wide) continue;
           if (cluster && (m != 64 || !wavelet_cluster_ctas(n, c->levels, c->kind, r))) continue;
           WavArgs w = wav_args(c, c->st);
           w.rb = r;

@@ -320,13 +320,43 @@ k_wav_coarse(const float2* __restrict__ src, size_t src_ss, int src_ld, float2* 
   }
 }
 
+// Clusters of the one-launch form above WCL_NMAX that the current device
+// holds at once (0: it cannot launch them), asked once per device.
+static int wide_resident(int n, int kind) {
+  static PerDeviceOnce once;
+  static int held[64][2][3];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 0;
+  once.run([dev] {
+    for (int i = 0; i < 3; ++i) {
+      constexpr int side[3] = {320, 384, 512};
+      held[dev][0][i] = wcl_wide_haar(side[i]);
+      held[dev][1][i] = wcl_wide_db4(side[i]);
+    }
+    return true;
+  });
+  const int i = n == 320 ? 0 : n == 384 ? 1 : n == 512 ? 2 : -1;
+  return i < 0 ? 0 : held[dev][kind - 1][i];
+}
+
 // Rows per CTA of the one-launch form (0 when it does not apply): the
 // fewest rows (most CTAs, at most 8 per cluster) for which every level has an
 // even number of rows per CTA.  choice: 0 default, 1 weights mirrored in
-// shared memory, 2 read from HBM; *mirror receives which.
+// shared memory, 2 read from HBM; *mirror receives which.  Above 256^2 only the
+// default takes it, with clusters of n / 32 CTAs where the device launches
+// them.  Solves of 20 PCG steps, 5 levels, against the tiled levels with 8 rows
+// a CTA: 512^2 D4 1 slice 4.8 -> 2.5 ms, 8 slices 6.5 -> 4.6 (two waves of
+// clusters, 7 fit at once), 64 slices 25.2 -> 21.4; 320^2 5 slices 3.8 -> 2.1,
+// 120 slices 17.3 -> 16.2; 384^2 8 slices 5.0 -> 2.7, 80 slices 19.0 -> 18.6;
+// Haar gains more.  No batch is left for which the tiled levels are faster.
 static int wcl_rows_per_cta(int n, int L, int kind, int choice, bool* mirror) {
   if (kind != 1 && kind != 2) return 0;
   if (choice != 0 && choice != 1 && choice != 2) return 0;
+  if (choice == 0 && n > WCL_NMAX) {
+    if (L < 1 || L > WCL_LMAX || (n >> L) % 4 || !wide_resident(n, kind)) return 0;
+    if (mirror) *mirror = true;
+    return WCL_WIDE_R;
+  }
   if (n % 8 || n > WCL_NMAX || L < 1 || L > WCL_LMAX || (n >> L) % 4) return 0;
   for (int C = 8; C >= 1; --C) {
     if (n % (C << L) || n / C > WCL_RMAX) continue;

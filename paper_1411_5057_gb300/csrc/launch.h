@@ -69,7 +69,8 @@ void wavelet_forward(const WavArgs& a, const float2* x, float2* c, float* w, int
 void wavelet_inverse(const WavArgs& a, const float2* c, float2* x, const float2* r, int real);
 // u = Phi^T (s o Phi x), s = w (MUL_W) or 1/(abar + lam w) (MUL_PINV).
 // Where a slice fits the shared memory of one thread-block cluster (rb 0, 1
-// or 2) every level runs in one launch and c is not touched; otherwise
+// or 2; above 256^2 only rb 0) every level runs in one launch and c is not
+// touched; otherwise
 // (rb 4, 8, 16, or no fit) the fine levels are tiled, a launch per level,
 // their scaled details going through c, and the levels that fit one CTA's
 // shared memory are fused.  Optional partial Re<r, u>.

@@ -77,6 +77,7 @@ FI void inv_haar(float2 a, float2 d, float2& x0, float2& x1) {
 constexpr int WCL_NMAX = 256;
 constexpr int WCL_LMAX = 5;
 constexpr int WCL_RMAX = 32;  // rows per CTA: two CTAs per SM fit with the weights mirrored
+constexpr int WCL_WIDE_R = 32;  // rows per CTA of the sizes above WCL_NMAX (clusters of 10, 12, 16)
 
 FI unsigned wcl_rank() {
   unsigned r;
@@ -371,7 +372,7 @@ FI void wcl_push(const float2* D, const float2* Hb, const uint64_t* bar, int n, 
 // its arguments served every size but 256^2 before: 228 us at 304 slices of
 // 128^2, against 144 us for four times the pixels at 256^2.
 template <int NT, int RT, int LT, int KT, int TH>
-__global__ void __launch_bounds__(TH, 2)
+__global__ void __launch_bounds__(TH, NT <= 256 ? 2 : 1)
 k_wav_cluster(const float2* x, float2* u, const float* __restrict__ w, int L_arg, int mode, int mirror, 
               const float2* __restrict__ r, double* __restrict__ part, int real, SliceState* __restrict__ st) {
   const int s = blockIdx.y;
@@ -497,25 +498,48 @@ struct WclArgs {
   cudaStream_t stream;
 };
 
-template <int N, int R, int L, int KT, int TH> bool wcl_launch_as(const WclArgs& a) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(N / R, a.batch);
+template <int N, int R, int TH>
+inline void wcl_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int levels, bool mirror, int batch,
+                       cudaStream_t stream) {
+  cfg = {};
+  cfg.gridDim = dim3(N / R, batch);
   cfg.blockDim = dim3(TH);
-  cfg.dynamicSmemBytes = wcl_smem_bytes(N, R, a.levels, a.mirror);
-  cfg.stream = a.stream;
-  cudaLaunchAttribute at[1];
+  cfg.dynamicSmemBytes = wcl_smem_bytes(N, R, levels, mirror);
+  cfg.stream = stream;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = N / R;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+}
+
+template <int N, int R, int L, int KT, int TH> bool wcl_launch_as(const WclArgs& a) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[1];
+  wcl_config<N, R, TH>(cfg, at, a.levels, a.mirror, a.batch, a.stream);
   return cudaLaunchKernelEx(&cfg, k_wav_cluster<N, R, L, KT, TH>, a.x, a.u, a.w, a.levels, a.mode, a.mirror, a.r,
                             a.part, a.real, a.st) == cudaSuccess;
 }
 template <int N, int R, int L, int KT, int TH> bool wcl_attr_as() {
   return cudaFuncSetAttribute(k_wav_cluster<N, R, L, KT, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               wcl_smem_bytes(N, R, L ? L : WCL_LMAX, true)) == cudaSuccess;
+}
+// A cluster above the portable 8 CTAs: how many the device holds at once, 0
+// where it cannot be launched.
+template <int N, int R, int KT, int TH> int wcl_wide_resident() {
+  auto k = k_wav_cluster<N, R, 0, KT, TH>;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[1];
+  wcl_config<N, R, TH>(cfg, at, WCL_LMAX, true, 1, nullptr);
+  int clusters = 0;
+  if (!wcl_attr_as<N, R, 0, KT, TH>() ||
+      cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&clusters, k, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return clusters;
 }
 
 // Every (size, rows per CTA) that wcl_rows_per_cta gives, with the threads per
@@ -526,13 +550,29 @@ template <int N, int R, int L, int KT, int TH> bool wcl_attr_as() {
   X(80, 10, 256) X(80, 16, 256) X(96, 12, 256) X(96, 16, 256) X(128, 16, 256) X(128, 32, 256) X(160, 20, 512)      \
   X(160, 32, 512) X(192, 24, 512) X(192, 32, 512) X(256, 32, 512)
 
+// The sizes above WCL_NMAX: one CTA per SM, more CTAs than a portable cluster.
+// 512 threads at 512^2: 1024 leave 64 registers and spill (8 slices of 20 PCG
+// steps 5.05 against 4.58 ms).
+#define WCL_WIDE_SHAPES(X) X(320, 640) X(384, 768) X(512, 512)
+
 template <int KT> bool wcl_launch_kind(int n, int R, const WclArgs& a) {
   if (n == 256 && a.levels == 4) return wcl_launch_as<256, 32, 4, KT, 512>(a);
 #define WCL_CASE(N_, R_, T_) \
   if (n == N_ && R == R_) return wcl_launch_as<N_, R_, 0, KT, T_>(a);
   WCL_SHAPES(WCL_CASE)
 #undef WCL_CASE
+#define WCL_CASE(N_, T_) \
+  if (n == N_ && R == WCL_WIDE_R) return wcl_launch_as<N_, WCL_WIDE_R, 0, KT, T_>(a);
+  WCL_WIDE_SHAPES(WCL_CASE)
+#undef WCL_CASE
   return false;
+}
+template <int KT> int wcl_wide_kind(int n) {
+#define WCL_CASE(N_, T_) \
+  if (n == N_) return wcl_wide_resident<N_, WCL_WIDE_R, KT, T_>();
+  WCL_WIDE_SHAPES(WCL_CASE)
+#undef WCL_CASE
+  return 0;
 }
 template <int KT> bool wcl_attrs_kind() {
   bool ok = wcl_attr_as<256, 32, 4, KT, 512>();
@@ -543,6 +583,8 @@ template <int KT> bool wcl_attrs_kind() {
 }
 bool wcl_launch_haar(int n, int R, const WclArgs& a);
 bool wcl_launch_db4(int n, int R, const WclArgs& a);
+int wcl_wide_haar(int n);
+int wcl_wide_db4(int n);
 bool wcl_prepare_haar();
 bool wcl_prepare_db4();
 
