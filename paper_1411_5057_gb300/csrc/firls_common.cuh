@@ -143,4 +143,46 @@ FI double block_sum(double v, double* red) {
   return s;
 }
 
+// s + e = a + b exactly.
+FI void two_sum(float a, float b, float& s, float& e) {
+  const float t = a + b, bb = t - a;
+  e = (a - (t - bb)) + (b - bb);
+  s = t;
+}
+
+// A sum carried in three floats, for kernels that accumulate many values each:
+// the device has 2 FP64 lanes per clock and SM.  A product of two floats is
+// exactly p + e with e = fma(a, b, -p); each two_sum is exact and the third
+// float takes the remainders, so it loses less than an FP64 sum.
+struct Sum3 {
+  float s, c, cc;  // value s + c + cc
+  FI void add(float v) {
+    float e, f;
+    two_sum(s, v, s, e);
+    two_sum(c, e, c, f);
+    cc += f;
+  }
+  FI void add(float v, float lo) {  // v + lo, |lo| <= ulp(v)
+    float e, f;
+    two_sum(s, v, s, e);
+    two_sum(c, lo, c, f);
+    cc += f;
+    two_sum(c, e, c, f);
+    cc += f;
+  }
+  FI void add_product(float a, float b) {
+    const float p = a * b;
+    add(p, fmaf(a, b, -p));
+  }
+  FI void add(const Sum3& o) {
+    add(o.s, o.c);
+    cc += o.cc;
+  }
+  FI Sum3 from_lane(int o) const {
+    return {__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o),
+            __shfl_xor_sync(0xffffffffu, cc, o)};
+  }
+  FI double value() const { return (double)s + ((double)c + (double)cc); }
+};
+
 }  // namespace firls

@@ -204,46 +204,12 @@ enum DensePcg { DP_INIT = 0, DP_STEP = 1 };
 
 constexpr int QT = 512;  // threads of the PCG kernel
 
-// Inner products of a problem's vectors.  The device has 2 FP64 lanes per
-// clock and SM: converting and accumulating 4000 products in FP64 took most of
-// the PCG kernel.  A product of two floats is exactly p + e with
-// e = fma(a, b, -p), and a sum carried in three floats loses less than an FP64
-// one (each two_sum is exact, the third float takes the remainders), so only
-// the final value is FP64.  Floats have less range than doubles: a result
-// outside [SUM_LO, SUM_HI] (or NaN) is formed again in FP64, so tiny and huge
+// Inner products of a problem's vectors as Sum3: converting and accumulating
+// 4000 products in FP64 took most of the PCG kernel.  Floats have less range
+// than doubles: a result outside [SUM_LO, SUM_HI] (or NaN) is formed again in FP64, so tiny and huge
 // problems give what they gave.  Inside, the low halves lost to underflow are
 // at most N 2^-149 < 2e-41, 2e-16 of SUM_LO.
 constexpr double SUM_LO = 1e-25, SUM_HI = 1e30;
-
-FI void two_sum(float a, float b, float& s, float& e) {
-  const float t = a + b, bb = t - a;
-  e = (a - (t - bb)) + (b - bb);
-  s = t;
-}
-
-struct Sum3 {
-  float s, c, cc;  // value s + c + cc
-  FI void add(float v, float lo) {  // v + lo, |lo| <= ulp(v)
-    float e, f;
-    two_sum(s, v, s, e);
-    two_sum(c, lo, c, f);
-    cc += f;
-    two_sum(c, e, c, f);
-    cc += f;
-  }
-  FI void add_product(float a, float b) {
-    const float p = a * b;
-    add(p, fmaf(a, b, -p));
-  }
-  FI void add(const Sum3& o) {
-    add(o.s, o.c);
-    cc += o.cc;
-  }
-  FI Sum3 from_lane(int o) const {
-    return {__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o),
-            __shfl_xor_sync(0xffffffffu, cc, o)};
-  }
-};
 
 struct DotRed {
   Sum3 part[2][QT / 32];
@@ -287,7 +253,7 @@ FI void dots(DotRed& red, const float4 (&a0)[V], const float4 (&b0)[V], const fl
     if (two || lane < 16) t = red.part[lane >> 4][lane & 15];
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) t.add(t.from_lane(o));
-    const double mine = (double)t.s + ((double)t.c + (double)t.cc);
+    const double mine = t.value();
     const double other = __shfl_xor_sync(0xffffffffu, mine, 16);
     if (lane == 0) {
       const bool ok = fabs(mine) > SUM_LO && fabs(mine) < SUM_HI && (!two || (fabs(other) > SUM_LO && fabs(other) < SUM_HI));

@@ -660,15 +660,16 @@ struct CnnLayers {
   CnnLayer l[NL];
 };
 
-// The end of a training step for every layer: the gradients (fixed-order FP64
-// sums of the per-CTA partials), Adam (Kingma & Ba) on the FP32 masters and the
-// packed BF16 copies.  A CTA takes 32 parameters, 8 threads each to fetch and
-// add the partials (coalesced over the parameters).  One launch instead of 30,
-// and the sums no longer 296 loads in a row per thread (107 us per layer).
+// The end of a training step for every layer: the gradients (fixed-order sums
+// of the per-CTA partials, carried in three floats), Adam (Kingma & Ba) on the
+// FP32 masters and the packed BF16 copies.  A CTA takes 32 parameters, 8 threads
+// each to fetch and add the partials (coalesced over the parameters).  One launch
+// instead of 30, and the sums no longer 296 loads in a row per thread (107 us per
+// layer); 43 MB of partials, 49 us with FP64 sums, 21 us with these.
 constexpr int UP_PARAMS = 32, UP_PARTS = 8;
 __global__ void __launch_bounds__(UP_PARAMS* UP_PARTS) k_cnn_update(CnnLayers layers, int ctas, float lr, float b1,
                                                                     float b2, float eps, float c1, float c2) {
-  __shared__ double red[UP_PARTS][UP_PARAMS];
+  __shared__ Sum3 red[UP_PARTS][UP_PARAMS];
   int li = NL - 1;
   while (li > 0 && (int)blockIdx.x < layers.l[li].first) --li;
   const CnnLayer& L = layers.l[li];
@@ -676,24 +677,26 @@ __global__ void __launch_bounds__(UP_PARAMS* UP_PARTS) k_cnn_update(CnnLayers la
   const int u = threadIdx.x % UP_PARAMS, k = threadIdx.x / UP_PARAMS;
   const int i = (blockIdx.x - L.first) * UP_PARAMS + u;
   const int t = i / (L.cin * L.cout), ci = (i / L.cout) % L.cin, co = i % L.cout;
-  double s = 0.0;
-  if (i < nw) {
-    const size_t stride = (size_t)9 * L.cinp * L.coutp;
-    const float* p = L.pw + ((size_t)t * L.cinp + ci) * L.coutp + co;
-#pragma unroll 4
-    for (int c = k; c < ctas; c += UP_PARTS) s += p[c * stride];
-  } else if (i < nw + L.cout) {
-    const float* p = L.pb + (i - nw);
-    for (int c = k; c < ctas; c += UP_PARTS) s += p[(size_t)c * L.coutp];
+  const bool weight = i < nw;
+  const size_t stride = weight ? (size_t)9 * L.cinp * L.coutp : (size_t)L.coutp;
+  const float* parts = weight ? L.pw + ((size_t)t * L.cinp + ci) * L.coutp + co : L.pb + (i - nw);
+  Sum3 s{0.f, 0.f, 0.f};
+  if (i < nw + L.cout) {
+#pragma unroll 8
+    for (int c = k; c < ctas; c += UP_PARTS) s.add(__ldcs(parts + c * stride));
   }
   red[k][u] = s;
   __syncthreads();
   if (k != 0 || i >= nw + L.cout) return;
 #pragma unroll
-  for (int c = 1; c < UP_PARTS; ++c) s += red[c][u];
-  const bool weight = i < nw;
+  for (int c = 1; c < UP_PARTS; ++c) s.add(red[c][u]);
   const int q = weight ? i : i - nw;
-  const float gi = (float)s;
+  float gi = (float)s.value();
+  if (!isfinite(gi)) {  // the floats overflowed on the way, or the gradient is not finite: FP64 decides
+    double wide = 0.0;
+    for (int c = 0; c < ctas; ++c) wide += parts[c * stride];
+    gi = (float)wide;
+  }
   (weight ? L.gw : L.gb)[q] = gi;
   float* m = weight ? L.mw : L.mb;
   float* v = weight ? L.vw : L.vb;
