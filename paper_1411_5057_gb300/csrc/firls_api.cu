@@ -60,6 +60,7 @@ struct firls_ctx {
   int wait_test = 0;  // failure-detection test: the ILU's bounded waits run out (firls_set_wait_test)
   SliceState* st = nullptr;
   double* part = nullptr;
+  double* fobj = nullptr;  // F_eps of two estimates per slice
   float *lam_d = nullptr, *lamtv_d = nullptr;
   std::vector<void*> allocs;
   std::string err;
@@ -710,6 +711,7 @@ extern "C" firls_status firls_create(firls_ctx** out, int n_rows, int n_cols, in
   A(&c->st, (size_t)batch);
   A(&c->stw, (size_t)batch);
   A(&c->part, (size_t)batch * NSLOT * MAXPART);
+  A(&c->fobj, 2 * (size_t)batch);
   A(&c->lam_d, (size_t)batch);
   A(&c->lamtv_d, (size_t)batch);
   if (s != FIRLS_OK) {
@@ -1187,34 +1189,11 @@ firls_status objective_parts(firls_ctx* c, const void* b, const firls_params* p,
   return cuda_check(c, cudaGetLastError(), "objective");
 }
 
-firls_status objective_read(firls_ctx* c, const firls_params* p, double* out) {
-  const int B = c->batch, n = c->n;
-  std::vector<double> h((size_t)B * NSLOT * MAXPART);
-  CU(cudaMemcpyAsync(h.data(), c->part, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, c->stream));
-  CU(cudaStreamSynchronize(c->stream));
-  const int nd = fft_col_ctas(n), nr = axpy_ctas(n);
-  for (int s = 0; s < B; ++s) {
-    auto sum = [&](int slot, int np) {
-      double a = 0.0;
-      for (int i = 0; i < np; ++i) a += h[((size_t)s * NSLOT + slot) * MAXPART + i];
-      return a;
-    };
-    const double lam = p->lambda_per_slice ? p->lambda_per_slice[s] : p->lambda;
-    const double lt = p->lambda_tv_per_slice ? p->lambda_tv_per_slice[s] : p->lambda_tv;
-    double f = 0.5 * sum(SLOT_DQ, nd);
-    if (c->kind) f += lam * sum(SLOT_RZ, nr);
-    if (has_tv(c)) f += lt * sum(SLOT_RR, nr);
-    out[s] = f;
-  }
-  // multi-contrast: F_eps of the whole image (the joint regularisers sit in
-  // its first slice's parts), the same value for each of its contrasts
-  const int C = c->channels;
-  for (int s0 = 0; C > 1 && s0 < B; s0 += C) {
-    double f = 0.0;
-    for (int t = 0; t < C; ++t) f += out[s0 + t];
-    for (int t = 0; t < C; ++t) out[s0 + t] = f;
-  }
-  return FIRLS_OK;
+// F_eps from the parts, into fobj[which][batch] on the device.  The lambdas are
+// those that upload_params left there.
+void objective_values(firls_ctx* c, int which) {
+  objective_sum(c->batch, c->stream, c->part, fft_col_ctas(c->n), axpy_ctas(c->n), c->kind != 0, has_tv(c), c->lam_d,
+                c->lamtv_d, c->fobj + (size_t)which * c->batch, c->channels);
 }
 
 // ---- continuous batching: per-slot load, run, status, read-out ----
@@ -1573,7 +1552,10 @@ extern "C" firls_status firls_objective(firls_ctx* c, const void* b, const firls
   TRY(check_params(c, p));
   TRY(upload_params(c, p));
   TRY(objective_parts(c, b, p, static_cast<const float2*>(x)));
-  return objective_read(c, p, out);
+  objective_values(c, 0);
+  CU(cudaMemcpyAsync(out, c->fobj, sizeof(double) * c->batch, cudaMemcpyDeviceToHost, c->stream));
+  CU(cudaStreamSynchronize(c->stream));
+  return FIRLS_OK;
 }
 
 extern "C" firls_status firls_warm_start_guard(firls_ctx* c, const void* b, const firls_params* p, const void* x1,
@@ -1584,9 +1566,8 @@ extern "C" firls_status firls_warm_start_guard(firls_ctx* c, const void* b, cons
   TRY(upload_params(c, p));
   const int B = c->batch, n = c->n;
   const size_t slice = sizeof(float2) * (size_t)n * n;
-  std::vector<double> f1(B), f0(B);
   TRY(objective_parts(c, b, p, static_cast<const float2*>(x1)));
-  TRY(objective_read(c, p, f1.data()));
+  objective_values(c, 1);
   // A^H b into the context's atb buffer
   FftArgs a = fft_args(c);
   a.b = static_cast<const float2*>(b);
@@ -1597,12 +1578,18 @@ extern "C" firls_status firls_warm_start_guard(firls_ctx* c, const void* b, cons
   a.x = nullptr;
   fft_col_inv(n, a);
   TRY(objective_parts(c, b, p, c->atb));
-  TRY(objective_read(c, p, f0.data()));
+  objective_values(c, 0);
+  const bool aligned = (reinterpret_cast<uintptr_t>(x1) | reinterpret_cast<uintptr_t>(x0)) % 16 == 0;
+  if (aligned) guard_pick(B, n, c->stream, c->fobj + B, c->fobj, x1, c->atb, x0);
+  std::vector<double> f(2 * (size_t)B);
+  CU(cudaMemcpyAsync(f.data(), c->fobj, sizeof(double) * f.size(), cudaMemcpyDeviceToHost, c->stream));
+  CU(cudaStreamSynchronize(c->stream));
   for (int s = 0; s < B; ++s) {
-    const bool use = std::isfinite(f1[s]) && f1[s] <= f0[s];
+    const bool use = guard_keeps(f[B + s], f[s]);
+    if (chosen) chosen[s] = use ? 1 : 0;
+    if (aligned) continue;
     const void* src = use ? static_cast<const char*>(x1) + s * slice : static_cast<const void*>(c->atb + (size_t)s * n * n);
     CU(cudaMemcpyAsync(static_cast<char*>(x0) + s * slice, src, slice, cudaMemcpyDeviceToDevice, c->stream));
-    if (chosen) chosen[s] = use ? 1 : 0;
   }
   return cuda_check(c, cudaGetLastError(), "warm_start_guard");
 }

@@ -1165,6 +1165,49 @@ FI double image_parts(const double* part, int s, int slot, int np, int C) {
   return a;
 }
 
+// F_eps of every slice from the partial sums of its terms (SLOT_DQ: |M F x - b|^2,
+// SLOT_RZ: wavelet, SLOT_RR: TV); of the whole image for each of its C contrasts.
+// On the device so that a caller reads 8 bytes a slice, not 6 KB of partials.
+__global__ void k_objective(int B, int C, const double* part, int nd, int nr, int wavelet, int tv,
+                            const float* __restrict__ lam, const float* __restrict__ lam_tv, double* __restrict__ f) {
+  const int s = sc_slice();
+  if (s >= B) return;
+  const int s0 = s - s % C;
+  double sum = 0.0;
+  for (int t = s0; t < s0 + C; ++t) {
+    double v = 0.5 * sum_parts(part, t, SLOT_DQ, nd);
+    if (wavelet) v += (double)lam[t] * sum_parts(part, t, SLOT_RZ, nr);
+    if (tv) v += (double)lam_tv[t] * sum_parts(part, t, SLOT_RR, nr);
+    sum = t == s0 ? v : sum + v;
+  }
+  if ((threadIdx.x & 31) == 0) f[s] = sum;
+}
+
+void objective_sum(int batch, cudaStream_t s, const double* part, int nd, int nr, bool wavelet, bool tv,
+                   const float* lam, const float* lam_tv, double* f, int channels) {
+  k_objective<<<sc_ctas(batch), 32 * SC_WARPS, 0, s>>>(batch, channels, part, nd, nr, wavelet, tv, lam, lam_tv, f);
+}
+
+// The warm start of each slice: x1 where its objective is finite and no larger
+// than that of A^H b, else A^H b.  One launch for the batch (a copy per slice
+// took 2 us each: 64 slices of 256^2 130 -> 11 us).
+__global__ void k_guard_pick(int N4, const double* __restrict__ f1, const double* __restrict__ f0, const float4* x1,
+                             const float4* __restrict__ atb, float4* x0) {
+  const int s = blockIdx.y;
+  const float4* src = (guard_keeps(f1[s], f0[s]) ? x1 : atb) + (size_t)s * N4;
+  float4* dst = x0 + (size_t)s * N4;
+#pragma unroll 4
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N4; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
+
+void guard_pick(int batch, int n, cudaStream_t s, const double* f1, const double* f0, const void* x1,
+                const float2* atb, void* x0) {
+  const int N4 = n * n / 2;
+  const int ctas = std::max(1, std::min(32, N4 / 1024));
+  k_guard_pick<<<dim3(ctas, batch), 256, 0, s>>>(N4, f1, f0, static_cast<const float4*>(x1),
+                                                 reinterpret_cast<const float4*>(atb), static_cast<float4*>(x0));
+}
+
 __global__ void k_state_init(int B, SliceState* st, const double* part, int np, const int* counts, int N,
                              const float* lam, const float* lam_tv, float eps, int outer_max, int phase, int C) {
   const int s = sc_slice();

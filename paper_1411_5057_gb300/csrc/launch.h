@@ -157,6 +157,14 @@ void l21_sum(int batch, int n, cudaStream_t s, const float2* c, const int* gidx,
              int gsize, float eps, double* part, int slot, int channels = 1);
 void tv_sum(int batch, int n, cudaStream_t s, const float2* x, float eps, double* part, int slot, int aniso,
             int channels = 1);
+// f[s] = F_eps of slice s from the partial sums of its terms (nd and nr of them)
+void objective_sum(int batch, cudaStream_t s, const double* part, int nd, int nr, bool wavelet, bool tv,
+                   const float* lam, const float* lam_tv, double* f, int channels);
+// whether a slice keeps the warm start x1 of objective f1, f0 that of A^H b
+__host__ __device__ inline bool guard_keeps(double f1, double f0) { return f1 - f1 == 0.0 && f1 <= f0; }
+// x0 = x1 or A^H b per slice; x1 and x0 16-byte aligned
+void guard_pick(int batch, int n, cudaStream_t s, const double* f1, const double* f0, const void* x1,
+                const float2* atb, void* x0);
 
 // PCG scalar updates (one thread per slice).  channels C > 1: the inner
 // products are summed over the C consecutive slices of a multi-contrast
