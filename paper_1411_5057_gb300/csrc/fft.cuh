@@ -243,4 +243,50 @@ FI void fft_line(float2 (&v)[FftCfg<N>::E], float* bre, float* bim, const float2
   fft_pass<N, 0, 1, DIR>(v, bre, bim, tw, t);
 }
 
+// The same FFT for a column of a 16-column tile: thread (t, c) holds rows
+// t + T e of column c, and the exchange goes through buf[row][16] of the CTA, so
+// that half a warp always moves one 128-byte row, free of bank conflicts.  Every
+// arithmetic step is fft_pass's.
+constexpr int FFT_COLS = 16;
+template <int N, int PASS, int P, int DIR>
+FI void fft_pass_col(float2 (&v)[FftCfg<N>::E], float2* buf, const float2* tw, int t, int c) {
+  using C = FftCfg<N>;
+  constexpr int R = C::radix(PASS);
+  constexpr int E = C::E, T = C::T, M = E / R;
+  constexpr bool LAST = (PASS == C::NP - 1);
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const int i = t + T * m;
+    const int k = (P == 1) ? 0 : (i % P);
+    float2 a[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) a[q] = v[m + q * M];
+    if (P > 1) {
+      const float2* twp = tw + (P - C::radix(0)) + k;
+#pragma unroll
+      for (int q = 1; q < R; ++q) a[q] = cmul(a[q], twiddle<DIR>(twp, (q - 1) * P));
+    }
+    Dft<R, DIR>::run(a);
+    if (LAST) {
+#pragma unroll
+      for (int q = 0; q < R; ++q) v[m + q * M] = a[q];
+    } else {
+      const int j = (i / P) * P * R + k;
+#pragma unroll
+      for (int q = 0; q < R; ++q) buf[(j + q * P) * FFT_COLS + c] = a[q];
+    }
+  }
+  if constexpr (!LAST) {
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < E; ++s) v[s] = buf[(t + T * s) * FFT_COLS + c];
+    __syncthreads();
+    fft_pass_col<N, PASS + 1, P * R, DIR>(v, buf, tw, t, c);
+  }
+}
+template <int N, int DIR>
+FI void fft_col(float2 (&v)[FftCfg<N>::E], float2* buf, const float2* tw, int t, int c) {
+  fft_pass_col<N, 0, 1, DIR>(v, buf, tw, t, c);
+}
+
 }  // namespace firls

@@ -6,15 +6,15 @@
 //   partial inner product Re<d, S d>.
 // The unnormalised transforms are scaled once: 1/N for F^H R F, 1/n for
 // F^H R b.  Rows: T threads of one warp per row (coalesced loads of
-// t + T*s).  Columns: tiles of 16 columns x n rows staged in shared memory
-// with 128-byte row segments.
+// t + T*s).  Columns: 16 columns x n rows per CTA, loaded and stored by the
+// threads that transform them in 128-byte row segments.
 #include "fft.cuh"
 #include "launch.h"
 #include "per_device.h"
 
 namespace firls {
 
-constexpr int COLS = 16;  // columns per column-pass CTA
+constexpr int COLS = FFT_COLS;  // columns per column-pass CTA
 
 template <int N> __host__ __device__ constexpr int rows_per_cta() {
   int r = 256 / FftCfg<N>::T;
@@ -32,18 +32,9 @@ template <int N> constexpr int row_smem_bytes(bool tv = false, bool aniso = fals
   return b;
 }
 
-// Shared memory of a column-pass CTA: twiddles (padded table) | region | mask
-// tile transposed ([COLS][N] bytes).  The region holds the N x COLS complex
-// tile (rows of 16 float2, XOR-swizzled: element (r, c) at r*COLS + (c ^ (r
-// mod COLS)), so that row-major fills and 16-row column reads are both free
-// of bank conflicts) or, while the FFT runs, the per-column exchange lines.
-template <int N> __host__ __device__ constexpr int col_region_bytes() {
-  return N * COLS * 8 > COLS * 2 * fft_line_words<N>() * 4 ? N * COLS * 8 : COLS * 2 * fft_line_words<N>() * 4;
-}
-template <int N> __host__ __device__ constexpr int col_smem_bytes() {
-  return tw_bytes<N>() + col_region_bytes<N>() + N * COLS;
-}
-FI int tslot(int r, int c) { return r * COLS + (c ^ (r & (COLS - 1))); }
+// Shared memory of a column-pass CTA: twiddles (padded table) | exchange buffer
+// [N][COLS] | mask bytes [N][COLS].
+template <int N> __host__ __device__ constexpr int col_smem_bytes() { return tw_bytes<N>() + N * COLS * 8 + N * COLS; }
 
 FI void cp_async16_fft(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
@@ -185,49 +176,22 @@ __global__ void __launch_bounds__(256) k_row_ahb(const float2* __restrict__ b, c
   for (int e = 0; e < E; ++e) t_out[base + t + T * e] = v[e];
 }
 
-// Load a 16-column tile of t into shared memory (SoA, row stride COLS+1).
+// A column pass: thread (t, c) loads rows t + T e of column c0 + c itself, all at
+// once; a warp's load is two whole 128-byte lines, and nothing passes through
+// shared memory but the FFT's own exchanges.  (A tile staged through shared
+// memory on the way in and out: 91 us for the masked pass over 304 slices of
+// 256^2, this 70: 4.9 TB/s.)
 template <int N>
-FI void load_col_tile(const float2* __restrict__ src, float2* tile, size_t sbase, int c0) {
-  // every thread issues all its 16-byte loads (two columns each) before the
-  // first shared-memory store, so a whole tile is in flight at once
-  constexpr int NT = COLS * FftCfg<N>::T, HC = COLS / 2, K = N * HC / NT;
-  static_assert(N * HC % NT == 0, "column tile split");
-  float4 g[K];
+FI void load_cols(float2 (&v)[FftCfg<N>::E], const float2* __restrict__ src, size_t sbase, int c0, int t, int c) {
+  const float2* p = src + sbase + (size_t)t * N + c0 + c;
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int idx = threadIdx.x + NT * k, r = idx / HC, cp = idx % HC;
-    g[k] = *reinterpret_cast<const float4*>(src + sbase + (size_t)r * N + c0 + 2 * cp);
-  }
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int idx = threadIdx.x + NT * k, r = idx / HC, cp = idx % HC;
-    tile[tslot(r, 2 * cp)] = make_float2(g[k].x, g[k].y);
-    tile[tslot(r, 2 * cp + 1)] = make_float2(g[k].z, g[k].w);
-  }
+  for (int e = 0; e < FftCfg<N>::E; ++e) v[e] = p[(size_t)FftCfg<N>::T * e * N];
 }
-
 template <int N>
-FI void store_col_tile(float2* __restrict__ dst, const float2* tile, size_t sbase, int c0) {
-  constexpr int NT = COLS * FftCfg<N>::T, HC = COLS / 2, K = N * HC / NT;
+FI void store_cols(float2* __restrict__ dst, const float2 (&v)[FftCfg<N>::E], size_t sbase, int c0, int t, int c) {
+  float2* p = dst + sbase + (size_t)t * N + c0 + c;
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int idx = threadIdx.x + NT * k, r = idx / HC, cp = idx % HC;
-    const float2 a = tile[tslot(r, 2 * cp)], b = tile[tslot(r, 2 * cp + 1)];
-    *reinterpret_cast<float4*>(dst + sbase + (size_t)r * N + c0 + 2 * cp) = make_float4(a.x, a.y, b.x, b.y);
-  }
-}
-
-// The 16 mask bytes of each row of a column tile (one 16-byte load per row),
-// stored transposed: mskt[c * N + r].
-template <int N>
-FI void load_mask_tile(const uint8_t* __restrict__ mask, uint8_t* mskt, size_t sbase, int c0) {
-  constexpr int NT = COLS * FftCfg<N>::T;
-  for (int r = threadIdx.x; r < N; r += NT) {
-    const uint4 m = *reinterpret_cast<const uint4*>(mask + sbase + (size_t)r * N + c0);
-    const unsigned w[4] = {m.x, m.y, m.z, m.w};
-#pragma unroll
-    for (int c = 0; c < COLS; ++c) mskt[c * N + r] = (uint8_t)(w[c >> 2] >> (8 * (c & 3)));
-  }
+  for (int e = 0; e < FftCfg<N>::E; ++e) p[(size_t)FftCfg<N>::T * e * N] = v[e];
 }
 
 // In place on t: t = colIFFT(mask * colFFT(t)) for a 16-column tile.
@@ -236,42 +200,29 @@ __global__ void __launch_bounds__(512) k_col_mask(float2* __restrict__ tbuf, con
                                                   const SliceState* __restrict__ st,
                                                   const float2* __restrict__ twg) {
   using C = FftCfg<N>;
-  constexpr int E = C::E, T = C::T, LW = fft_line_words<N>();
+  constexpr int E = C::E, T = C::T;
   const int s = blockIdx.y;
   if (st != nullptr && !slice_running(st, s)) return;
   extern __shared__ __align__(16) unsigned char smem[];
   float2* tw = reinterpret_cast<float2*>(smem);
-  float2* tile = reinterpret_cast<float2*>(smem + tw_bytes<N>());
-  uint8_t* mskt = smem + tw_bytes<N>() + col_region_bytes<N>();
+  float2* buf = reinterpret_cast<float2*>(smem + tw_bytes<N>());
+  uint8_t* mskt = smem + tw_bytes<N>() + N * COLS * 8;
   const int c0 = blockIdx.x * COLS;
   const size_t sbase = (size_t)s * N * N;
-  load_twiddles<N>(tw, twg);
-  load_mask_tile<N>(mask, mskt, sbase, c0);
-  load_col_tile<N>(tbuf, tile, sbase, c0);
-  __syncthreads();
-  const int c = threadIdx.x / T, t = threadIdx.x % T;
+  const int c = threadIdx.x % COLS, t = threadIdx.x / COLS;
   float2 v[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int r = t + T * e;
-    v[e] = tile[tslot(r, c)];
-  }
+  load_cols<N>(v, tbuf, sbase, c0, t, c);
+  for (int r = threadIdx.x; r < N; r += COLS * T) cp_async16_fft(mskt + r * COLS, mask + sbase + (size_t)r * N + c0);
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  load_twiddles<N>(tw, twg);
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   __syncthreads();
-  float* bre = reinterpret_cast<float*>(tile) + c * 2 * LW;
-  float* bim = bre + LW;
-  fft_line<N, -1>(v, bre, bim, tw, t);
+  fft_col<N, -1>(v, buf, tw, t, c);
 #pragma unroll
   for (int e = 0; e < E; ++e)
-    if (!mskt[c * N + t + T * e]) v[e] = make_float2(0.f, 0.f);
-  fft_line<N, +1>(v, bre, bim, tw, t);
-  __syncthreads();
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int r = t + T * e;
-    tile[tslot(r, c)] = v[e];
-  }
-  __syncthreads();
-  store_col_tile<N>(tbuf, tile, sbase, c0);
+    if (!mskt[(t + T * e) * COLS + c]) v[e] = make_float2(0.f, 0.f);
+  fft_col<N, +1>(v, buf, tw, t, c);
+  store_cols<N>(tbuf, v, sbase, c0, t, c);
 }
 
 // atb = (1/n) colIFFT(t)  [real: imaginary part dropped]; x = atb if x != null;
@@ -282,26 +233,20 @@ __global__ void __launch_bounds__(512) k_col_inv(const float2* __restrict__ tbuf
                                                  double* __restrict__ part,
                                                  const float2* __restrict__ twg) {
   using C = FftCfg<N>;
-  constexpr int E = C::E, T = C::T, LW = fft_line_words<N>();
+  constexpr int E = C::E, T = C::T;
   const int s = blockIdx.y;
   extern __shared__ __align__(16) unsigned char smem[];
   float2* tw = reinterpret_cast<float2*>(smem);
-  float2* tile = reinterpret_cast<float2*>(smem + tw_bytes<N>());
+  float2* buf = reinterpret_cast<float2*>(smem + tw_bytes<N>());
   __shared__ double red[32];
   const int c0 = blockIdx.x * COLS;
   const size_t sbase = (size_t)s * N * N;
-  load_twiddles<N>(tw, twg);
-  load_col_tile<N>(tbuf, tile, sbase, c0);
-  __syncthreads();
-  const int c = threadIdx.x / T, t = threadIdx.x % T;
+  const int c = threadIdx.x % COLS, t = threadIdx.x / COLS;
   float2 v[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int r = t + T * e;
-    v[e] = tile[tslot(r, c)];
-  }
+  load_cols<N>(v, tbuf, sbase, c0, t, c);
+  load_twiddles<N>(tw, twg);
   __syncthreads();
-  fft_line<N, +1>(v, reinterpret_cast<float*>(tile) + c * 2 * LW, reinterpret_cast<float*>(tile) + c * 2 * LW + LW, tw, t);
+  fft_col<N, +1>(v, buf, tw, t, c);
   const float sc = 1.0f / (float)N;
   float acc = 0.f;
 #pragma unroll
@@ -309,20 +254,8 @@ __global__ void __launch_bounds__(512) k_col_inv(const float2* __restrict__ tbuf
     v[e] = make_float2(v[e].x * sc, real ? 0.f : v[e].y * sc);
     acc += cabs2(v[e]);
   }
-  __syncthreads();
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int r = t + T * e;
-    tile[tslot(r, c)] = v[e];
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < N * COLS; idx += blockDim.x) {
-    const int r = idx / COLS, cc = idx % COLS;
-    const float2 o = tile[tslot(r, cc)];
-    const size_t gi = sbase + (size_t)r * N + c0 + cc;
-    atb[gi] = o;
-    if (x) x[gi] = o;
-  }
+  store_cols<N>(atb, v, sbase, c0, t, c);
+  if (x) store_cols<N>(x, v, sbase, c0, t, c);
   const double tot = block_sum((double)acc, red);
   if (threadIdx.x == 0) part[((size_t)s * NSLOT + SLOT_RHS) * MAXPART + blockIdx.x] = tot;
 }
@@ -334,39 +267,26 @@ template <int N>
 __global__ void __launch_bounds__(512) k_col_dc(float2* __restrict__ tbuf, const float2* __restrict__ b,
                                                 const uint8_t* __restrict__ mask, const float2* __restrict__ twg) {
   using C = FftCfg<N>;
-  constexpr int E = C::E, T = C::T, LW = fft_line_words<N>();
+  constexpr int E = C::E, T = C::T;
   const int s = blockIdx.y;
   extern __shared__ __align__(16) unsigned char smem[];
   float2* tw = reinterpret_cast<float2*>(smem);
-  float2* tile = reinterpret_cast<float2*>(smem + tw_bytes<N>());
+  float2* buf = reinterpret_cast<float2*>(smem + tw_bytes<N>());
   const int c0 = blockIdx.x * COLS;
   const size_t sbase = (size_t)s * N * N;
-  load_twiddles<N>(tw, twg);
-  load_col_tile<N>(tbuf, tile, sbase, c0);
-  __syncthreads();
-  const int c = threadIdx.x / T, t = threadIdx.x % T;
+  const int c = threadIdx.x % COLS, t = threadIdx.x / COLS;
   float2 v[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int r = t + T * e;
-    v[e] = tile[tslot(r, c)];
-  }
+  load_cols<N>(v, tbuf, sbase, c0, t, c);
+  load_twiddles<N>(tw, twg);
   __syncthreads();
-  fft_line<N, -1>(v, reinterpret_cast<float*>(tile) + c * 2 * LW, reinterpret_cast<float*>(tile) + c * 2 * LW + LW, tw, t);
+  fft_col<N, -1>(v, buf, tw, t, c);
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const size_t gi = sbase + (size_t)(t + T * e) * N + c0 + c;
     if (mask[gi]) v[e] = cscale(b[gi], (float)N);
   }
-  fft_line<N, +1>(v, reinterpret_cast<float*>(tile) + c * 2 * LW, reinterpret_cast<float*>(tile) + c * 2 * LW + LW, tw, t);
-  __syncthreads();
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int r = t + T * e;
-    tile[tslot(r, c)] = v[e];
-  }
-  __syncthreads();
-  store_col_tile<N>(tbuf, tile, sbase, c0);
+  fft_col<N, +1>(v, buf, tw, t, c);
+  store_cols<N>(tbuf, v, sbase, c0, t, c);
 }
 
 // Data term of F: partial sum over sampled entries of |(1/n) colFFT(t) - b|^2,
@@ -376,26 +296,20 @@ __global__ void __launch_bounds__(512) k_col_resid(const float2* __restrict__ tb
                                                    const uint8_t* __restrict__ mask, double* __restrict__ part,
                                                    int slot, const float2* __restrict__ twg) {
   using C = FftCfg<N>;
-  constexpr int E = C::E, T = C::T, LW = fft_line_words<N>();
+  constexpr int E = C::E, T = C::T;
   const int s = blockIdx.y;
   extern __shared__ __align__(16) unsigned char smem[];
   float2* tw = reinterpret_cast<float2*>(smem);
-  float2* tile = reinterpret_cast<float2*>(smem + tw_bytes<N>());
+  float2* buf = reinterpret_cast<float2*>(smem + tw_bytes<N>());
   __shared__ double red[32];
   const int c0 = blockIdx.x * COLS;
   const size_t sbase = (size_t)s * N * N;
-  load_twiddles<N>(tw, twg);
-  load_col_tile<N>(tbuf, tile, sbase, c0);
-  __syncthreads();
-  const int c = threadIdx.x / T, t = threadIdx.x % T;
+  const int c = threadIdx.x % COLS, t = threadIdx.x / COLS;
   float2 v[E];
-#pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int r = t + T * e;
-    v[e] = tile[tslot(r, c)];
-  }
+  load_cols<N>(v, tbuf, sbase, c0, t, c);
+  load_twiddles<N>(tw, twg);
   __syncthreads();
-  fft_line<N, -1>(v, reinterpret_cast<float*>(tile) + c * 2 * LW, reinterpret_cast<float*>(tile) + c * 2 * LW + LW, tw, t);
+  fft_col<N, -1>(v, buf, tw, t, c);
   const float sc = 1.0f / (float)N;
   float acc = 0.f;
 #pragma unroll
