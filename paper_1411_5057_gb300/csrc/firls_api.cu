@@ -289,13 +289,13 @@ void enqueue_weights(firls_ctx* c, const float2* x, int precond, const SliceStat
   if (has_tv(c)) {
     // with TV, 1/a of the penta-diagonal P is also 1/diag(S) (the Jacobi scale)
     tv_weights(B, n, c->stream, view, x, c->wtv, tv2_of(c), c->channels);
-    if (c->kind) wavelet_diag(B, n, c->levels, c->stream, view, c->ww, c->wdiag, c->sqtab, c->sqlen);
+    if (c->kind) wavelet_diag(B, n, c->levels, c->kind, c->stream, view, c->ww, c->wdiag, c->sqtab, c->sqlen);
     penta_setup(B, n, c->stream, view, c->wtv, tv2_of(c), c->kind ? c->wdiag : nullptr, c->ia);
     if (uses_ilu(c, precond)) ilu_pack(B, n, c->stream, view, false, c->wtv, tv2_of(c), c->ia, c->wa, w2s_of(c));
     // ILU(0): the pivots of the incomplete factorisation replace 1/a
     if (precond == FIRLS_PRECOND_ILU0) ilu0_pivots(B, n, c->stream, c->st, view, c->wa, w2s_of(c), c->ia);
   } else if (precond == FIRLS_PRECOND_JACOBI) {
-    wavelet_diag(B, n, c->levels, c->stream, view, c->ww, c->wdiag, c->sqtab, c->sqlen);
+    wavelet_diag(B, n, c->levels, c->kind, c->stream, view, c->ww, c->wdiag, c->sqtab, c->sqlen);
     jacobi_wavelet_setup(B, n, c->stream, view, c->wdiag, c->ia);
   }
 }

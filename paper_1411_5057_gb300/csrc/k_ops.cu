@@ -377,9 +377,7 @@ static void wcl_launch(const WavArgs& a, int R, bool mirror, const float2* x, co
 
 static int coarse_smem(int m0) { return m0 * (m0 + 1) * 8; }
 
-bool wavelet_diag_prepare();
-
-// Dynamic shared-memory limits of the wavelet and pseudo-diagonal kernels,
+// Dynamic shared-memory limits of the wavelet kernels,
 // set once per device.
 static void set_wav_attrs() {
   static PerDeviceOnce once;
@@ -390,7 +388,6 @@ static void set_wav_attrs() {
     ok = cudaFuncSetAttribute(k_wav_coarse, A, coarse_smem(COARSE_LIMIT)) == cudaSuccess && ok;
     ok = wcl_prepare_haar() && ok;
     ok = wcl_prepare_db4() && ok;
-    ok = wavelet_diag_prepare() && ok;
     return ok;
   });
 }
@@ -618,101 +615,124 @@ void joint_wavelet_weights(int batch, int n, int channels, cudaStream_t s, const
 // so the diagonal is a separable sum over levels and subbands:
 //   diag(r, c) = sum_l sum_br sum_pr F_{l,br}(r - 2^l pr) T_{l,br}(pr, c),
 //   T_{l,br}(pr, c) = sum_{bands (br, bc)} sum_pc F_{l,bc}(c - 2^l pc) w_band(pr, pc),
-// indices periodic.  A CTA owns WD_RB output rows: per level it forms the
-// T rows those outputs need in shared memory (both row types), then adds
-// their row-filtered sums.  Bands at level l (h = n >> l, Mallat layout):
+// indices periodic.  Bands at level l (h = n >> l, Mallat layout):
 // (0,1) rows [0,h) cols [h,2h); (1,0) rows [h,2h) cols [0,h); (1,1) rows and
 // cols [h,2h); at the last level also (0,0), rows and cols [0,h).
-constexpr int WD_RB = 16;
-constexpr int WD_PRMAX = WD_RB / 2 + 4;  // coarse rows a level needs (filters of <= 3 * 2^l taps)
+//
+// A filter has at most TAPS 2^l taps, so an output meets TAPS coarse rows and a
+// T value TAPS coefficients per band: T_{l,br}(p, c) for p = r >> l, .. - (TAPS -
+// 1).  A thread owns WD_RB output rows of one column; per level it walks down
+// the coarse rows with the last TAPS T values of both types in registers, and
+// each fine row adds its filtered sum.  The groups of fine rows that share
+// r >> l are fixed at compile time (r0 is a multiple of 16), so only the row
+// filter's taps come from shared memory, as one float4 per type.  Bound by the
+// load/store pipe (14 weights and 8 tap vectors a pixel at four levels).  T rows
+// shared by a CTA, with taps and row indices found per term, took 690 us at 304
+// slices of 256^2; this takes 200 (weights stage as a whole: 1028 -> 536 us there,
+// 506 -> 166 at 304 x 128^2, 98 -> 45 for one slice).
+constexpr int WD_RB = 16, WD_LMAX = 9;  // n <= 512
+constexpr int WD_COLS = 64;             // threads: enough CTAs for one slice
 
-// NT, LT: side and levels fixed at compile time (0: from the arguments), so
-// that the common shape's row and column index arithmetic is shifts and masks.
-template <int NT, int LT>
-__global__ void __launch_bounds__(256) k_wavelet_diag(int n_arg, int levels_arg, const SliceState* __restrict__ st,
-                                                      const float* __restrict__ w, float* __restrict__ out,
-                                                      const float* __restrict__ sqtab,
-                                                      const int* __restrict__ sqlen) {
-  const int s = blockIdx.y;
+template <int TAPS, int LG>  // 2^LG fine rows of the 16 share a coarse row
+FI void wd_level(float (&acc)[WD_RB], int n, int l, bool last, int r0, int c, const float* __restrict__ ws,
+                 const float* __restrict__ F0, const float* __restrict__ F1, int len0, int len1,
+                 const float4 (*fr)[WD_RB]) {
+  constexpr int G = 1 << LG, NP = WD_RB >> LG;
+  const int h = n >> l, p0 = r0 >> l, cq = c >> l, phase = c & ((1 << l) - 1);
+  float f0[TAPS], f1[TAPS];
+  int q[TAPS];
+#pragma unroll
+  for (int i = 0; i < TAPS; ++i) {
+    const int sc = phase + (i << l);
+    f0[i] = sc < len0 ? F0[sc] : 0.f;
+    f1[i] = sc < len1 ? F1[sc] : 0.f;
+    q[i] = ((cq - i) % h + h) % h;
+  }
+  float t0[TAPS] = {}, t1[TAPS] = {};  // [i]: T of coarse row p - i, types 0 and 1
+#pragma unroll
+  for (int pp = 1 - TAPS; pp < NP; ++pp) {
+#pragma unroll
+    for (int i = TAPS - 1; i > 0; --i) {
+      t0[i] = t0[i - 1];
+      t1[i] = t1[i - 1];
+    }
+    const float* wl = ws + (size_t)(((p0 + pp) % h + h) % h) * n;  // row of type 0
+    const float* wh = wl + (size_t)h * n;
+    float a = 0.f, b = 0.f;
+    if (last) {
+#pragma unroll
+      for (int i = 0; i < TAPS; ++i) a = fmaf(f0[i], wl[q[i]], a);
+    }
+#pragma unroll
+    for (int i = 0; i < TAPS; ++i) a = fmaf(f1[i], wl[h + q[i]], a);
+#pragma unroll
+    for (int i = 0; i < TAPS; ++i) b = fmaf(f0[i], wh[q[i]], b);
+#pragma unroll
+    for (int i = 0; i < TAPS; ++i) b = fmaf(f1[i], wh[h + q[i]], b);
+    t0[0] = a;
+    t1[0] = b;
+    if (pp < 0) continue;
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      const float4 u = fr[0][k], v = fr[1][k];
+      const float uu[3] = {u.x, u.y, u.z}, vv[3] = {v.x, v.y, v.z};
+      float o = acc[pp * G + k];
+#pragma unroll
+      for (int i = 0; i < TAPS; ++i) o = fmaf(uu[i], t0[i], o);
+#pragma unroll
+      for (int i = 0; i < TAPS; ++i) o = fmaf(vv[i], t1[i], o);
+      acc[pp * G + k] = o;
+    }
+  }
+}
+
+template <int TAPS>
+__global__ void __launch_bounds__(WD_COLS, 10) k_wavelet_diag(int n, int levels, const SliceState* __restrict__ st,
+                                                          const float* __restrict__ w, float* __restrict__ out,
+                                                          const float* __restrict__ sqtab,
+                                                          const int* __restrict__ sqlen) {
+  const int s = blockIdx.z;
   if (!slice_running(st, s)) return;
-  const int n = NT ? NT : n_arg, levels = LT ? LT : levels_arg;
-  extern __shared__ __align__(16) float tsm[];  // [2][WD_PRMAX][n]
-  const int r0 = blockIdx.x * WD_RB;
-  const int rows = min(WD_RB, n - r0);
+  const int r0 = blockIdx.y * WD_RB;
+  // fr[l - 1][type][k]: the taps that meet fine row r0 + k (those of its phase)
+  __shared__ float4 fr[WD_LMAX][2][WD_RB];
+  for (int i = threadIdx.x; i < levels * 2 * WD_RB; i += WD_COLS) {
+    const int k = i % WD_RB, type = i / WD_RB % 2, l = i / (2 * WD_RB) + 1;
+    const int phase = (r0 + k) & ((1 << l) - 1), len = sqlen[(l - 1) * 2 + type];
+    const float* F = sqtab + (size_t)((l - 1) * 2 + type) * n;
+    float f[3];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const int sr = phase + (t << l);
+      f[t] = sr < len ? F[sr] : 0.f;
+    }
+    fr[l - 1][type][k] = make_float4(f[0], f[1], f[2], 0.f);
+  }
+  __syncthreads();
+  const int c = blockIdx.x * WD_COLS + threadIdx.x;
+  if (c >= n) return;
   const size_t base = (size_t)s * n * n;
-  const float* ws = w + base;
-  constexpr int PER = WD_RB * 512 / 256;  // outputs per thread, n <= 512
-  float acc[PER];
+  float acc[WD_RB];
 #pragma unroll
-  for (int k = 0; k < PER; ++k) acc[k] = 0.f;
-#pragma unroll
-  for (int l = 1; l <= levels; ++l) {  // a constant trip count (unrolled) for LT > 0
-    const int h = n >> l, step = 1 << l, msk = step - 1;
-    const int len[2] = {sqlen[(l - 1) * 2], sqlen[(l - 1) * 2 + 1]};
-    const float* F[2] = {sqtab + (size_t)((l - 1) * 2) * n, sqtab + (size_t)((l - 1) * 2 + 1) * n};
-    const int lmax = len[0] > len[1] ? len[0] : len[1];
-    // coarse rows pr = pr_lo + j (mod h), j < cnt, cover every r - sr with sr < lmax
-    const int pr_lo = (r0 - (lmax - 1) - (step - 1)) >> l;  // floor division (arithmetic shift)
-    int cnt = ((r0 + rows - 1) >> l) - pr_lo + 1;
-    if (cnt > WD_PRMAX) cnt = WD_PRMAX;
-    const int pr0 = ((pr_lo % h) + h) % h;
-    __syncthreads();  // the previous level's T rows are no longer read
-    for (int idx = threadIdx.x; idx < 2 * cnt * n; idx += blockDim.x) {
-      const int br = idx / (cnt * n), j = (idx / n) % cnt, c = idx % n;
-      const int pr = (pr0 + j) % h;
-      float t = 0.f;
-      for (int bc = 0; bc < 2; ++bc) {
-        if (br == 0 && bc == 0 && l != levels) continue;  // LL is a band only at the last level
-        const float* wrow = ws + (size_t)(br * h + pr) * n + bc * h;
-        const float* fc = F[bc];
-        for (int sc = c & msk; sc < len[bc]; sc += step) {
-          int pc = c - sc;
-          if (pc < 0) pc += n;
-          t = fmaf(fc[sc], wrow[pc >> l], t);
-        }
-      }
-      tsm[(size_t)(br * WD_PRMAX + j) * n + c] = t;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int idx = threadIdx.x + 256 * k;
-      if (idx < rows * n) {
-        const int r = r0 + idx / n, c = idx % n;
-        float a = acc[k];
-        for (int br = 0; br < 2; ++br) {
-          const float* fr = F[br];
-          for (int sr = r & msk; sr < len[br]; sr += step) {
-            int pr = r - sr;
-            if (pr < 0) pr += n;
-            const int j = (((pr >> l) - pr0) % h + h) % h;
-            a = fmaf(fr[sr], tsm[(size_t)(br * WD_PRMAX + j) * n + c], a);
-          }
-        }
-        acc[k] = a;
-      }
-    }
+  for (int k = 0; k < WD_RB; ++k) acc[k] = 0.f;
+  for (int l = 1; l <= levels; ++l) {
+    const float* F0 = sqtab + (size_t)(l - 1) * 2 * n;
+    const int len0 = sqlen[(l - 1) * 2], len1 = sqlen[(l - 1) * 2 + 1];
+    const bool last = l == levels;
+    if (l == 1) wd_level<TAPS, 1>(acc, n, l, last, r0, c, w + base, F0, F0 + n, len0, len1, fr[l - 1]);
+    else if (l == 2) wd_level<TAPS, 2>(acc, n, l, last, r0, c, w + base, F0, F0 + n, len0, len1, fr[l - 1]);
+    else if (l == 3) wd_level<TAPS, 3>(acc, n, l, last, r0, c, w + base, F0, F0 + n, len0, len1, fr[l - 1]);
+    else wd_level<TAPS, 4>(acc, n, l, last, r0, c, w + base, F0, F0 + n, len0, len1, fr[l - 1]);
   }
 #pragma unroll
-  for (int k = 0; k < PER; ++k) {
-    const int idx = threadIdx.x + 256 * k;
-    if (idx < rows * n) out[base + (size_t)(r0 + idx / n) * n + idx % n] = acc[k];
-  }
+  for (int k = 0; k < WD_RB; ++k) out[base + (size_t)(r0 + k) * n + c] = acc[k];
 }
 
-bool wavelet_diag_prepare() {
-  const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  bool ok = cudaFuncSetAttribute(k_wavelet_diag<0, 0>, A, 2 * WD_PRMAX * 512 * 4) == cudaSuccess;
-  return cudaFuncSetAttribute(k_wavelet_diag<256, 4>, A, 2 * WD_PRMAX * 256 * 4) == cudaSuccess && ok;
-}
-
-void wavelet_diag(int batch, int n, int levels, cudaStream_t s, const SliceState* st, const float* w,
+void wavelet_diag(int batch, int n, int levels, int kind, cudaStream_t s, const SliceState* st, const float* w,
                   float* out, const float* sqtab, const int* sqlen) {
-  const dim3 grid((n + WD_RB - 1) / WD_RB, batch);
-  if (n == 256 && levels == 4)
-    k_wavelet_diag<256, 4><<<grid, 256, 2 * WD_PRMAX * n * 4, s>>>(n, levels, st, w, out, sqtab, sqlen);
-  else
-    k_wavelet_diag<0, 0><<<grid, 256, 2 * WD_PRMAX * n * 4, s>>>(n, levels, st, w, out, sqtab, sqlen);
+  const dim3 grid((n + WD_COLS - 1) / WD_COLS, n / WD_RB, batch);  // n % 16 = 0 for every size
+  if (kind == 2) k_wavelet_diag<3><<<grid, WD_COLS, 0, s>>>(n, levels, st, w, out, sqtab, sqlen);
+  else k_wavelet_diag<1><<<grid, WD_COLS, 0, s>>>(n, levels, st, w, out, sqtab, sqlen);
 }
 
 // P = abar I + lam_tv (D1^T W1 D1 + D2^T W2 D2) [+ lam diag(Phi^T W Phi)]

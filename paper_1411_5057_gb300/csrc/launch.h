@@ -91,7 +91,7 @@ void tv_weights(int batch, int n, cudaStream_t s, const SliceState* st, const fl
 // ww = (sum over the C contrasts of |c_j|^2 + eps)^(-1/2) for every contrast.
 void joint_wavelet_weights(int batch, int n, int channels, cudaStream_t s, const SliceState* st, const float2* cw,
                            float* ww);
-void wavelet_diag(int batch, int n, int levels, cudaStream_t s, const SliceState* st, const float* w,
+void wavelet_diag(int batch, int n, int levels, int kind, cudaStream_t s, const SliceState* st, const float* w,
                   float* out, const float* sqtab, const int* sqlen);
 void penta_setup(int batch, int n, cudaStream_t s, const SliceState* st, const float* wtv, const float* wtv2,
                  const float* wdiag, float* ia);
