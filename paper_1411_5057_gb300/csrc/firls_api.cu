@@ -243,8 +243,10 @@ bool uses_ilu(const firls_ctx* c, int precond) {
 // q = S d  (mode 0: d = z; 1: d = z + beta d; 2: d as given; -1: per slice,
 // d = x^k for a slice starting its outer step, else z or z + beta d); skew: z
 // and q in the ILU's layout
-void enqueue_S(firls_ctx* c, int mode, const float2* zin, float2* din, float2* q, bool skew) {
+void enqueue_S(firls_ctx* c, int mode, const float2* zin, float2* din, float2* q, bool skew,
+               bool chained = false) {
   FftArgs a = fft_args(c);
+  a.chained = chained;
   a.skew = skew ? 1 : 0;
   a.atb = c->atb;
   a.z = zin;
@@ -258,6 +260,7 @@ void enqueue_S(firls_ctx* c, int mode, const float2* zin, float2* din, float2* q
   { TMark m(c, FIRLS_K_COL_FFT_MASK, 1); fft_col_mask(c->n, a); }
   if (c->kind) {
     WavArgs w = wav_args(c, c->st);
+    w.chained = chained;
     TMark m(c, FIRLS_K_WAVELET_S, wavelet_apply_launches(c->n, c->levels, c->kind, c->tune_rb, c->tune_cmax));
     wavelet_apply(w, din, c->cw, c->ww, WAV_MUL_W, c->u, nullptr, a.real);
   }
@@ -310,10 +313,19 @@ bool alpha_in_ilu(const firls_ctx* c, const firls_params& sc) {
   return uses_ilu(c, sc.precond) && c->channels == 1;
 }
 
+// Whether a lone context's macro steps chain their launches (launch_chained): up
+// to 2^16 pixels, where the grids leave the SMs room.  20 PCG steps, Haar: 64^2
+// 1 slice 617 -> 566 us, 16 676 -> 650, 64 slices 725 -> 754; 128^2 4 slices 824
+// -> 770, 16 854 -> 878; 256^2 1 slice 980 -> 925, 4 1015 -> 1034.  With TV 0 to 3 %
+// below the line; far above it the waiting CTAs hold the room of the kernel
+// before them (304 slices of 256^2: 16.5 -> 18.1 ms), and beside other contexts
+// they do at any size.
+bool chains(const firls_ctx* c) { return (size_t)c->batch * c->n * c->n <= (1u << 16); }
+
 // Residual update and z = P^{-1} r, then rho (first residual) or beta and the
 // PCG stop.  mode ILU_INIT: the first residual r = A^H b - q for every
 // running slice; ILU_PER_SLICE: each slice by its phase.  x updates go to dx.
-void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc) {
+void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc, bool chained = false) {
   const int B = run_batch(c), n = c->n;
   const int real = (c->flags & FIRLS_REAL_X) ? 1 : 0;
   const bool init = mode == ILU_INIT;
@@ -324,10 +336,10 @@ void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc) {
     {
       TMark m(c, FIRLS_K_AXPY, 1);
       axpy_diag_step(B, n, c->stream, c->st, c->part, am, c->r, c->q, c->atb,
-                     sc.precond == FIRLS_PRECOND_JACOBI ? c->ia : nullptr, c->z);
+                     sc.precond == FIRLS_PRECOND_JACOBI ? c->ia : nullptr, c->z, chained);
     }
     TMark m(c, FIRLS_K_SCALARS, 1);
-    pcg_scalars(B, c->stream, c->st, c->part, axpy_ctas(n), axpy_ctas(n), sm, ps, c->channels);
+    pcg_scalars(B, c->stream, c->st, c->part, axpy_ctas(n), axpy_ctas(n), sm, ps, c->channels, chained);
     return;
   }
   if (has_tv(c)) {
@@ -341,26 +353,27 @@ void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc) {
       const int shape = (c->tune_ilu && B == c->batch) ? c->tune_ilu : 0;
       const int alpha_np = (mode == ILU_PER_SLICE && alpha_in_ilu(c, sc)) ? fft_row_ctas(n) : 0;
       ilu_step(B, n, c->stream, c->st, c->part, mode, c->r, c->q, c->u, c->z, c->wa, w2s_of(c), shape,
-               fuse ? 1 : 0, ps, c->wait_test, alpha_np);
+               fuse ? 1 : 0, ps, c->wait_test, alpha_np, chained);
     }
     if (!fuse) {
       TMark m(c, FIRLS_K_SCALARS, 1);
-      pcg_scalars(B, c->stream, c->st, c->part, 1, 1, sm, ps, c->channels);
+      pcg_scalars(B, c->stream, c->st, c->part, 1, 1, sm, ps, c->channels, chained);
     }
     return;
   }
   {
     TMark m(c, FIRLS_K_AXPY, 1);
-    axpy_step(B, n, c->stream, c->st, c->part, am, c->r, c->q, c->atb);
+    axpy_step(B, n, c->stream, c->st, c->part, am, c->r, c->q, c->atb, chained);
   }
   WavArgs w = wav_args(c, c->st);
+  w.chained = chained;
   {
     TMark m(c, FIRLS_K_WAVELET_P, wavelet_apply_launches(n, c->levels, c->kind, c->tune_rb, c->tune_cmax));
     wavelet_apply(w, c->r, c->cw, c->ww, WAV_MUL_PINV, c->z, c->r, real);
   }
   TMark m(c, FIRLS_K_SCALARS, 1);
   const int np = wavelet_apply_ctas(n, c->levels, c->kind, c->tune_rb, c->tune_cmax);
-  pcg_scalars(B, c->stream, c->st, c->part, np, axpy_ctas(n), sm, ps, c->channels);
+  pcg_scalars(B, c->stream, c->st, c->part, np, axpy_ctas(n), sm, ps, c->channels, chained);
 }
 
 // The end of every outer step whose PCG has stopped: x += dx, the relative
@@ -383,7 +396,7 @@ void enqueue_outer_end(firls_ctx* c, const firls_params& sc) {
 // boundary stage in every macro step, an outer step with J PCG steps spans
 // J + 1 macro steps; with one every P macro steps a slice waits at most
 // P - 1 macro steps per outer step.
-void enqueue_macro(firls_ctx* c, const firls_params& sc, bool boundary_stage = true) {
+void enqueue_macro(firls_ctx* c, const firls_params& sc, bool boundary_stage = true, bool chained = false) {
   const int B = run_batch(c), n = c->n;
   if (boundary_stage) {
     {
@@ -393,12 +406,12 @@ void enqueue_macro(firls_ctx* c, const firls_params& sc, bool boundary_stage = t
     }
     enqueue_weights(c, c->x, sc.precond, c->stw);
   }
-  enqueue_S(c, -1, c->z, c->d, c->q, uses_ilu(c, sc.precond));
+  enqueue_S(c, -1, c->z, c->d, c->q, uses_ilu(c, sc.precond), chained);
   if (!alpha_in_ilu(c, sc)) {
     TMark m(c, FIRLS_K_SCALARS, 1);
-    pcg_alpha(B, c->stream, c->st, c->part, fft_row_ctas(n), c->channels);
+    pcg_alpha(B, c->stream, c->st, c->part, fft_row_ctas(n), c->channels, chained);
   }
-  enqueue_precond(c, ILU_PER_SLICE, sc);
+  enqueue_precond(c, ILU_PER_SLICE, sc, chained);
 }
 
 int period_of(const firls_params& sc) { return sc.boundary_period > 1 ? sc.boundary_period : 1; }
@@ -516,7 +529,7 @@ firls_status macro_graph(firls_ctx* c, const firls_params& sc, int steps, cudaGr
   if (c->timing) marks_reset(c);
   cudaGraph_t g = nullptr;
   CU(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-  for (int i = 0; i < steps; ++i) enqueue_macro(c, sc, i % period_of(sc) == 0);
+  for (int i = 0; i < steps; ++i) enqueue_macro(c, sc, i % period_of(sc) == 0, chains(c));
   cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   if (e != cudaSuccess) return cuda_check(c, e, "graph capture");
   cudaGraphExec_t ex = nullptr;
@@ -553,7 +566,7 @@ firls_status run_macro(firls_ctx* c, const firls_params& sc, long total, int chu
     if (t) marks_reset(c);
     for (long k = 0; k < total; ++k) {
       if (k == chunk) c->timing = false;
-      enqueue_macro(c, sc, k % period_of(sc) == 0);
+      enqueue_macro(c, sc, k % period_of(sc) == 0, chains(c));
     }
     c->timing = t;
     c->marks_valid = t;

@@ -71,6 +71,14 @@ FI float2 cmul(float2 a, float2 b) {
 FI float cabs2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
 FI float rdot2(float2 a, float2 b) { return fmaf(a.x, b.x, a.y * b.y); }
 
+// First statement of a kernel that launch_chained starts: returns when the kernel
+// before it in the stream has completed and its writes are visible (at once
+// after a plain launch), then lets the next kernel's CTAs take the room that this
+// one leaves.
+FI void chained_start() {
+  asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
 FI bool slice_running(const SliceState* st, int s) { return st[s].active && !st[s].done; }
 FI bool slice_in_pcg(const SliceState* st, int s) { return slice_running(st, s) && st[s].phase == PH_PCG; }
 // A slice that takes part in this macro step's S apply and PCG update.

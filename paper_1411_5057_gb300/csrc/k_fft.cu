@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(256) k_row_fwd(const float2* __restrict__ z, f
                                                  const SliceState* __restrict__ st,
                                                  const float2* __restrict__ twg, int mode_arg,
                                                  const float2* __restrict__ x, float2* __restrict__ dx) {
+  chained_start();
   using C = FftCfg<N>;
   constexpr int R = rows_per_cta<N>(), E = C::E, T = C::T, LW = fft_line_words<N>();
   const int s = blockIdx.y;
@@ -199,6 +200,7 @@ template <int N>
 __global__ void __launch_bounds__(512) k_col_mask(float2* __restrict__ tbuf, const uint8_t* __restrict__ mask,
                                                   const SliceState* __restrict__ st,
                                                   const float2* __restrict__ twg) {
+  chained_start();
   using C = FftCfg<N>;
   constexpr int E = C::E, T = C::T;
   const int s = blockIdx.y;
@@ -334,6 +336,7 @@ __global__ void __launch_bounds__(256) k_row_inv(const float2* __restrict__ tbuf
                                                  double* __restrict__ part, int real,
                                                  const float2* __restrict__ twg, const float* __restrict__ wtv2,
                                                  const float2* __restrict__ atb) {
+  chained_start();
   using C = FftCfg<N>;
   constexpr int R = rows_per_cta<N>(), E = C::E, T = C::T, LW = fft_line_words<N>();
   const int s = blockIdx.y;
@@ -475,8 +478,8 @@ template <int N> struct FftLaunch {
   }
   static void col_mask(const FftArgs& a) {
     set_smem_attrs<N>();
-    k_col_mask<N><<<dim3(N / COLS, a.batch), COLS * FftCfg<N>::T, col_smem_bytes<N>(), a.stream>>>(
-        a.t, a.mask, a.st, a.tw);
+    launch_chained(a.chained, k_col_mask<N>, dim3(N / COLS, a.batch), dim3(COLS * FftCfg<N>::T), col_smem_bytes<N>(), a.stream,
+                   a.t, a.mask, a.st, a.tw);
   }
   static void col_inv(const FftArgs& a) {
     set_smem_attrs<N>();
@@ -496,8 +499,9 @@ template <int N> struct FftLaunch {
   static void row_inv(const FftArgs& a) {
     set_smem_attrs<N>();
     const auto k = a.skew ? k_row_inv<N, true> : k_row_inv<N, false>;
-    k<<<dim3(N / R, a.batch), R * FftCfg<N>::T, row_smem_bytes<N>(a.wtv != nullptr, a.wtv2 != nullptr),
-        a.stream>>>(a.t, a.d, a.u, a.wtv, a.q, a.st, a.part, a.real, a.tw, a.wtv2, a.atb);
+    launch_chained(a.chained, k, dim3(N / R, a.batch), dim3(R * FftCfg<N>::T),
+                   row_smem_bytes<N>(a.wtv != nullptr, a.wtv2 != nullptr), a.stream, a.t, a.d, a.u, a.wtv, a.q, a.st,
+                   a.part, a.real, a.tw, a.wtv2, a.atb);
   }
 };
 

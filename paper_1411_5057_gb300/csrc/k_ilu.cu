@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
           const float4* __restrict__ q_all, float4* y_all, float4* __restrict__ z_all,
           const float4* __restrict__ wa_all, const float2* __restrict__ w2_all, int fuse, PcgSched ps,
           int wait_test, int alpha_np) {
+  chained_start();
   const int s = blockIdx.x;
   if (!slice_running(st, s)) return;
   const int t = threadIdx.x, lane = t & 31, b = t >> 5;
@@ -506,7 +507,7 @@ bool ilu_shape_fits(int n, int shape, bool aniso) {
 
 void ilu_step(int batch, int n, cudaStream_t s, SliceState* st, double* part, int mode, float2* r, const float2* q,
               float2* y, float2* z, const float4* wa, const float2* w2s, int shape, int fuse_scalars, PcgSched ps,
-              int wait_test, int alpha_np) {
+              int wait_test, int alpha_np, bool chained) {
   if (shape <= 0) shape = ilu_default_shape(batch);
   const bool deep = shape / 10 == 4;
   // r, q, y, z and the weights: 40 bytes a pixel against an L2 of 129 MB.  304
@@ -515,8 +516,8 @@ void ilu_step(int batch, int n, cudaStream_t s, SliceState* st, double* part, in
   const bool far = 40.0 * n * n * batch > 100e6;
   const IluKernel k = w2s ? ilu_kernel<true>(n, deep, far) : ilu_kernel<false>(n, deep, far);
   auto f4 = [](float2* p) { return reinterpret_cast<float4*>(p); };
-  k<<<batch, 32 * wv_bands(n), wv_rows_bytes(n), s>>>(n, mode, st, part, f4(r), reinterpret_cast<const float4*>(q),
-                                                      f4(y), f4(z), wa, w2s, fuse_scalars, ps, wait_test, alpha_np);
+  launch_chained(chained, k, dim3(batch), dim3(32 * wv_bands(n)), wv_rows_bytes(n), s, n, mode, st, part, f4(r),
+                 reinterpret_cast<const float4*>(q), f4(y), f4(z), wa, w2s, fuse_scalars, ps, wait_test, alpha_np);
 }
 
 void ilu_pack(int batch, int n, cudaStream_t s, const SliceState* st, bool all, const float* wtv,

@@ -370,7 +370,7 @@ static void wcl_launch(const WavArgs& a, int R, bool mirror, const float2* x, co
                        const float2* r, int real) {
   const WclArgs c{x,    u,    w,       a.levels,
                   mode, mirror ? 1 : 0, r, r ? a.part : nullptr,
-                  real, const_cast<SliceState*>(a.st), a.batch, a.stream};
+                  real, const_cast<SliceState*>(a.st), a.batch, a.stream, a.chained};
   if (a.kind == 2) wcl_launch_db4(a.n, R, c);
   else wcl_launch_haar(a.n, R, c);
 }
@@ -782,6 +782,7 @@ int axpy_ctas(int n) {
 
 __global__ void k_axpy(int N, int mode_arg, const SliceState* __restrict__ st, double* __restrict__ part,
                        float2* r, const float2* __restrict__ q, const float2* atb) {
+  chained_start();
   const int s = blockIdx.y;
   if (!slice_running(st, s)) return;
   const int ph = st[s].phase;
@@ -820,8 +821,8 @@ __global__ void k_axpy(int N, int mode_arg, const SliceState* __restrict__ st, d
 }
 
 void axpy_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* r,
-               const float2* q, const float2* atb) {
-  k_axpy<<<dim3(axpy_ctas(n), batch), 256, 0, s>>>(n * n, mode, st, part, r, q, atb);
+               const float2* q, const float2* atb, bool chained) {
+  launch_chained(chained, k_axpy, dim3(axpy_ctas(n), batch), dim3(256), 0, s, n * n, mode, st, part, r, q, atb);
 }
 
 // Residual update with a diagonal preconditioner (Jacobi PCG, sdiag = 1 /
@@ -829,6 +830,7 @@ void axpy_step(int batch, int n, cudaStream_t s, const SliceState* st, double* p
 __global__ void k_axpy_diag(int N, int mode_arg, const SliceState* __restrict__ st, double* __restrict__ part,
                             float2* __restrict__ r, const float2* __restrict__ q, const float2* __restrict__ atb,
                             const float* __restrict__ sdiag, float2* __restrict__ z) {
+  chained_start();
   const int s = blockIdx.y;
   if (!slice_running(st, s)) return;
   const int ph = st[s].phase;
@@ -860,8 +862,8 @@ __global__ void k_axpy_diag(int N, int mode_arg, const SliceState* __restrict__ 
 }
 
 void axpy_diag_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* r,
-                    const float2* q, const float2* atb, const float* sdiag, float2* z) {
-  k_axpy_diag<<<dim3(axpy_ctas(n), batch), 256, 0, s>>>(n * n, mode, st, part, r, q, atb, sdiag, z);
+                    const float2* q, const float2* atb, const float* sdiag, float2* z, bool chained) {
+  launch_chained(chained, k_axpy_diag, dim3(axpy_ctas(n), batch), dim3(256), 0, s, n * n, mode, st, part, r, q, atb, sdiag, z);
 }
 
 __global__ void k_jacobi_wavelet(int N, const SliceState* __restrict__ st, const float* __restrict__ wdiag,
@@ -1292,14 +1294,15 @@ void boundary_view(int batch, cudaStream_t s, SliceState* st, SliceState* view) 
 }
 
 __global__ void k_alpha(int B, SliceState* st, const double* part, int np, int C) {
+  chained_start();
   const int s = sc_slice();
   if (s >= B || !slice_in_pcg(st, s)) return;
   const double dq = image_parts(part, s, SLOT_DQ, np, C);
   if ((threadIdx.x & 31) == 0) pcg_alpha_from(st + s, dq);
 }
 
-void pcg_alpha(int batch, cudaStream_t s, SliceState* st, const double* part, int np, int channels) {
-  k_alpha<<<sc_ctas(batch), 32 * SC_WARPS, 0, s>>>(batch, st, part, np, channels);
+void pcg_alpha(int batch, cudaStream_t s, SliceState* st, const double* part, int np, int channels, bool chained) {
+  launch_chained(chained, k_alpha, dim3(sc_ctas(batch)), dim3(32 * SC_WARPS), 0, s, batch, st, part, np, channels);
 }
 
 // After z = P^{-1} r: rho (first residual, slices at the start of an outer
@@ -1307,6 +1310,7 @@ void pcg_alpha(int batch, cudaStream_t s, SliceState* st, const double* part, in
 // of them for every running slice.
 __global__ void k_pcg_scalars(int B, SliceState* st, const double* part, int np_rz, int np_rr, int mode,
                               PcgSched ps, int C) {
+  chained_start();
   const int s = sc_slice();
   if (s >= B || !slice_running(st, s) || st[s].fault) return;
   const int ph = st[s].phase;
@@ -1321,8 +1325,9 @@ __global__ void k_pcg_scalars(int B, SliceState* st, const double* part, int np_
 }
 
 void pcg_scalars(int batch, cudaStream_t s, SliceState* st, const double* part, int np_rz, int np_rr, int mode,
-                 const PcgSched& ps, int channels) {
-  k_pcg_scalars<<<sc_ctas(batch), 32 * SC_WARPS, 0, s>>>(batch, st, part, np_rz, np_rr, mode, ps, channels);
+                 const PcgSched& ps, int channels, bool chained) {
+  launch_chained(chained, k_pcg_scalars, dim3(sc_ctas(batch)), dim3(32 * SC_WARPS), 0, s, batch, st, part, np_rz, np_rr, mode, ps,
+                 channels);
 }
 
 // Outer-loop stop.  kind 0: relative change <= tol.  kind 1: estimated

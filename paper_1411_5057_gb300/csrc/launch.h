@@ -8,6 +8,30 @@
 
 namespace firls {
 
+// Launch, if chained with a programmatic dependency on the kernel before it in the
+// stream: the CTAs are set up while that one drains and wait in chained_start, which
+// every kernel launched so calls first, in every thread.  For the short kernels
+// of a macro step on little data (chains() in firls_api.cu has the figures).
+template <typename... P, typename... A>
+inline void launch_chained(bool chained, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                           A... args) {
+  if (!chained) {
+    k<<<grid, block, smem, s>>>(static_cast<P>(args)...);
+    return;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);  // a failure stays with cudaGetLastError
+}
+
 struct FftArgs {
   int batch = 0;
   cudaStream_t stream = 0;
@@ -32,6 +56,7 @@ struct FftArgs {
   float2* dx = nullptr;         // row FFT: dx += alpha d of the PCG step before
   int mode = 0;
   int real = 0;
+  bool chained = false;  // column mask and row IFFT: launch_chained
 };
 
 bool fft_size_supported(int n);
@@ -60,6 +85,7 @@ struct WavArgs {
   double* part = nullptr;
   int rb = 0;          // rows per CTA of the tiled levels (0: default 8)
   int coarse_max = 0;  // largest side kept in shared memory (0: default 64)
+  bool chained = false;  // the one-launch form: launch_chained
 };
 // c = Phi x (Mallat, stride n) with the final store scaled per `mode`:
 // RAW: c; MUL_W: w*c; MUL_PINV: c / (abar + lam w); SINGLETON_W: writes
@@ -121,7 +147,8 @@ enum IluMode { ILU_INIT = 0, ILU_STEP = 1, ILU_PER_SLICE = -1 };
 // from the S apply's alpha_np partial sums of <d, S d> (pcg_alpha's work)
 void ilu_step(int batch, int n, cudaStream_t s, SliceState* st, double* part, int mode, float2* r, const float2* q,
               float2* y, float2* z, const float4* wa, const float2* w2s, int shape, int fuse_scalars = 0,
-              PcgSched ps = PcgSched{0.f, 0, 1 << 30, 0, 0}, int wait_test = 0, int alpha_np = 0);
+              PcgSched ps = PcgSched{0.f, 0, 1 << 30, 0, 0}, int wait_test = 0, int alpha_np = 0,
+              bool chained = false);
 int ilu_default_shape(int batch);
 bool ilu_shape_fits(int n, int shape, bool aniso = false);
 
@@ -132,11 +159,11 @@ enum AxpyMode { AXPY_INIT = 0, AXPY_STEP = 1, AXPY_PER_SLICE = -1 };
 // Residual update (INIT: r = A^H b - q; STEP: r -= alpha q) with a diagonal preconditioner z = sdiag o r (sdiag null: z = r), partial
 // Re<r, z> into SLOT_RZ and ||r||^2 into SLOT_RR (axpy_ctas parts).
 void axpy_diag_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* r,
-                    const float2* q, const float2* atb, const float* sdiag, float2* z);
+                    const float2* q, const float2* atb, const float* sdiag, float2* z, bool chained = false);
 // Jacobi scale of a wavelet-only system: ia = 1 / (abar + lam diag(Phi^T W Phi)).
 void jacobi_wavelet_setup(int batch, int n, cudaStream_t s, const SliceState* st, const float* wdiag, float* ia);
 void axpy_step(int batch, int n, cudaStream_t s, const SliceState* st, double* part, int mode, float2* r,
-               const float2* q, const float2* atb);
+               const float2* q, const float2* atb, bool chained = false);
 int axpy_ctas(int n);
 
 void group_norms(int batch, int n, int n_groups, cudaStream_t s, const SliceState* st,
@@ -170,10 +197,11 @@ void guard_pick(int batch, int n, cudaStream_t s, const double* f1, const double
 // products are summed over the C consecutive slices of a multi-contrast
 // image, whose slices then carry the same scalars (here, in outer_end and in
 // state_init's ||A^H b||^2).
-void pcg_alpha(int batch, cudaStream_t s, SliceState* st, const double* part, int nparts, int channels = 1);
+void pcg_alpha(int batch, cudaStream_t s, SliceState* st, const double* part, int nparts, int channels = 1,
+               bool chained = false);
 enum ScalarsMode { SCALARS_INIT = 0, SCALARS_STEP = 1, SCALARS_PER_SLICE = -1 };
 void pcg_scalars(int batch, cudaStream_t s, SliceState* st, const double* part, int nparts_rz, int nparts_rr,
-                 int mode, const PcgSched& ps, int channels = 1);
+                 int mode, const PcgSched& ps, int channels = 1, bool chained = false);
 // view = st with every slice not at the start of its outer step marked done
 // (and the slices whose outer step is due move to PH_START)
 void boundary_view(int batch, cudaStream_t s, SliceState* st, SliceState* view);

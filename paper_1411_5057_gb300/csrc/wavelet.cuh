@@ -375,6 +375,7 @@ template <int NT, int RT, int LT, int KT, int TH>
 __global__ void __launch_bounds__(TH, NT <= 256 ? 2 : 1)
 k_wav_cluster(const float2* x, float2* u, const float* __restrict__ w, int L_arg, int mode, int mirror, 
               const float2* __restrict__ r, double* __restrict__ part, int real, SliceState* __restrict__ st) {
+  chained_start();
   const int s = blockIdx.y;
   // the same slice for every CTA of the cluster: all of them leave or none
   if (st != nullptr && !slice_running(st, s)) return;
@@ -496,6 +497,7 @@ struct WclArgs {
   SliceState* st;
   int batch;
   cudaStream_t stream;
+  bool chained;
 };
 
 template <int N, int R, int TH>
@@ -516,8 +518,13 @@ inline void wcl_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int lev
 
 template <int N, int R, int L, int KT, int TH> bool wcl_launch_as(const WclArgs& a) {
   cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   wcl_config<N, R, TH>(cfg, at, a.levels, a.mirror, a.batch, a.stream);
+  if (a.chained) {
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+  }
   return cudaLaunchKernelEx(&cfg, k_wav_cluster<N, R, L, KT, TH>, a.x, a.u, a.w, a.levels, a.mode, a.mirror, a.r,
                             a.part, a.real, a.st) == cudaSuccess;
 }
