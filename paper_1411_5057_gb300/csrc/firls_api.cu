@@ -361,19 +361,25 @@ void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc, bool chaine
     }
     return;
   }
-  {
+  WavArgs w = wav_args(c, c->st);
+  w.chained = chained;
+  const int np = wavelet_apply_ctas(n, c->levels, c->kind, c->tune_rb, c->tune_cmax);
+  int np_rr = axpy_ctas(n);
+  if (wavelet_updates(n, c->levels, c->kind, c->tune_rb)) {
+    w.upd_q = c->q;
+    w.upd_atb = c->atb;
+    w.upd_mode = am;
+    np_rr = np;
+  } else {
     TMark m(c, FIRLS_K_AXPY, 1);
     axpy_step(B, n, c->stream, c->st, c->part, am, c->r, c->q, c->atb, chained);
   }
-  WavArgs w = wav_args(c, c->st);
-  w.chained = chained;
   {
     TMark m(c, FIRLS_K_WAVELET_P, wavelet_apply_launches(n, c->levels, c->kind, c->tune_rb, c->tune_cmax));
     wavelet_apply(w, c->r, c->cw, c->ww, WAV_MUL_PINV, c->z, c->r, real);
   }
   TMark m(c, FIRLS_K_SCALARS, 1);
-  const int np = wavelet_apply_ctas(n, c->levels, c->kind, c->tune_rb, c->tune_cmax);
-  pcg_scalars(B, c->stream, c->st, c->part, np, axpy_ctas(n), sm, ps, c->channels, chained);
+  pcg_scalars(B, c->stream, c->st, c->part, np, np_rr, sm, ps, c->channels, chained);
 }
 
 // The end of every outer step whose PCG has stopped: x += dx, the relative

@@ -370,7 +370,8 @@ static void wcl_launch(const WavArgs& a, int R, bool mirror, const float2* x, co
                        const float2* r, int real) {
   const WclArgs c{x,    u,    w,       a.levels,
                   mode, mirror ? 1 : 0, r, r ? a.part : nullptr,
-                  real, const_cast<SliceState*>(a.st), a.batch, a.stream, a.chained};
+                  real, const_cast<SliceState*>(a.st), a.batch, a.stream, a.chained,
+                  a.upd_q ? const_cast<float2*>(r) : nullptr, a.upd_q, a.upd_atb, a.upd_mode};
   if (a.kind == 2) wcl_launch_db4(a.n, R, c);
   else wcl_launch_haar(a.n, R, c);
 }
@@ -519,6 +520,11 @@ void wavelet_apply(const WavArgs& a, const float2* x, float2* c, float* w, int m
 int wavelet_cluster_ctas(int n, int levels, int kind, int rb) {
   const int R = wcl_rows_per_cta(n, levels, kind, rb, nullptr);
   return R ? n / R : 0;
+}
+
+// Whether wavelet_apply takes the residual update in (WavArgs::upd_q).
+bool wavelet_updates(int n, int levels, int kind, int rb) {
+  return n <= WCL_NMAX && wcl_rows_per_cta(n, levels, kind, rb, nullptr) > 0;
 }
 
 // Partial-sum count of the wavelet_apply stage that computes Re<r, Phi^T ...>.

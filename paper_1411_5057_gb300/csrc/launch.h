@@ -86,6 +86,12 @@ struct WavArgs {
   int rb = 0;          // rows per CTA of the tiled levels (0: default 8)
   int coarse_max = 0;  // largest side kept in shared memory (0: default 64)
   bool chained = false;  // the one-launch form: launch_chained
+  // the one-launch form with r, where wavelet_updates: the residual update on the
+  // way in (axpy_step's work with these arguments; ||r||^2 partials, one per CTA, in
+  // SLOT_RR)
+  const float2* upd_q = nullptr;
+  const float2* upd_atb = nullptr;
+  int upd_mode = 0;
 };
 // c = Phi x (Mallat, stride n) with the final store scaled per `mode`:
 // RAW: c; MUL_W: w*c; MUL_PINV: c / (abar + lam w); SINGLETON_W: writes
@@ -103,6 +109,7 @@ void wavelet_inverse(const WavArgs& a, const float2* c, float2* x, const float2*
 void wavelet_apply(const WavArgs& a, const float2* x, float2* c, float* w, int mode, float2* u,
                    const float2* r, int real);
 int wavelet_cluster_ctas(int n, int levels, int kind, int rb);
+bool wavelet_updates(int n, int levels, int kind, int rb);
 int wavelet_apply_ctas(int n, int levels, int kind, int rb, int coarse_max);
 int wavelet_apply_launches(int n, int levels, int kind, int rb, int coarse_max);
 void wav_prepare();

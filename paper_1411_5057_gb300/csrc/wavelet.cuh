@@ -371,16 +371,25 @@ FI void wcl_push(const float2* D, const float2* Hb, const uint64_t* bar, int n, 
 // levels too (0: from the argument).  One instantiation that took them all from
 // its arguments served every size but 256^2 before: 228 us at 304 slices of
 // 128^2, against 144 us for four times the pixels at 256^2.
-template <int NT, int RT, int LT, int KT, int TH>
+//
+// UPD (z = P^{-1} r of a PCG step): the load is the residual update as well:
+// r -= alpha q, or r = A^H b - q for a slice at the start of its outer step, and
+// the partial ||r||^2.  A launch and a pass over r less than an update of its own
+// (solves of 60 slices of 256^2 4231 -> 4125 us, of one of 64^2 1588 -> 1502).  Up
+// to WCL_NMAX: above, the clusters leave SMs idle that an update of its own uses
+// (8 slices of 512^2: 7697 us apart, 8108 in one).
+template <int NT, int RT, int LT, int KT, int TH, bool UPD>
 __global__ void __launch_bounds__(TH, NT <= 256 ? 2 : 1)
-k_wav_cluster(const float2* x, float2* u, const float* __restrict__ w, int L_arg, int mode, int mirror, 
-              const float2* __restrict__ r, double* __restrict__ part, int real, SliceState* __restrict__ st) {
+k_wav_cluster(const float2* x, float2* u, const float* __restrict__ w, int L_arg, int mode, int mirror,
+              const float2* r, double* __restrict__ part, int real, SliceState* __restrict__ st, float2* rw,
+              const float2* __restrict__ q_in, const float2* __restrict__ atb, int axpy_mode) {
   chained_start();
   const int s = blockIdx.y;
   // the same slice for every CTA of the cluster: all of them leave or none
   if (st != nullptr && !slice_running(st, s)) return;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[32];
+  __shared__ Sum3 rr_part[UPD ? TH / 32 : 1];
   constexpr int n = NT, R = RT, kind = KT;
   constexpr unsigned C = NT / RT;
   const int L = LT ? LT : L_arg, tid = threadIdx.x;
@@ -393,7 +402,8 @@ k_wav_cluster(const float2* x, float2* u, const float* __restrict__ w, int L_arg
   const float* ws = w + (size_t)s * nn;
   {
     const float2* xs = x + (size_t)s * nn + (size_t)rank * R * n;
-    for (int q = tid; q < R * n / 2; q += TH) wcl_cp16(D + 2 * q, xs + 2 * q);
+    if (!UPD)
+      for (int q = tid; q < R * n / 2; q += TH) wcl_cp16(D + 2 * q, xs + 2 * q);
     asm volatile("cp.async.commit_group;\n" ::: "memory");
     if (mirror) {  // the weight of the coefficient each position will hold
       for (int q = tid; q < R * n / 4; q += TH) {
@@ -414,8 +424,58 @@ k_wav_cluster(const float2* x, float2* u, const float* __restrict__ w, int L_arg
                    : "memory");
     }
   }
+  bool updated = false;
+  if (UPD) {
+    const int ph = st[s].phase;
+    updated = axpy_mode != AXPY_PER_SLICE || slice_working(ph);
+    const bool first = axpy_mode == AXPY_INIT || (axpy_mode == AXPY_PER_SLICE && ph == PH_START);
+    const float alpha = (float)st[s].alpha;
+    const size_t off = ((size_t)s * nn + (size_t)rank * R * n) / 2;
+    float4* r4 = reinterpret_cast<float4*>(rw) + off;
+    const float4* src = updated && first ? reinterpret_cast<const float4*>(atb) + off : r4;
+    const float4* q4 = reinterpret_cast<const float4*>(q_in) + off;
+    Sum3 rr{0.f, 0.f, 0.f};
+    constexpr int UN = 4;  // 16-byte loads of r and of q in flight per thread
+    for (int i0 = tid; i0 < R * n / 2; i0 += UN * TH) {
+      float4 rv[UN], qv[UN];
+#pragma unroll
+      for (int e = 0; e < UN; ++e) {
+        const int i = i0 + e * TH;
+        if (i < R * n / 2) {
+          rv[e] = src[i];
+          if (updated) qv[e] = q4[i];
+        }
+      }
+      float acc = 0.f;
+#pragma unroll
+      for (int e = 0; e < UN; ++e) {
+        const int i = i0 + e * TH;
+        if (i >= R * n / 2) continue;
+        float2 a = make_float2(rv[e].x, rv[e].y), b = make_float2(rv[e].z, rv[e].w);
+        if (updated) {
+          const float2 qa = make_float2(qv[e].x, qv[e].y), qb = make_float2(qv[e].z, qv[e].w);
+          a = first ? csub(a, qa) : cfma(-alpha, qa, a);
+          b = first ? csub(b, qb) : cfma(-alpha, qb, b);
+          acc += cabs2(a) + cabs2(b);
+          r4[i] = make_float4(a.x, a.y, b.x, b.y);
+        }
+        reinterpret_cast<float4*>(D)[i] = make_float4(a.x, a.y, b.x, b.y);
+      }
+      rr.add(acc);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rr.add(rr.from_lane(o));
+    if ((tid & 31) == 0) rr_part[tid >> 5] = rr;
+  }
   asm volatile("cp.async.wait_group 1;\n" ::: "memory");
   __syncthreads();
+  if (UPD && updated && tid < 32) {
+    Sum3 rr{0.f, 0.f, 0.f};
+    if (tid < TH / 32) rr = rr_part[tid];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rr.add(rr.from_lane(o));
+    if (tid == 0) part[((size_t)s * NSLOT + SLOT_RR) * MAXPART + rank] = rr.value();
+  }
   if (kind == 2)  // every CTA's mbarriers armed before any remote write
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
   WclScale sc;
@@ -498,6 +558,9 @@ struct WclArgs {
   int batch;
   cudaStream_t stream;
   bool chained;
+  float2* rw;  // residual to update on the way in (x = r = rw), or null
+  const float2 *q, *atb;
+  int axpy_mode;
 };
 
 template <int N, int R, int TH>
@@ -525,17 +588,25 @@ template <int N, int R, int L, int KT, int TH> bool wcl_launch_as(const WclArgs&
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 2;
   }
-  return cudaLaunchKernelEx(&cfg, k_wav_cluster<N, R, L, KT, TH>, a.x, a.u, a.w, a.levels, a.mode, a.mirror, a.r,
-                            a.part, a.real, a.st) == cudaSuccess;
+  auto k = k_wav_cluster<N, R, L, KT, TH, false>;
+  if constexpr (N <= WCL_NMAX) {
+    if (a.rw) k = k_wav_cluster<N, R, L, KT, TH, true>;
+  }
+  return cudaLaunchKernelEx(&cfg, k, a.x, a.u, a.w, a.levels, a.mode, a.mirror, a.r,
+                            a.part, a.real, a.st, a.rw, a.q, a.atb, a.axpy_mode) == cudaSuccess;
 }
 template <int N, int R, int L, int KT, int TH> bool wcl_attr_as() {
-  return cudaFuncSetAttribute(k_wav_cluster<N, R, L, KT, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              wcl_smem_bytes(N, R, L ? L : WCL_LMAX, true)) == cudaSuccess;
+  const int bytes = wcl_smem_bytes(N, R, L ? L : WCL_LMAX, true);
+  const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  bool ok = cudaFuncSetAttribute(k_wav_cluster<N, R, L, KT, TH, false>, A, bytes) == cudaSuccess;
+  if constexpr (N <= WCL_NMAX)
+    ok = cudaFuncSetAttribute(k_wav_cluster<N, R, L, KT, TH, true>, A, bytes) == cudaSuccess && ok;
+  return ok;
 }
 // A cluster above the portable 8 CTAs: how many the device holds at once, 0
 // where it cannot be launched.
 template <int N, int R, int KT, int TH> int wcl_wide_resident() {
-  auto k = k_wav_cluster<N, R, 0, KT, TH>;
+  auto k = k_wav_cluster<N, R, 0, KT, TH, false>;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
   wcl_config<N, R, TH>(cfg, at, WCL_LMAX, true, 1, nullptr);
