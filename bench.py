@@ -71,21 +71,20 @@ REF_OUTER_PER_RECON = 43   # FP64 oracle outer steps (x 60 PCG) to 1e-4 of x* on
 # input read once and every output written once (complex64 8 B, float 4 B,
 # mask 1 B).  Wavelet passes move the full pyramid (4/3 of the image).
 ALG_BYTES_PER_PX = {
-    "row_fft": 32.0,            # read z, d; write d, t
+    "row_fft": 48.0,            # read z, d, dx; write d, dx, t
     "col_fft_mask": 17.0,       # read t, mask; write t
     "wavelet_S": 8.0 + 4.0 + 8.0,     # read d and w, write u = Phi^T (w o Phi d)
     "row_ifft_combine": 36.0,   # read t, d, u, W_tv; write q
-    "ilu": 64.0,                # read x, d, r, q, W_tv, 1/a; write x, r, z
-    "axpy": 32.0,
+    "ilu": 40.0,                # read r, q, W_tv and 1/a (packed); write r, z
+    "axpy": 24.0,               # read r, q; write r
 }
 
 # DRAM bytes per pixel per launch (dram__bytes_read.sum + dram__bytes_write.sum)
-# of the dominant kernel at the bench's 304 slots of 256^2, by the ILU ring
-# shape the autotuner picks, from one-pass ncu captures of those two counters
-# (profiles/kernels_tv_db4_256_b96.md gives the commands), for the kernel as
-# it is now: 1.634 GB per launch with ring 22, 1.618 GB with ring 42.  Other
-# shapes: not measured (traffic null).
-MEASURED_TRAFFIC_PER_PX = {("ilu", 22): 82.0, ("ilu", 42): 81.2}
+# of a kernel class at the bench's 304 slots of 256^2, by tuned ILU shape, from
+# one-pass ncu captures of those two counters (profiles/kernels_tv_db4_256_b96.md
+# gives the commands).  Classes and shapes not listed: not measured (traffic
+# null).
+MEASURED_TRAFFIC_PER_PX = {}
 
 
 def problem(seed):
