@@ -463,15 +463,13 @@ firls_status check_params(firls_ctx* c, const firls_params* p) {
 
 firls_status upload_params(firls_ctx* c, const firls_params* p) {
   const int B = c->batch;
-  std::vector<float> l(B), lt(B);
+  std::vector<float> l(2 * (size_t)B);
   for (int s = 0; s < B; ++s) {
-    l[s] = p->lambda_per_slice ? p->lambda_per_slice[s] : p->lambda;
-    lt[s] = has_tv(c) ? (p->lambda_tv_per_slice ? p->lambda_tv_per_slice[s] : p->lambda_tv) : 0.f;
-    if (!c->kind) l[s] = 0.f;
+    l[s] = c->kind ? (p->lambda_per_slice ? p->lambda_per_slice[s] : p->lambda) : 0.f;
+    l[B + s] = has_tv(c) ? (p->lambda_tv_per_slice ? p->lambda_tv_per_slice[s] : p->lambda_tv) : 0.f;
   }
-  CU(cudaMemcpyAsync(c->lam_d, l.data(), sizeof(float) * B, cudaMemcpyHostToDevice, c->stream));
-  CU(cudaMemcpyAsync(c->lamtv_d, lt.data(), sizeof(float) * B, cudaMemcpyHostToDevice, c->stream));
-  // pageable copies: make sure the host vectors may go out of scope
+  CU(cudaMemcpyAsync(c->lam_d, l.data(), sizeof(float) * l.size(), cudaMemcpyHostToDevice, c->stream));
+  // a pageable copy: make sure the host vector may go out of scope
   CU(cudaStreamSynchronize(c->stream));
   return FIRLS_OK;
 }
@@ -731,8 +729,8 @@ extern "C" firls_status firls_create(firls_ctx** out, int n_rows, int n_cols, in
   A(&c->stw, (size_t)batch);
   A(&c->part, (size_t)batch * NSLOT * MAXPART);
   A(&c->fobj, 2 * (size_t)batch);
-  A(&c->lam_d, (size_t)batch);
-  A(&c->lamtv_d, (size_t)batch);
+  A(&c->lam_d, 2 * (size_t)batch);  // both lambdas in one block: one copy uploads them
+  if (c->lam_d) c->lamtv_d = c->lam_d + batch;
   if (s != FIRLS_OK) {
     firls_destroy(c);
     return s;
