@@ -82,9 +82,9 @@ ALG_BYTES_PER_PX = {
 # DRAM bytes per pixel per launch (dram__bytes_read.sum + dram__bytes_write.sum)
 # of a kernel class at the bench's 304 slots of 256^2, by tuned ILU shape, from
 # one-pass ncu captures of those two counters (profiles/kernels_tv_db4_256_b96.md
-# gives the commands).  Classes and shapes not listed: not measured (traffic
-# null).
-MEASURED_TRAFFIC_PER_PX = {}
+# gives the commands): 1.303 GB per launch with shape 22, 1.219 GB with shape 42.
+# Classes and shapes not listed: not measured (traffic null).
+MEASURED_TRAFFIC_PER_PX = {("ilu", 22): 65.4, ("ilu", 42): 61.2}
 
 
 def problem(seed):
