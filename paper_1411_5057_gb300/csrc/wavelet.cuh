@@ -313,7 +313,10 @@ FI void wcl_col_edge(float2* Dc, const float2* H, const uint64_t* bar, bool& ok,
 // 2m threads the pairs of a column are split into `parts` ranges, one thread
 // each: every part first reads the rows its neighbouring part will overwrite
 // (forward: the next part's first two rows; inverse: the previous part's
-// last pair), the CTA synchronises, then all parts stream in place.
+// last pair), the CTA synchronises, then all parts stream in place.  Whole
+// columns (parts 1) synchronise before the first store too: wcl_push's threads
+// read the boundary rows, and another thread than the one that reads a column's
+// element there updates it.
 FI void wcl_cols(float2* D, const float2* H, const uint64_t* bar, bool& ok, int n, int sr, int Rl, int m, int kind,
                  bool inverse, bool last_level, const WclScale& sc, int nth) {
   const int rs = sr * n, npair = Rl / 2;
@@ -321,6 +324,7 @@ FI void wcl_cols(float2* D, const float2* H, const uint64_t* bar, bool& ok, int 
   int parts = 1;
   while (parts * 2 * m <= nth && npair % (parts * 2) == 0) parts *= 2;  // equal ranges only
   if (parts == 1) {
+    if (halo) __syncthreads();  // wcl_push reads the boundary rows that this step overwrites
     for (int j = threadIdx.x; j < m; j += nth) {
       const bool lo_final = last_level || j >= m / 2;
       if (halo)
