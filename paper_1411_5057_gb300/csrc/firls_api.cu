@@ -1169,7 +1169,10 @@ extern "C" firls_status firls_apply_S_P(firls_ctx* c, const firls_params* p, con
   if (c->skewed) {
     ilu_skew(B, n, c->stream, true, c->atb, c->q);
     enqueue_precond(c, ILU_INIT, one);
-    ilu_skew(B, n, c->stream, false, c->z, static_cast<float2*>(z));
+    // the layout change stores 16 bytes at a time; z may have any alignment
+    const bool aligned = reinterpret_cast<uintptr_t>(z) % 16 == 0;
+    ilu_skew(B, n, c->stream, false, c->z, aligned ? static_cast<float2*>(z) : c->u);
+    if (!aligned) CU(cudaMemcpyAsync(z, c->u, bytes, cudaMemcpyDeviceToDevice, c->stream));
   } else {
     CU(cudaMemsetAsync(c->q, 0, bytes, c->stream));
     enqueue_precond(c, ILU_INIT, one);
