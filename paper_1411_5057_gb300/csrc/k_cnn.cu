@@ -21,6 +21,7 @@
 
 #include <cuda_bf16.h>
 
+#include "cnn_index.h"
 #include "firls.h"
 #include "firls_common.cuh"
 #include "per_device.h"
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv3x3_tc(int n, int tiles, 
       for (int px = px0; px < TC_HR * TC_HW; px += STEP) {
         const bool inside = (unsigned)y < (unsigned)n && (unsigned)x < (unsigned)n;
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst),
-                     "l"(src + (inside ? (y * n + x) * CIN : 0)), "r"(inside ? 16 : 0)
+                     "l"(src + (inside ? cnn_pixel(y, x, n, CIN) : 0)), "r"(inside ? 16 : 0)
                      : "memory");
         dst += STEP * 16;
         x += STEP;
