@@ -151,14 +151,16 @@ FI double block_sum(double v, double* red) {
   return s;
 }
 
-// s + e = a + b exactly.
+// s + e = a + b exactly (Knuth's TwoSum).  The rounded intrinsics keep the compiler
+// from contracting a product that was passed in into these sums, which would
+// leave its low half out of s and in e.
 FI void two_sum(float a, float b, float& s, float& e) {
-  const float t = a + b, bb = t - a;
-  e = (a - (t - bb)) + (b - bb);
+  const float t = __fadd_rn(a, b), bb = __fsub_rn(t, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
   s = t;
 }
 
-// A sum carried in three floats, for kernels that accumulate many values each:
+// A cascaded sum in three floats, for kernels that accumulate many values each:
 // the device has 2 FP64 lanes per clock and SM.  A product of two floats is
 // exactly p + e with e = fma(a, b, -p); each two_sum is exact and the third
 // float takes the remainders, so it loses less than an FP64 sum.
@@ -179,7 +181,7 @@ struct Sum3 {
     cc += f;
   }
   FI void add_product(float a, float b) {
-    const float p = a * b;
+    const float p = __fmul_rn(a, b);
     add(p, fmaf(a, b, -p));
   }
   FI void add(const Sum3& o) {
