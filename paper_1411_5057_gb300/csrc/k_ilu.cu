@@ -271,6 +271,9 @@ __global__ void __launch_bounds__(MAXT, MINB)
     }
   }
   if (!ok) abort_flag = 1;
+  // in a part band the lanes past the image read lane `last`'s y below; their
+  // coefficients are 0, but the values have to be those it has just stored
+  __syncwarp();
   {  // ---- backward: step m = K - 1 - k, from the last row and column
     float2 p0 = make_float2(0.f, 0.f);  // lam W z of this row's last pair, and its
     float4 pv = make_float4(0.f, 0.f, 0.f, 0.f);  // vertical one (W2 for l1 TV)
