@@ -50,6 +50,7 @@ struct firls_ctx {
   float4* wa = nullptr;
   float2* w2s = nullptr;
   bool skewed = false;
+  bool skew_room = false;  // r, z, q and u have the size of that layout (1.24 x at 256^2, 9.75 x at 16^2)
   float* wg = nullptr;
   int *gidx = nullptr, *goff = nullptr, *inv_off = nullptr, *inv_ids = nullptr;
   int *gcounts = nullptr, *gcursor = nullptr, *gerr = nullptr;
@@ -102,10 +103,21 @@ firls_status cuda_check(firls_ctx* c, cudaError_t e, const char* what) {
 template <typename T> firls_status dalloc(firls_ctx* c, T** p, size_t count) {
   void* v = nullptr;
   cudaError_t e = cudaMalloc(&v, count * sizeof(T) + 16);
-  if (e != cudaSuccess) return cuda_check(c, e, "cudaMalloc");
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next call
+    return cuda_check(c, e, "cudaMalloc");
+  }
   c->allocs.push_back(v);
   *p = static_cast<T*>(v);
   return FIRLS_OK;
+}
+
+// cudaFree of an allocation of this context (or nothing)
+void dfree(firls_ctx* c, void* p) {
+  if (!p) return;
+  cudaFree(p);
+  for (auto& a : c->allocs)
+    if (a == p) a = nullptr;
 }
 
 #define TRY(expr)                        \
@@ -490,6 +502,27 @@ firls_status match_layout(firls_ctx* c, int precond) {
   return cuda_check(c, cudaGetLastError(), "layout change");
 }
 
+// r, z, q and u at the size of the sweeps' layout, for the first operator with TV.  One
+// after the other, so that the old and the new form of only one exist at a time; r
+// and z keep what live slots have there.  The captured graphs, which hold the old
+// addresses, are dropped by firls_set_operator before anything can run.
+firls_status sweep_room(firls_ctx* c) {
+  if (c->skew_room) return FIRLS_OK;
+  const size_t natural = (size_t)c->batch * c->n * c->n;
+  for (float2** v : {&c->q, &c->u, &c->r, &c->z}) {
+    float2* room = nullptr;
+    TRY(dalloc(c, &room, ilu_slice_elems(c->n) * c->batch));
+    if (v == &c->r || v == &c->z) {
+      CU(cudaMemcpyAsync(room, *v, sizeof(float2) * natural, cudaMemcpyDeviceToDevice, c->stream));
+      CU(cudaStreamSynchronize(c->stream));
+    }
+    dfree(c, *v);
+    *v = room;
+  }
+  c->skew_room = true;
+  return FIRLS_OK;
+}
+
 float eps_of(const firls_params* p) { return p->eps > 0.f ? p->eps : 1e-10f; }
 
 // A^H b into atb (and x when x0 is null), ||A^H b||^2 partials, state init
@@ -718,13 +751,10 @@ extern "C" firls_status firls_create(firls_ctx** out, int n_rows, int n_cols, in
   A(&c->mask, BN);
   A(&c->counts, (size_t)batch);
   A(&c->tw, (size_t)n);
-  for (float2** p : {&c->atb, &c->x, &c->d, &c->t, &c->cw, &c->dx}) A(p, BN);
-  // these take the ILU's skewed layout too
-  const size_t BS = std::max(N, ilu_slice_elems(n)) * batch;
-  for (float2** p : {&c->r, &c->z, &c->q, &c->u}) A(p, BS);
+  for (float2** p : {&c->atb, &c->x, &c->r, &c->z, &c->d, &c->q, &c->t, &c->u, &c->cw, &c->dx}) A(p, BN);
   A(&c->tmpA, BH);
   A(&c->tmpB, BH);
-  for (float** p : {&c->ww, &c->wtv, &c->ia, &c->wdiag, &c->wtv2}) A(p, BN);
+  for (float** p : {&c->ww, &c->wtv, &c->ia, &c->wdiag}) A(p, BN);
   A(&c->st, (size_t)batch);
   A(&c->stw, (size_t)batch);
   A(&c->part, (size_t)batch * NSLOT * MAXPART);
@@ -803,20 +833,9 @@ extern "C" firls_status firls_set_operator(firls_ctx* c, const uint8_t* mask, un
     }
     if (total < 0) return fail(c, FIRLS_E_GROUPMAP, "negative member count");
     // (re)allocate the map buffers
-    auto rel = [&](void* p) {
-      if (!p) return;
-      cudaFree(p);
-      for (auto& a : c->allocs)
-        if (a == p) a = nullptr;
-    };
-    rel(c->gidx);
-    rel(c->goff);
-    rel(c->inv_off);
-    rel(c->inv_ids);
-    rel(c->gcounts);
-    rel(c->gcursor);
-    rel(c->gerr);
-    rel(c->wg);
+    for (void* p : {(void*)c->gidx, (void*)c->goff, (void*)c->inv_off, (void*)c->inv_ids, (void*)c->gcounts,
+                    (void*)c->gcursor, (void*)c->gerr, (void*)c->wg})
+      dfree(c, p);
     c->gidx = c->goff = nullptr;
     TRY(dalloc(c, &c->gidx, (size_t)total));
     if (group_off) TRY(dalloc(c, &c->goff, (size_t)n_groups + 1));
@@ -847,19 +866,26 @@ extern "C" firls_status firls_set_operator(firls_ctx* c, const uint8_t* mask, un
     std::vector<float> tab;
     std::vector<int> len;
     basis_tables(n, wavelet_levels, kind == 1 ? FIRLS_PSI_HAAR : FIRLS_PSI_DB4, tab, len);
-    if (c->sqtab) {
-      cudaFree(c->sqtab);
-      cudaFree(c->sqlen);
-      for (auto& a : c->allocs)
-        if (a == c->sqtab || a == c->sqlen) a = nullptr;
-    }
+    dfree(c, c->sqtab);
+    dfree(c, c->sqlen);
+    c->sqtab = nullptr;
+    c->sqlen = nullptr;
     TRY(dalloc(c, &c->sqtab, tab.size()));
     TRY(dalloc(c, &c->sqlen, len.size()));
     CU(cudaMemcpy(c->sqtab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(c->sqlen, len.data(), sizeof(int) * len.size(), cudaMemcpyHostToDevice));
   }
-  if ((psi_kind & (FIRLS_PSI_TV | FIRLS_PSI_TV_ANISO)) && !c->wa) TRY(dalloc(c, &c->wa, ilu_slice_elems(n) / 2 * B));
-  if ((psi_kind & FIRLS_PSI_TV_ANISO) && !c->w2s) TRY(dalloc(c, &c->w2s, ilu_slice_elems(n) / 2 * B));
+  if (psi_kind & (FIRLS_PSI_TV | FIRLS_PSI_TV_ANISO)) {
+    TRY(sweep_room(c));
+    if (!c->wa) TRY(dalloc(c, &c->wa, ilu_slice_elems(n) / 2 * B));
+  }
+  if (psi_kind & FIRLS_PSI_TV_ANISO) {
+    if (!c->wtv2) {
+      TRY(dalloc(c, &c->wtv2, N * B));
+      CU(cudaMemsetAsync(c->wtv2, 0, sizeof(float) * N * B, c->stream));
+    }
+    if (!c->w2s) TRY(dalloc(c, &c->w2s, ilu_slice_elems(n) / 2 * B));
+  }
   c->psi = psi_kind;
   c->kind = kind;
   c->levels = kind ? wavelet_levels : 0;
@@ -1342,7 +1368,8 @@ extern "C" firls_status firls_slot_move(firls_ctx* c, int from, int to) {
   for (float2* v : {c->r, c->z}) CU(mv(v, c->skewed ? NS : N));
   if (c->wa) CU(mv(c->wa, NS / 2));
   if (c->w2s) CU(mv(c->w2s, NS / 2));
-  for (float* v : {c->ww, c->wtv, c->ia, c->wdiag, c->wtv2}) CU(mv(v, N));
+  for (float* v : {c->ww, c->wtv, c->ia, c->wdiag}) CU(mv(v, N));
+  if (c->wtv2) CU(mv(c->wtv2, N));
   if (c->groups) CU(mv(c->wg, (size_t)c->n_groups));
   CU(mv(c->st, 1));
   CU(mv(c->stw, 1));
