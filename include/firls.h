@@ -295,8 +295,9 @@ firls_status firls_set_active_slots(firls_ctx* ctx, int k);
  * HBM, where the slice fits; 4, 8, 16: rows per CTA of the tiled levels), the
  * largest wavelet block kept in shared memory by the tiled form (32, 64), the
  * ILU shape (42: long chunks, one CTA per SM; 22: short ones, two).  cache_path (may be NULL) is a text file of earlier
- * results keyed by "n batch psi levels": a hit skips the timing, a miss
- * appends the new result.  Overwrites the context's workspace; call after
+ * results keyed by "n batch psi levels" and a number that changes with the
+ * kernels that were timed: a hit skips the timing, a miss appends the new
+ * result.  Overwrites the context's workspace; call after
  * firls_set_operator and before solving.  Synchronises the stream. */
 firls_status firls_autotune(firls_ctx* ctx, const char* cache_path);
 

@@ -57,7 +57,7 @@ struct firls_ctx {
   float* sqtab = nullptr;
   int* sqlen = nullptr;
   // tile shapes (autotuned or defaults)
-  int tune_rb = 0, tune_cmax = 0, tune_ilu = 0;  // 0: ILU ring shape chosen from n and batch
+  int tune_rb = 0, tune_cmax = 0, tune_ilu = 0;  // 0: the ILU's chunks by size and batch
   int wait_test = 0;  // failure-detection test: the ILU's bounded waits run out (firls_set_wait_test)
   SliceState* st = nullptr;
   double* part = nullptr;
@@ -1389,6 +1389,8 @@ extern "C" firls_status firls_slot_get(firls_ctx* c, int s, void* x_out) {
 
 // ---- autotuner: tile shapes timed on the context's own buffers ----
 namespace {
+constexpr int TUNED_KERNELS = 2;  // raised when a timed kernel or its candidates change
+
 bool tune_cache_lookup(const char* path, const std::string& key, int* rb, int* cm, int* il) {
   if (!path || !*path) return false;
   FILE* f = std::fopen(path, "r");
@@ -1431,13 +1433,17 @@ extern "C" firls_status firls_autotune(firls_ctx* c, const char* cache_path) {
   if (!c->op_set) return fail(c, FIRLS_E_STATE, "operator not set");
   const int B = c->batch, n = c->n;
   char keybuf[128];
-  std::snprintf(keybuf, sizeof keybuf, "n=%d batch=%d psi=%u levels=%d ", n, B, c->psi, c->levels);
+  // TUNED_KERNELS: results timed on kernels since replaced are not reused (an entry
+  // from before the wide clusters would pin 320^2 to 512^2 to the tiled levels)
+  std::snprintf(keybuf, sizeof keybuf, "n=%d batch=%d psi=%u levels=%d kernels=%d ", n, B, c->psi, c->levels,
+                TUNED_KERNELS);
   const std::string key(keybuf);
   int rb = 0, cm = 0, il = 0;
   if (!tune_cache_lookup(cache_path, key, &rb, &cm, &il)) {
     // deterministic, finite contents for timing
-    const size_t BN = (size_t)B * n * n;
-    for (float2* v : {c->x, c->d, c->r, c->q, c->z, c->atb, c->u, c->cw}) cudaMemsetAsync(v, 0, BN * 8, c->stream);
+    const size_t BN = (size_t)B * n * n, BS = c->skew_room ? ilu_slice_elems(n) * B : BN;
+    for (float2* v : {c->x, c->d, c->atb, c->cw}) cudaMemsetAsync(v, 0, BN * 8, c->stream);
+    for (float2* v : {c->r, c->q, c->z, c->u}) cudaMemsetAsync(v, 0, BS * 8, c->stream);
     for (float* v : {c->ww, c->wtv, c->wdiag}) cudaMemsetAsync(v, 0, BN * 4, c->stream);
     firls_params p{};
     p.outer_iters = p.pcg_iters = 1;
