@@ -204,6 +204,14 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const char* a0 = reinterpret_cast<const char*>(fwd ? (init ? q : r) : y);
     const char* a1 = reinterpret_cast<const char*>(fwd ? q : wa);
     const char* a2 = reinterpret_cast<const char*>(wa);
+    if (ANISO) {  // W2: two lines per step
+#pragma unroll
+      for (int i = 0; i < CS * 2; i += 32) {
+        const int j = i + lane, k = k0 + j / 2, l16 = j % 2 * 16;
+        const char* p = reinterpret_cast<const char*>(w2) + (ptrdiff_t)k * 256 + l16 * 8;
+        if (j < CS * 2 && l16 <= min(last, k) && l16 + 15 > k - H) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+      }
+    }
 #pragma unroll
     for (int i = 0; i < (fwd ? 3 : 2) * LINES; i += 32) {
       const int j = i + lane, a = j / LINES, k = k0 + (j % LINES) / 4, l8 = j % 4 * 8;
@@ -473,13 +481,16 @@ typedef void (*IluKernel)(int, int, SliceState*, double*, float4*, const float4*
                           const float2*, int, PcgSched, int, int);
 // Chunks of 8 steps where the CTA has the registers of an SM to itself (up to
 // 256 rows); of 4 with two CTAs of 256^2 per SM; of 5 and 4 above 256 rows,
-// where the CTA has more warps.
+// where the CTA has more warps.  l1 TV holds W2 in the chunks too: of 3 steps where a
+// thread has 128 registers (4 spilled: 304 slices of 256^2 337 -> 275 us, 304 of
+// 128^2 132 -> 96, 40 of 512^2 486 -> 385; the row scans before took 297, 95 and 557).
 template <bool ANISO>
 IluKernel ilu_kernel(int n, bool deep, bool far) {
-  if (wv_bands(n) > 12) return k_ilu<4, 512, 1, 0, ANISO>;
+  constexpr int CS = ANISO ? 3 : 4;
+  if (wv_bands(n) > 12) return k_ilu<CS, 512, 1, 0, ANISO>;
   if (wv_bands(n) > 8) return k_ilu<5, 384, 1, 0, ANISO>;
   if (deep) return far ? k_ilu<8, 256, 1, 4, ANISO> : k_ilu<8, 256, 1, 0, ANISO>;
-  return far ? k_ilu<4, 256, 2, 4, ANISO> : k_ilu<4, 256, 2, 0, ANISO>;
+  return far ? k_ilu<CS, 256, 2, 4, ANISO> : k_ilu<CS, 256, 2, 0, ANISO>;
 }
 
 }  // namespace
