@@ -506,10 +506,21 @@ bool ilu_prepare() {
   return ok;
 }
 
-// Shapes are numbered 10 * G + S: G = 4 takes chunks of 8 steps (one CTA per
-// SM), G = 2 of 4 steps; S has no effect.  All shapes give the same results
-// bit for bit.
-int ilu_default_shape(int batch) { return batch <= 152 ? 42 : 22; }
+// Shapes are numbered 10 * G + S: G = 4 takes long chunks (8 warps per SM), G = 2
+// short ones (16); S has no effect.  All shapes give the same results bit for bit.
+// A full wave of short chunks serves twice the slices in about 1.9 times the time of a
+// wave of long ones (128^2: 608 slices 140 us, 304 74), so the default takes the long
+// ones where they need fewer than 1.9 times the waves.  Long and short, us: 128^2 152
+// slices 57 and 69, 304 73 and 94, 400 122 and 107, 800 197 and 224; 64^2 300 slices
+// 32 and 39, 900 75 and 67, 1500 115 and 129; 256^2 152 slices 132 and 175, 160 217 and
+// 197, 304 260 and 254.  (By the batch alone, 152 slices at every size, 304 slices of 128^2
+// were no faster than with the row scans before.)
+int ilu_default_shape(int n, int batch) {
+  const int bands = wv_bands(n), sms = 152;
+  if (bands > 8) return 22;  // one form there
+  auto waves = [&](int warps) { return (batch + sms * (warps / bands) - 1) / (sms * (warps / bands)); };
+  return 10 * waves(8) < 19 * waves(16) ? 42 : 22;
+}
 
 // The shapes that set_tuning takes for a size.
 bool ilu_shape_fits(int n, int shape, bool aniso) {
@@ -522,7 +533,7 @@ bool ilu_shape_fits(int n, int shape, bool aniso) {
 void ilu_step(int batch, int n, cudaStream_t s, SliceState* st, double* part, int mode, float2* r, const float2* q,
               float2* y, float2* z, const float4* wa, const float2* w2s, int shape, int fuse_scalars, PcgSched ps,
               int wait_test, int alpha_np, bool chained) {
-  if (shape <= 0) shape = ilu_default_shape(batch);
+  if (shape <= 0) shape = ilu_default_shape(n, batch);
   const bool deep = shape / 10 == 4;
   // r, q, y, z and the weights: 40 bytes a pixel against an L2 of 129 MB.  304
   // slices of 256^2: 247 us with the fetches into L2, 257 without; 16: 96

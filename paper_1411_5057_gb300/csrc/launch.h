@@ -147,7 +147,7 @@ void ilu_skew(int batch, int n, cudaStream_t s, bool to_skewed, const float2* sr
 enum IluMode { ILU_INIT = 0, ILU_STEP = 1, ILU_PER_SLICE = -1 };
 // all arrays skewed.  INIT: r = q (the first residual); STEP: r -= alpha q.
 // w2s null: isotropic TV.
-// shape: the sweeps' chunks (ilu_default_shape; 0: by the batch)
+// shape: the sweeps' chunks (0: ilu_default_shape)
 // fuse_scalars: the CTA finishes the PCG scalars itself from its sums (rho
 // at ILU_INIT; rr, the residual test against pcg_tol, beta and rho at ILU_STEP)
 // alpha_np > 0 (ILU_PER_SLICE): the CTA of a slice in PCG first forms alpha
@@ -156,7 +156,7 @@ void ilu_step(int batch, int n, cudaStream_t s, SliceState* st, double* part, in
               float2* y, float2* z, const float4* wa, const float2* w2s, int shape, int fuse_scalars = 0,
               PcgSched ps = PcgSched{0.f, 0, 1 << 30, 0, 0}, int wait_test = 0, int alpha_np = 0,
               bool chained = false);
-int ilu_default_shape(int batch);
+int ilu_default_shape(int n, int batch);
 bool ilu_shape_fits(int n, int shape, bool aniso = false);
 
 // AXPY_PER_SLICE (and ILU_PER_SLICE, SCALARS_PER_SLICE, mode < 0 of the row
