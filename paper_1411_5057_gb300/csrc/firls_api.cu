@@ -1191,15 +1191,16 @@ extern "C" firls_status firls_apply_S_P(firls_ctx* c, const firls_params* p, con
   firls_params one = *p;
   one.pcg_tol = 0.f;
   c->skewed = uses_ilu(c, p->precond);
-  CU(cudaMemcpyAsync(c->atb, r, bytes, cudaMemcpyDeviceToDevice, c->stream));
   if (c->skewed) {
-    ilu_skew(B, n, c->stream, true, c->atb, c->q);
+    // the layout change moves 16 bytes at a time; r and z may have any alignment
+    auto aligned = [](const void* v) { return reinterpret_cast<uintptr_t>(v) % 16 == 0; };
+    if (!aligned(r)) CU(cudaMemcpyAsync(c->atb, r, bytes, cudaMemcpyDeviceToDevice, c->stream));
+    ilu_skew(B, n, c->stream, true, aligned(r) ? static_cast<const float2*>(r) : c->atb, c->q);
     enqueue_precond(c, ILU_INIT, one);
-    // the layout change stores 16 bytes at a time; z may have any alignment
-    const bool aligned = reinterpret_cast<uintptr_t>(z) % 16 == 0;
-    ilu_skew(B, n, c->stream, false, c->z, aligned ? static_cast<float2*>(z) : c->u);
-    if (!aligned) CU(cudaMemcpyAsync(z, c->u, bytes, cudaMemcpyDeviceToDevice, c->stream));
+    ilu_skew(B, n, c->stream, false, c->z, aligned(z) ? static_cast<float2*>(z) : c->u);
+    if (!aligned(z)) CU(cudaMemcpyAsync(z, c->u, bytes, cudaMemcpyDeviceToDevice, c->stream));
   } else {
+    CU(cudaMemcpyAsync(c->atb, r, bytes, cudaMemcpyDeviceToDevice, c->stream));
     CU(cudaMemsetAsync(c->q, 0, bytes, c->stream));
     enqueue_precond(c, ILU_INIT, one);
     CU(cudaMemcpyAsync(z, c->z, bytes, cudaMemcpyDeviceToDevice, c->stream));

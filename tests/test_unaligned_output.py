@@ -1,5 +1,6 @@
-"""z = P^{-1} r into a complex64 view that starts 8 bytes past a 16-byte boundary, for
-every preconditioner with TV and without: the same bits as into an aligned array."""
+"""z = P^{-1} r and q = S d from and into complex64 views that start 8 bytes past a 16-byte
+boundary, for every preconditioner with TV and without: the same bits as with
+aligned arrays."""
 import numpy as np
 import pytest
 
@@ -25,12 +26,14 @@ def test_unaligned_z(n, batch, psi, levels, precond):
     params = F.make_params(1, 1, lam=1e-2, lam_tv=1e-2 if psi & (fs.PSI_TV | 8) else 0.0, precond=precond)
     out = []
     for off in (0, 1):
-        room = [torch.empty(batch * n * n + 2, dtype=torch.complex64, device="cuda") for _ in range(2)]
+        room = [torch.empty(batch * n * n + 2, dtype=torch.complex64, device="cuda") for _ in range(5)]
         for v in room:
             v.fill_(7.0)
-        q, z = (v[off:off + batch * n * n].view(batch, n, n) for v in room)
-        assert z.data_ptr() % 16 == 8 * off
-        ctx.apply_S_P(params, x, d, q, r, z)
+        xv, dv, rv, q, z = (v[off:off + batch * n * n].view(batch, n, n) for v in room)
+        for v, w in ((xv, x), (dv, d), (rv, r)):
+            v.copy_(w)
+        assert all(v.data_ptr() % 16 == 8 * off for v in (xv, dv, rv, q, z))
+        ctx.apply_S_P(params, xv, dv, q, rv, z)
         torch.cuda.synchronize()
         assert all(torch.equal(v[off + batch * n * n:].real, torch.full((2 - off,), 7.0, device="cuda")) for v in room)
         out.append((q.clone(), z.clone()))
