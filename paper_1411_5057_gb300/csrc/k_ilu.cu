@@ -514,10 +514,12 @@ bool ilu_prepare() {
 // slices 57 and 69, 304 73 and 94, 400 122 and 107, 800 197 and 224; 64^2 300 slices
 // 32 and 39, 900 75 and 67, 1500 115 and 129; 256^2 152 slices 132 and 175, 160 217 and
 // 197, 304 260 and 254.  (By the batch alone, 152 slices at every size, 304 slices of 128^2
-// were no faster than with the row scans before.)
+// were no faster than with the row scans before.)  Below 32 rows half the lanes idle and a
+// sweep is short against the long chunks' start: 1500 slices of 16^2 37 and 23.
 int ilu_default_shape(int n, int batch) {
   const int bands = wv_bands(n), sms = 152;
   if (bands > 8) return 22;  // one form there
+  if (n < 32) return batch <= sms ? 42 : 22;
   auto waves = [&](int warps) { return (batch + sms * (warps / bands) - 1) / (sms * (warps / bands)); };
   return 10 * waves(8) < 19 * waves(16) ? 42 : 22;
 }
