@@ -305,8 +305,9 @@ void enqueue_weights(firls_ctx* c, const float2* x, int precond, const SliceStat
     // with TV, 1/a of the penta-diagonal P is also 1/diag(S) (the Jacobi scale)
     tv_weights(B, n, c->stream, view, x, c->wtv, tv2_of(c), c->channels);
     if (c->kind) wavelet_diag(B, n, c->levels, c->kind, c->stream, view, c->ww, c->wdiag, c->sqtab, c->sqlen);
-    penta_setup(B, n, c->stream, view, c->wtv, tv2_of(c), c->kind ? c->wdiag : nullptr, c->ia);
-    if (uses_ilu(c, precond)) ilu_pack(B, n, c->stream, view, false, c->wtv, tv2_of(c), c->ia, c->wa, w2s_of(c));
+    const float* wd = c->kind ? c->wdiag : nullptr;
+    if (uses_ilu(c, precond)) penta_pack(B, n, c->stream, view, c->wtv, tv2_of(c), wd, c->ia, c->wa, w2s_of(c));
+    else penta_setup(B, n, c->stream, view, c->wtv, tv2_of(c), wd, c->ia);
     // ILU(0): the pivots of the incomplete factorisation replace 1/a
     if (precond == FIRLS_PRECOND_ILU0) ilu0_pivots(B, n, c->stream, c->st, view, c->wa, w2s_of(c), c->ia);
   } else if (precond == FIRLS_PRECOND_JACOBI) {
@@ -492,7 +493,7 @@ firls_status match_layout(firls_ctx* c, int precond) {
   const bool want = uses_ilu(c, precond);
   if (want == c->skewed) return FIRLS_OK;
   const int B = c->batch, n = c->n;
-  if (want) ilu_pack(B, n, c->stream, c->st, true, c->wtv, tv2_of(c), c->ia, c->wa, w2s_of(c));
+  if (want) ilu_pack(B, n, c->stream, c->st, c->wtv, tv2_of(c), c->ia, c->wa, w2s_of(c));
   const size_t bytes = sizeof(float2) * (size_t)B * (want ? ilu_slice_elems(n) : (size_t)n * n);
   for (float2* v : {c->r, c->z}) {  // u is free between macro steps
     ilu_skew(B, n, c->stream, want, v, c->u);
@@ -1452,7 +1453,6 @@ extern "C" firls_status firls_autotune(firls_ctx* c, const char* cache_path) {
     p.lambda_tv = 1e-3f;
     TRY(upload_params(c, &p));
     state_init(B, c->stream, c->st, c->part, 0, c->counts, n, c->lam_d, c->lamtv_d, 1e-10f, 1, PH_START);
-    if (has_tv(c)) penta_setup(B, n, c->stream, c->st, c->wtv, tv2_of(c), nullptr, c->ia);
     float best = 1e30f;
     if (c->kind) {
       // rb 0 only where it is a form of its own (the clusters above 256^2)
@@ -1475,7 +1475,7 @@ extern "C" firls_status firls_autotune(firls_ctx* c, const char* cache_path) {
     }
     if (has_tv(c)) {
       best = 1e30f;
-      ilu_pack(B, n, c->stream, c->st, true, c->wtv, tv2_of(c), c->ia, c->wa, w2s_of(c));
+      penta_pack(B, n, c->stream, c->st, c->wtv, tv2_of(c), nullptr, c->ia, c->wa, w2s_of(c));
       for (int shape : {42, 22}) {
         if (!ilu_shape_fits(n, shape, is_aniso(c))) continue;
         const float t = time_ms(c, [&]() {

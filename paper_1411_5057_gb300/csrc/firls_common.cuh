@@ -136,6 +136,12 @@ FI void pcg_beta_from(SliceState* v, double rz, double rr, const PcgSched& ps) {
   v->rho = rz;
 }
 
+// Diagonal of the TV penta-diagonal P: abar + lam_tv (W1_i + W1_{i+1} + W2_i +
+// W2_{i+n}), wc, wr, wv, wd in that order (W1 = W2 for isotropic TV: wv = wc).
+template <bool ANISO> FI float penta_diag(float abar, float lt, float wc, float wr, float wv, float wd) {
+  return ANISO ? abar + lt * (wc + wr + wv + wd) : abar + lt * (2.f * wc + wr + wd);
+}
+
 // Block-wide FP64 sum; result valid in thread 0.  `red` holds >= 32 doubles.
 FI double block_sum(double v, double* red) {
 #pragma unroll

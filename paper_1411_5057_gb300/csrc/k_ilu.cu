@@ -439,39 +439,90 @@ __global__ void __launch_bounds__(512) k_ilu0_pivots(int n, SliceState* st_all, 
   if (!ok) st_all[s].fault = 1;
 }
 
-// (lam W, 1/a) of the TV term in the skewed layout, and lam W2 for l1 TV, of
-// the slices st shows running (all: of every slice).
-__global__ void k_ilu_pack(int n, const SliceState* __restrict__ st, int all, const float* __restrict__ wtv,
-                           const float* __restrict__ wtv2, const float* __restrict__ ia, float4* __restrict__ wa,
-                           float2* __restrict__ w2s) {
-  const int s = blockIdx.y;
-  if (!all && !slice_running(st, s)) return;
-  const float lam = st[s].lam_tv;
-  const int H = n / 2, K = wv_steps(n), total = wv_bands(n) * K * 32;
-  const size_t nat = (size_t)s * n * H, out = (size_t)s * total;
-  const float2* W = reinterpret_cast<const float2*>(wtv) + nat;
-  const float2* A = reinterpret_cast<const float2*>(ia) + nat;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const int L = i & 31, k = (i >> 5) % K, row = (i >> 5) / K * 32 + L, c = k - L;
-    if (row >= n || c < 0 || c >= H) continue;
-    const float2 w = W[row * H + c], a = A[row * H + c];
-    wa[out + i] = make_float4(lam * w.x, a.x, lam * w.y, a.y);
-    if (wtv2) {
-      const float2 v = (reinterpret_cast<const float2*>(wtv2) + nat)[row * H + c];
-      w2s[out + i] = make_float2(lam * v.x, lam * v.y);
-    }
+// The kernels that write the skewed layout run in its order: a warp takes a step of
+// a band, lane L the pair of row L, and a CTA SK_STEPS consecutive steps, whose reads
+// of a natural array are SK_STEPS consecutive pairs of each row.  (Scattered 16-byte
+// stores from the natural order cost more than scattered loads: a complex array of 304
+// slices of 256^2 76 us, this way 47.)
+constexpr int SK_STEPS = 32;
+static dim3 skew_grid(int n, int batch) { return dim3((wv_steps(n) + SK_STEPS - 1) / SK_STEPS, wv_bands(n), batch); }
+
+// fn(row, c, index of the pair in the slice) for this thread's pairs
+template <typename Fn> FI void skew_pairs(int n, Fn&& fn) {
+  const int lane = threadIdx.x & 31, row = blockIdx.y * 32 + lane, K = wv_steps(n);
+  if (row >= n) return;
+#pragma unroll
+  for (int u = 0; u < SK_STEPS; u += 8) {
+    const int k = blockIdx.x * SK_STEPS + u + (threadIdx.x >> 5), c = k - lane;
+    if ((unsigned)c < (unsigned)(n / 2)) fn(row, c, (blockIdx.y * K + k) * 32 + lane);
   }
 }
 
-// Between the natural and the skewed layout of a complex array.
-__global__ void k_skew(int n, int to_skewed, const float4* __restrict__ src, float4* __restrict__ dst) {
+// The set-up of the sweeps for the slices st shows running, in one pass over the
+// weights: 1/a of P (Eq. ptv, k_penta's formula) in the natural order, (lam W, 1/a)
+// and for l1 TV lam W2 skewed.  Bound by memory, 16 bytes a pixel (l1 24).  304 slices
+// of 256^2 84 us, l1 110 (k_penta and a pack of its result took 127 and 161).
+template <bool ANISO>
+__global__ void __launch_bounds__(256) k_penta_pack(int n, const SliceState* __restrict__ st,
+                                                    const float* __restrict__ wtv, const float* __restrict__ wtv2,
+                                                    const float* __restrict__ wdiag, float* __restrict__ ia,
+                                                    float4* __restrict__ wa, float2* __restrict__ w2s) {
+  const int s = blockIdx.z;
+  if (!slice_running(st, s)) return;
+  const float abar = st[s].abar, lt = st[s].lam_tv, lw = st[s].lam;
+  const size_t nat = (size_t)s * n * n, out = (size_t)s * wv_bands(n) * wv_steps(n) * 32;
+  skew_pairs(n, [&](int row, int c, int at) {
+    const size_t i = nat + (size_t)row * n + 2 * c;
+    auto pair = [](const float* p) { return *reinterpret_cast<const float2*>(p); };
+    const float* V = ANISO ? wtv2 : wtv;  // the vertical weights
+    const float2 w = pair(wtv + i);
+    const float2 v = ANISO ? pair(V + i) : w;
+    const float2 below = row < n - 1 ? pair(V + i + n) : make_float2(0.f, 0.f);
+    const float right = 2 * c + 2 < n ? wtv[i + 2] : 0.f;
+    float a0 = penta_diag<ANISO>(abar, lt, w.x, w.y, v.x, below.x);
+    float a1 = penta_diag<ANISO>(abar, lt, w.y, right, v.y, below.y);
+    if (wdiag) {
+      const float2 g = pair(wdiag + i);
+      a0 = fmaf(lw, g.x, a0);
+      a1 = fmaf(lw, g.y, a1);
+    }
+    const float2 r = make_float2(1.0f / a0, 1.0f / a1);
+    *reinterpret_cast<float2*>(ia + i) = r;
+    wa[out + at] = make_float4(lt * w.x, r.x, lt * w.y, r.y);
+    if (ANISO) w2s[out + at] = make_float2(lt * v.x, lt * v.y);
+  });
+}
+
+// The packed weights from W, W2 and an 1/a that is there already, of every slice.
+__global__ void __launch_bounds__(256) k_ilu_pack(int n, const SliceState* __restrict__ st,
+                                                  const float* __restrict__ wtv, const float* __restrict__ wtv2,
+                                                  const float* __restrict__ ia, float4* __restrict__ wa,
+                                                  float2* __restrict__ w2s) {
+  const int s = blockIdx.z;
+  const float lam = st[s].lam_tv;
+  const size_t nat = (size_t)s * n * n, out = (size_t)s * wv_bands(n) * wv_steps(n) * 32;
+  skew_pairs(n, [&](int row, int c, int at) {
+    const size_t i = nat + (size_t)row * n + 2 * c;
+    const float2 w = *reinterpret_cast<const float2*>(wtv + i), a = *reinterpret_cast<const float2*>(ia + i);
+    wa[out + at] = make_float4(lam * w.x, a.x, lam * w.y, a.y);
+    if (wtv2) {
+      const float2 v = *reinterpret_cast<const float2*>(wtv2 + i);
+      w2s[out + at] = make_float2(lam * v.x, lam * v.y);
+    }
+  });
+}
+
+// A complex array from the natural to the skewed layout, and back.
+__global__ void __launch_bounds__(256) k_to_skewed(int n, const float4* __restrict__ src, float4* __restrict__ dst) {
+  const size_t nat = (size_t)blockIdx.z * n * (n / 2), out = (size_t)blockIdx.z * wv_bands(n) * wv_steps(n) * 32;
+  skew_pairs(n, [&](int row, int c, int at) { dst[out + at] = src[nat + (size_t)row * (n / 2) + c]; });
+}
+__global__ void k_from_skewed(int n, const float4* __restrict__ src, float4* __restrict__ dst) {
   const int H = n / 2, K = wv_steps(n), s = blockIdx.y;
   const size_t nat = (size_t)s * n * H, sk = (size_t)s * wv_bands(n) * K * 32;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * H; i += gridDim.x * blockDim.x) {
     const int row = i / H, c = i % H, L = row & 31;
-    const size_t j = sk + (size_t)((row >> 5) * K + c + L) * 32 + L;
-    if (to_skewed) dst[j] = src[nat + i];
-    else dst[nat + i] = src[j];
+    dst[nat + i] = src[sk + (size_t)((row >> 5) * K + c + L) * 32 + L];
   }
 }
 
@@ -547,10 +598,15 @@ void ilu_step(int batch, int n, cudaStream_t s, SliceState* st, double* part, in
                  reinterpret_cast<const float4*>(q), f4(y), f4(z), wa, w2s, fuse_scalars, ps, wait_test, alpha_np);
 }
 
-void ilu_pack(int batch, int n, cudaStream_t s, const SliceState* st, bool all, const float* wtv,
-              const float* wtv2, const float* ia, float4* wa, float2* w2s) {
-  const int total = wv_bands(n) * wv_steps(n) * 32;
-  k_ilu_pack<<<dim3(std::min((total + 255) / 256, 64), batch), 256, 0, s>>>(n, st, all ? 1 : 0, wtv, wtv2, ia, wa, w2s);
+void penta_pack(int batch, int n, cudaStream_t s, const SliceState* st, const float* wtv, const float* wtv2,
+                const float* wdiag, float* ia, float4* wa, float2* w2s) {
+  if (wtv2) k_penta_pack<true><<<skew_grid(n, batch), 256, 0, s>>>(n, st, wtv, wtv2, wdiag, ia, wa, w2s);
+  else k_penta_pack<false><<<skew_grid(n, batch), 256, 0, s>>>(n, st, wtv, wtv2, wdiag, ia, wa, w2s);
+}
+
+void ilu_pack(int batch, int n, cudaStream_t s, const SliceState* st, const float* wtv, const float* wtv2,
+              const float* ia, float4* wa, float2* w2s) {
+  k_ilu_pack<<<skew_grid(n, batch), 256, 0, s>>>(n, st, wtv, wtv2, ia, wa, w2s);
 }
 
 void ilu0_pivots(int batch, int n, cudaStream_t s, SliceState* st, const SliceState* view, float4* wa,
@@ -561,8 +617,10 @@ void ilu0_pivots(int batch, int n, cudaStream_t s, SliceState* st, const SliceSt
 }
 
 void ilu_skew(int batch, int n, cudaStream_t s, bool to_skewed, const float2* src, float2* dst) {
-  k_skew<<<dim3(std::min((n * n / 2 + 255) / 256, 64), batch), 256, 0, s>>>(
-      n, to_skewed ? 1 : 0, reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst));
+  const float4* from = reinterpret_cast<const float4*>(src);
+  float4* to = reinterpret_cast<float4*>(dst);
+  if (to_skewed) k_to_skewed<<<skew_grid(n, batch), 256, 0, s>>>(n, from, to);
+  else k_from_skewed<<<dim3(std::min((n * n / 2 + 255) / 256, 64), batch), 256, 0, s>>>(n, from, to);
 }
 
 }  // namespace firls

@@ -744,8 +744,7 @@ void wavelet_diag(int batch, int n, int levels, int kind, cudaStream_t s, const 
 // P = abar I + lam_tv (D1^T W1 D1 + D2^T W2 D2) [+ lam diag(Phi^T W Phi)]
 // (Eq. ptv; W1 = W2 = W for isotropic TV, wtv2 null): ia = 1 / a_i, the
 // inverse diagonal, a_i = abar + lam_tv (W1_i + W1_{i+1} + W2_i + W2_{i+n}).
-// The off-diagonals (-lam_tv W1_{i+1}, -lam_tv W2_{i+n}) are formed from the
-// weights inside the ILU sweeps.
+// For the Jacobi scale; the sweeps' set-up is k_penta_pack (k_ilu.cu).
 __global__ void k_penta(int n, const SliceState* __restrict__ st, const float* __restrict__ wtv,
                         const float* __restrict__ wtv2, const float* __restrict__ wdiag, float* __restrict__ ia) {
   const int s = blockIdx.y;
@@ -759,10 +758,10 @@ __global__ void k_penta(int n, const SliceState* __restrict__ st, const float* _
     float a;
     if (wtv2) {
       const float wd = r < n - 1 ? wtv2[base + i + n] : 0.f;
-      a = abar + lt * (wc + wr + wtv2[base + i] + wd);
+      a = penta_diag<true>(abar, lt, wc, wr, wtv2[base + i], wd);
     } else {
       const float wd = r < n - 1 ? wtv[base + i + n] : 0.f;
-      a = abar + lt * (2.f * wc + wr + wd);
+      a = penta_diag<false>(abar, lt, wc, wr, wc, wd);
     }
     if (wdiag) a = fmaf(lw, wdiag[base + i], a);
     ia[base + i] = 1.0f / a;

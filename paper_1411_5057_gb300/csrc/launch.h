@@ -131,10 +131,13 @@ void penta_setup(int batch, int n, cudaStream_t s, const SliceState* st, const f
 // ---- the TV preconditioner's sweeps (k_ilu.cu), on arrays in a skewed layout ----
 size_t ilu_slice_elems(int n);  // float2 per slice of a skewed array
 bool ilu_prepare();
-// wa = (lam W, 1/a) skewed, and for l1 TV w2s = lam W2 skewed, of the slices st
-// shows running (or all); before a sweep with new weights
-void ilu_pack(int batch, int n, cudaStream_t s, const SliceState* st, bool all, const float* wtv,
-              const float* wtv2, const float* ia, float4* wa, float2* w2s);
+// 1/a of P in ia, wa = (lam W, 1/a) skewed, and for l1 TV w2s = lam W2 skewed, of the
+// slices st shows running; before a sweep with new weights
+void penta_pack(int batch, int n, cudaStream_t s, const SliceState* st, const float* wtv, const float* wtv2,
+                const float* wdiag, float* ia, float4* wa, float2* w2s);
+// wa and w2s of every slice from an ia that is there already
+void ilu_pack(int batch, int n, cudaStream_t s, const SliceState* st, const float* wtv, const float* wtv2,
+              const float* ia, float4* wa, float2* w2s);
 // 1/a -> 1/d, the ILU(0) pivots (updated pivots, zero fill), in wa and ia
 void ilu0_pivots(int batch, int n, cudaStream_t s, SliceState* st, const SliceState* view, float4* wa,
                  const float2* w2s, float* ia);
@@ -200,7 +203,7 @@ __host__ __device__ inline bool guard_keeps(double f1, double f0) { return f1 - 
 void guard_pick(int batch, int n, cudaStream_t s, const double* f1, const double* f0, const void* x1,
                 const float2* atb, void* x0);
 
-// PCG scalar updates (one thread per slice).  channels C > 1: the inner
+// PCG scalar updates (a warp per slice).  channels C > 1: the inner
 // products are summed over the C consecutive slices of a multi-contrast
 // image, whose slices then carry the same scalars (here, in outer_end and in
 // state_init's ||A^H b||^2).
