@@ -74,9 +74,12 @@ int firls_size_supported(int n);
 /* Create a context for `batch` independent slices of n_rows x n_cols
  * (square: n_rows == n_cols).  `cuda_stream` is a cudaStream_t (NULL = the
  * legacy default stream).  The context allocates its device workspace
- * (about 14 complex64 + 6 float vectors per slice) on the current device.
+ * (about 10 complex64 + 4 float vectors per slice) on the current device, four
+ * of the complex vectors in firls_set_operator: with TV they and the packed
+ * weights take 18 more bytes a pixel at 256^2 (l1 TV 27).
  * Returns FIRLS_E_SHAPE for unsupported sizes, FIRLS_E_NOMEM if the
- * workspace does not fit. */
+ * workspace does not fit (firls_set_operator: if what the operator adds does
+ * not). */
 firls_status firls_create(firls_ctx** out, int n_rows, int n_cols, int batch,
                           unsigned flags, void* cuda_stream);
 

@@ -50,7 +50,7 @@ struct firls_ctx {
   float4* wa = nullptr;
   float2* w2s = nullptr;
   bool skewed = false;
-  bool skew_room = false;  // r, z, q and u have the size of that layout (1.24 x at 256^2, 9.75 x at 16^2)
+  size_t room[4] = {};  // float2 per slice that q, u, r and z hold (the operator decides: work_room)
   float* wg = nullptr;
   int *gidx = nullptr, *goff = nullptr, *inv_off = nullptr, *inv_ids = nullptr;
   int *gcounts = nullptr, *gcursor = nullptr, *gerr = nullptr;
@@ -503,24 +503,31 @@ firls_status match_layout(firls_ctx* c, int precond) {
   return cuda_check(c, cudaGetLastError(), "layout change");
 }
 
-// r, z, q and u at the size of the sweeps' layout, for the first operator with TV.  One
-// after the other, so that the old and the new form of only one exist at a time; r
-// and z keep what live slots have there.  The captured graphs, which hold the old
-// addresses, are dropped by firls_set_operator before anything can run.
-firls_status sweep_room(firls_ctx* c) {
-  if (c->skew_room) return FIRLS_OK;
-  const size_t natural = (size_t)c->batch * c->n * c->n;
-  for (float2** v : {&c->q, &c->u, &c->r, &c->z}) {
-    float2* room = nullptr;
-    TRY(dalloc(c, &room, ilu_slice_elems(c->n) * c->batch));
-    if (v == &c->r || v == &c->z) {
-      CU(cudaMemcpyAsync(room, *v, sizeof(float2) * natural, cudaMemcpyDeviceToDevice, c->stream));
-      CU(cudaStreamSynchronize(c->stream));
+// q, u, r and z at the size that the operator needs: n^2 a slice, or with TV that of the
+// sweeps' layout (1.24 n^2 at 256^2, 9.75 n^2 at 16^2).  A context that changes to TV keeps
+// what live slots have in r and z.  The captured graphs, which hold the old addresses,
+// are dropped by firls_set_operator before anything can run.
+firls_status work_room(firls_ctx* c, bool sweeps) {
+  const size_t natural = (size_t)c->n * c->n, need = sweeps ? ilu_slice_elems(c->n) : natural;
+  float2** const v[4] = {&c->q, &c->u, &c->r, &c->z};
+  for (int i = 0; i < 4; ++i) {
+    if (c->room[i] >= need) continue;
+    float2* old = *v[i];
+    if (i < 2) {  // made anew in every macro step
+      dfree(c, old);
+      *v[i] = old = nullptr;
+      c->room[i] = 0;
     }
-    dfree(c, *v);
-    *v = room;
+    float2* p = nullptr;
+    TRY(dalloc(c, &p, need * c->batch));
+    if (old) {
+      CU(cudaMemcpyAsync(p, old, sizeof(float2) * natural * c->batch, cudaMemcpyDeviceToDevice, c->stream));
+      CU(cudaStreamSynchronize(c->stream));
+      dfree(c, old);
+    }
+    *v[i] = p;
+    c->room[i] = need;
   }
-  c->skew_room = true;
   return FIRLS_OK;
 }
 
@@ -752,7 +759,7 @@ extern "C" firls_status firls_create(firls_ctx** out, int n_rows, int n_cols, in
   A(&c->mask, BN);
   A(&c->counts, (size_t)batch);
   A(&c->tw, (size_t)n);
-  for (float2** p : {&c->atb, &c->x, &c->r, &c->z, &c->d, &c->q, &c->t, &c->u, &c->cw, &c->dx}) A(p, BN);
+  for (float2** p : {&c->atb, &c->x, &c->d, &c->t, &c->cw, &c->dx}) A(p, BN);
   A(&c->tmpA, BH);
   A(&c->tmpB, BH);
   for (float** p : {&c->ww, &c->wtv, &c->ia, &c->wdiag}) A(p, BN);
@@ -760,6 +767,10 @@ extern "C" firls_status firls_create(firls_ctx** out, int n_rows, int n_cols, in
   A(&c->stw, (size_t)batch);
   A(&c->part, (size_t)batch * NSLOT * MAXPART);
   A(&c->fobj, 2 * (size_t)batch);
+  size_t free_bytes = 0, total_bytes = 0;
+  // a batch for whose q, u, r and z firls_set_operator would find no room is refused here
+  if (s == FIRLS_OK && cudaMemGetInfo(&free_bytes, &total_bytes) == cudaSuccess && free_bytes < 4 * BN * sizeof(float2))
+    s = FIRLS_E_NOMEM;
   A(&c->lam_d, 2 * (size_t)batch);  // both lambdas in one block: one copy uploads them
   if (c->lam_d) c->lamtv_d = c->lam_d + batch;
   if (s != FIRLS_OK) {
@@ -876,10 +887,9 @@ extern "C" firls_status firls_set_operator(firls_ctx* c, const uint8_t* mask, un
     CU(cudaMemcpy(c->sqtab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(c->sqlen, len.data(), sizeof(int) * len.size(), cudaMemcpyHostToDevice));
   }
-  if (psi_kind & (FIRLS_PSI_TV | FIRLS_PSI_TV_ANISO)) {
-    TRY(sweep_room(c));
-    if (!c->wa) TRY(dalloc(c, &c->wa, ilu_slice_elems(n) / 2 * B));
-  }
+  const bool tv = psi_kind & (FIRLS_PSI_TV | FIRLS_PSI_TV_ANISO);
+  TRY(work_room(c, tv));
+  if (tv && !c->wa) TRY(dalloc(c, &c->wa, ilu_slice_elems(n) / 2 * B));
   if (psi_kind & FIRLS_PSI_TV_ANISO) {
     if (!c->wtv2) {
       TRY(dalloc(c, &c->wtv2, N * B));
@@ -1443,7 +1453,7 @@ extern "C" firls_status firls_autotune(firls_ctx* c, const char* cache_path) {
   int rb = 0, cm = 0, il = 0;
   if (!tune_cache_lookup(cache_path, key, &rb, &cm, &il)) {
     // deterministic, finite contents for timing
-    const size_t BN = (size_t)B * n * n, BS = c->skew_room ? ilu_slice_elems(n) * B : BN;
+    const size_t BN = (size_t)B * n * n, BS = c->room[0] * B;
     for (float2* v : {c->x, c->d, c->atb, c->cw}) cudaMemsetAsync(v, 0, BN * 8, c->stream);
     for (float2* v : {c->r, c->q, c->z, c->u}) cudaMemsetAsync(v, 0, BS * 8, c->stream);
     for (float* v : {c->ww, c->wtv, c->wdiag}) cudaMemsetAsync(v, 0, BN * 4, c->stream);
