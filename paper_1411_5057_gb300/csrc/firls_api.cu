@@ -392,7 +392,7 @@ void enqueue_precond(firls_ctx* c, int mode, const firls_params& sc, bool chaine
     wavelet_apply(w, c->r, c->cw, c->ww, WAV_MUL_PINV, c->z, c->r, real);
   }
   TMark m(c, FIRLS_K_SCALARS, 1);
-  pcg_scalars(B, c->stream, c->st, c->part, np, np_rr, sm, ps, c->channels, chained);
+  pcg_scalars(B, c->stream, c->st, c->part, np, np_rr, sm, ps, c->channels, chained, w.upd_q ? c->r : nullptr, n);
 }
 
 // The end of every outer step whose PCG has stopped: x += dx, the relative

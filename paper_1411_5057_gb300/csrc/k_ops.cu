@@ -1310,19 +1310,38 @@ void pcg_alpha(int batch, cudaStream_t s, SliceState* st, const double* part, in
   launch_chained(chained, k_alpha, dim3(sc_ctas(batch)), dim3(32 * SC_WARPS), 0, s, batch, st, part, np, channels);
 }
 
+// The sum of squares of n4 float4 in FP64, in every lane of the warp that calls it.
+FI double wide_norm2(const float4* v, int n4) {
+  double a = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x & 31; i < n4; i += 32) {
+    const float4 x = v[i];
+    a += (double)x.x * x.x + (double)x.y * x.y + (double)x.z * x.z + (double)x.w * x.w;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
 // After z = P^{-1} r: rho (first residual, slices at the start of an outer
 // step) or beta and the PCG stop (slices in PCG); mode INIT / STEP forces one
 // of them for every running slice.
+// r (may be null): the residuals [B][N4], for ||r||^2 where the partial sums are not
+// finite.  Those of the update inside the wavelet transform are carried in three floats,
+// which end at 3.4e38 a CTA; a test there cost up to 0.7 % of a small solve.
 __global__ void k_pcg_scalars(int B, SliceState* st, const double* part, int np_rz, int np_rr, int mode,
-                              PcgSched ps, int C) {
+                              PcgSched ps, int C, const float4* __restrict__ r, int N4) {
   chained_start();
   const int s = sc_slice();
   if (s >= B || !slice_running(st, s) || st[s].fault) return;
   const int ph = st[s].phase;
   const bool init = mode == SCALARS_INIT || (mode == SCALARS_PER_SLICE && ph == PH_START);
   const bool step = mode == SCALARS_STEP || (mode == SCALARS_PER_SLICE && ph == PH_PCG);
-  const double rz = image_parts(part, s, SLOT_RZ, np_rz, C), rr = image_parts(part, s, SLOT_RR, np_rr, C);
-  if (threadIdx.x & 31) return;
+  const double rz = image_parts(part, s, SLOT_RZ, np_rz, C);
+  double rr = image_parts(part, s, SLOT_RR, np_rr, C);
+  const int lane = threadIdx.x & 31;
+  if (r != nullptr && __shfl_sync(0xffffffffu, !isfinite(rr), 0)) rr = wide_norm2(r + (size_t)(s - s % C) * N4, C * N4);
+  if (lane) return;
   if (init)
     pcg_rho_init_from(st + s, rz, rr);
   else if (step)
@@ -1330,9 +1349,9 @@ __global__ void k_pcg_scalars(int B, SliceState* st, const double* part, int np_
 }
 
 void pcg_scalars(int batch, cudaStream_t s, SliceState* st, const double* part, int np_rz, int np_rr, int mode,
-                 const PcgSched& ps, int channels, bool chained) {
+                 const PcgSched& ps, int channels, bool chained, const float2* r, int n) {
   launch_chained(chained, k_pcg_scalars, dim3(sc_ctas(batch)), dim3(32 * SC_WARPS), 0, s, batch, st, part, np_rz, np_rr, mode, ps,
-                 channels);
+                 channels, reinterpret_cast<const float4*>(r), n * n / 2);
 }
 
 // Outer-loop stop.  kind 0: relative change <= tol.  kind 1: estimated

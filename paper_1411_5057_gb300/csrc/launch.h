@@ -211,7 +211,8 @@ void pcg_alpha(int batch, cudaStream_t s, SliceState* st, const double* part, in
                bool chained = false);
 enum ScalarsMode { SCALARS_INIT = 0, SCALARS_STEP = 1, SCALARS_PER_SLICE = -1 };
 void pcg_scalars(int batch, cudaStream_t s, SliceState* st, const double* part, int nparts_rz, int nparts_rr,
-                 int mode, const PcgSched& ps, int channels = 1, bool chained = false);
+                 int mode, const PcgSched& ps, int channels = 1, bool chained = false, const float2* r = nullptr,
+                 int n = 0);
 // view = st with every slice not at the start of its outer step marked done
 // (and the slices whose outer step is due move to PH_START)
 void boundary_view(int batch, cudaStream_t s, SliceState* st, SliceState* view);

@@ -77,7 +77,6 @@ FI void inv_haar(float2 a, float2 d, float2& x0, float2& x1) {
 constexpr int WCL_NMAX = 256;
 constexpr int WCL_LMAX = 5;
 constexpr int WCL_RMAX = 32;  // rows per CTA: two CTAs per SM fit with the weights mirrored
-constexpr double RR_HI = 1e38;  // ||r||^2 of a CTA that three floats may carry
 constexpr int WCL_WIDE_R = 32;  // rows per CTA of the sizes above WCL_NMAX (clusters of 10, 12, 16)
 
 FI unsigned wcl_rank() {
@@ -379,7 +378,7 @@ FI void wcl_push(const float2* D, const float2* Hb, const uint64_t* bar, int n, 
 //
 // UPD (z = P^{-1} r of a PCG step): the load is the residual update as well:
 // r -= alpha q, or r = A^H b - q for a slice at the start of its outer step, and
-// the partial ||r||^2.  A launch and a pass over r less than an update of its own
+// the partial ||r||^2 (NaN beyond the FP32 range: k_pcg_scalars then sums r itself).  A launch and a pass over r less than an update of its own
 // (solves of 60 slices of 256^2 4231 -> 4125 us, of one of 64^2 1588 -> 1502).  Up
 // to WCL_NMAX: above, the clusters leave SMs idle that an update of its own uses
 // (8 slices of 512^2: 7697 us apart, 8108 in one).
@@ -479,20 +478,7 @@ k_wav_cluster(const float2* x, float2* u, const float* __restrict__ w, int L_arg
     if (tid < TH / 32) rr = rr_part[tid];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) rr.add(rr.from_lane(o));
-    double total = rr.value();
-    // floats have less range than the FP64 sums of an update of its own: a sum near
-    // or beyond their end (or NaN) is formed again from the residual just stored
-    if (__shfl_sync(0xffffffffu, !(total < RR_HI), 0)) {
-      const float4* r4 = reinterpret_cast<const float4*>(rw) + ((size_t)s * nn + (size_t)rank * R * n) / 2;
-      total = 0.0;
-      for (int i = tid; i < R * n / 2; i += 32) {
-        const float4 v = r4[i];
-        total += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-    }
-    if (tid == 0) part[((size_t)s * NSLOT + SLOT_RR) * MAXPART + rank] = total;
+    if (tid == 0) part[((size_t)s * NSLOT + SLOT_RR) * MAXPART + rank] = rr.value();
   }
   if (kind == 2)  // every CTA's mbarriers armed before any remote write
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
