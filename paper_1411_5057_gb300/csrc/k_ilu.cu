@@ -575,7 +575,9 @@ int ilu_default_shape(int n, int batch) {
   return 10 * waves(8) < 19 * waves(16) ? 42 : 22;
 }
 
-// The shapes that set_tuning takes for a size.
+// The shapes that set_tuning takes for a size: those of tuning files and callers from
+// when S counted the stages of a shared-memory ring, by the bytes it took.  The sweeps
+// need no such room; the set stays what it was.
 bool ilu_shape_fits(int n, int shape, bool aniso) {
   const int G = shape / 10, S = shape % 10;
   if ((G != 2 && G != 4) || S < 2 || S > 8 || n % G) return false;
