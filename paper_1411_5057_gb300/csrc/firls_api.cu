@@ -662,8 +662,8 @@ bool has_tolerances(const firls_params* p) {
 // step, so the batch moves in lockstep and an outer step of J PCG steps needs
 // its boundary stage only at the start of its J + 1 macro steps (a slice that
 // stops early, at rho = 0, waits there for the others).  One in every macro
-// step costs 9 launches that find nothing to do: 20 us a macro step for one
-// 256^2 slice, 110 us for 304.
+// step costs 9 launches that find nothing to do: over 20 steps 12 us a macro step
+// for one 256^2 slice (4125 -> 3889), 51 us for 304 (17740 -> 16725).
 bool in_lockstep(const firls_params* p) { return !(p->pcg_tol > 0.f) && period_of(*p) == 1; }
 
 // params->outer_iters outer steps of a batch in lockstep: one graph replay of

@@ -41,9 +41,13 @@
 // set to 0, so no load is conditional.
 //
 // Measured, row scans before and this form now, 256^2: 1 slice 158 and 92 us, 76
-// slices 160 and 105, 152 slices 174 and 132, 304 slices 289 and 250 (the row
-// scans also updated dx there, 24 of their 88 bytes a pixel, now in the row
-// FFT); 16 slices of 512^2 540 and 286, 64 of 320^2 230 and 179.
+// slices 160 and 105, 152 slices 174 and 132, 304 slices 289 and 250; 16 slices of
+// 512^2 540 and 286, 64 of 320^2 230 and 179.  The row scans also updated dx, 24 of
+// their 88 bytes a pixel, which the row FFT does now, and the row IFFT stores q skewed.
+// So many slices gain nothing by the form itself: a step's row FFT, row IFFT and sweeps
+// of 304 slices took 96 + 133 + 287 us and take 141 + 153 + 253, of 40 of 512^2 59 + 85 +
+// 547 and 83 + 104 + 314.  One form serves every batch all the same: a served queue
+// ends with few slices, where the sweeps are the step.
 #include <algorithm>
 
 #include "launch.h"
