@@ -151,9 +151,10 @@ typedef struct {
                           every this-many-th macro step (0 or 1: every one);
                           a slice waits at most boundary_period - 1 macro
                           steps per outer step, and the mostly idle set-up
-                          launches run that much less often.  firls_solve and
-                          firls_solve_multi without a PCG tolerance move in
-                          lockstep and run them once per outer step           */
+                          launches run that much less often.  firls_solve
+                          without a PCG tolerance moves in lockstep and runs
+                          them once per outer step, and so does
+                          firls_solve_multi without pcg_iters_late            */
 } firls_params;
 
 /* Preconditioners of the PCG steps, for the comparison of Sec. 5.2 (Fig. 2
